@@ -406,7 +406,7 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
     size_t o_flops = take(8 * U1);
     size_t o_bin = take(U1);
     size_t o_iprod = take(4 * U1);
-    size_t o_ctr = take(8 * (2 * NBIN + 8));
+    size_t o_ctr = take(8 * (CTR_REP * CTR_STRIDE + NBIN + 8));
     size_t o_binoff = take(8 * NBIN);
     size_t o_list = take(sizeof(int2) * U1);
     size_t o_nnz = take(8 * U1);
@@ -471,14 +471,19 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         }
         SG_CUDA(ctx, cudaMemcpyAsync(skbase, hb.data(), 8 * (np + 1), cudaMemcpyHostToDevice, st));
     }
-    SG_CUDA(ctx, cudaMemsetAsync(E->ctr, 0, 8 * (2 * NBIN + 8), st));
-    launch_analyze(st, E->it, E->cfg, E->flops, E->bin, E->item_prod, E->ctr, E->ctr + 2 * NBIN, sketch, skbase,
+    // counter copies of the analysis, then the scatter cursors and the slab tier's counters
+    unsigned long long* const cur = E->ctr + CTR_REP * CTR_STRIDE;
+    unsigned long long* const slab_ctr = cur + NBIN;
+    SG_CUDA(ctx, cudaMemsetAsync(E->ctr, 0, 8 * (CTR_REP * CTR_STRIDE + NBIN + 8), st));
+    launch_analyze(st, E->it, E->cfg, E->flops, E->bin, E->item_prod, E->ctr, E->ctr + NBIN, sketch, skbase,
                    E->feat, E->maxlen);
-    unsigned long long hc[NBIN + 1];
-    SG_TRY(read_back(ctx, hc, E->ctr, sizeof(unsigned long long) * NBIN));
-    SG_TRY(read_back(ctx, hc + NBIN, E->ctr + 2 * NBIN, sizeof(unsigned long long)));
+    unsigned long long hc[CTR_REP * CTR_STRIDE];
+    SG_TRY(read_back(ctx, hc, E->ctr, sizeof(hc)));
     SG_TRY(sync_ctx(ctx));
+    E->err_dev = (const int*)(slab_ctr + 3);
     int64_t acc = 0;
+    for (int b = 0; b <= NBIN; ++b)
+        for (int r = 1; r < CTR_REP; ++r) hc[b] += hc[r * CTR_STRIDE + b];
     for (int b = 0; b < NBIN; ++b) {
         E->bin_cnt[b] = (int64_t)hc[b];
         E->bin_off[b] = acc;
@@ -486,7 +491,7 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
     }
     E->flops_total = (int64_t)hc[NBIN];
     SG_CUDA(ctx, cudaMemcpyAsync(E->bin_off_dev, E->bin_off, sizeof(int64_t) * NBIN, cudaMemcpyHostToDevice, st));
-    launch_bin_scatter(st, E->it, E->bin, E->item_prod, E->bin_off_dev, E->ctr + NBIN, E->list);
+    launch_bin_scatter(st, E->it, E->bin, E->item_prod, E->bin_off_dev, cur, E->list);
     const int64_t nd = E->bin_cnt[BIN_DENSE];
     E->dw = DenseWork();
     if (nd > 0 && E->it.max_m <= BLOCK_TIER_MAX_ROWS) {
@@ -514,20 +519,20 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         dw.dlist = E->list + E->bin_off[BIN_DENSE];
         dw.ndense = nd;
         dw.items = (int2*)(db + o_items);
-        dw.nitems = E->ctr + 2 * NBIN + 1;
+        dw.nitems = slab_ctr + 1;
         dw.nparts = (int8_t*)(db + o_np);
         dw.sbase = (int32_t*)(db + o_sb);
         dw.bbase = (int64_t*)(db + o_bb);
-        unsigned long long* bnd_total = E->ctr + 2 * NBIN + 6;
-        dw.store_ctr = E->ctr + 2 * NBIN + 2;
-        dw.err = (int*)(E->ctr + 2 * NBIN + 3);
-        unsigned long long* store_bound = E->ctr + 2 * NBIN + 4;
+        unsigned long long* bnd_total = slab_ctr + 6;
+        dw.store_ctr = slab_ctr + 2;
+        dw.err = (int*)(slab_ctr + 3);
+        unsigned long long* store_bound = slab_ctr + 4;
         dw.RB = E->cfg.dense_rows;
         launch_dense_items(st, E->it, dw.dlist, nd, E->flops, E->cfg.part_flops, dw.RB, (int2*)dw.items,
-                           E->ctr + 2 * NBIN + 1, (int8_t*)dw.nparts, (int32_t*)dw.sbase, store_bound,
+                           slab_ctr + 1, (int8_t*)dw.nparts, (int32_t*)dw.sbase, store_bound,
                            (int64_t*)dw.bbase, bnd_total);
         unsigned long long hs[3] = {0, 0, 0};
-        SG_TRY(read_back(ctx, &hs[0], E->ctr + 2 * NBIN + 1, 8));
+        SG_TRY(read_back(ctx, &hs[0], slab_ctr + 1, 8));
         SG_TRY(read_back(ctx, &hs[1], store_bound, 8));
         SG_TRY(read_back(ctx, &hs[2], bnd_total, 8));
         SG_TRY(sync_ctx(ctx));
@@ -554,7 +559,7 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
     }
     if (sr == SPGEMM_OR_AND_BOOL) {
         // boolean operands without a stored false value: the bitmap tiers take every output as true
-        int* vals_zero = (int*)(E->ctr + 2 * NBIN + 5);
+        int* vals_zero = (int*)(slab_ctr + 5);
         if (ctx->bool_hint >= 0) SG_CUDA(ctx, cudaMemsetAsync(vals_zero, ctx->bool_hint ? 1 : 0, 4, st));
         else launch_false_values(st, E->it, vals_zero);
         E->dw.vals_zero = vals_zero;
@@ -613,7 +618,7 @@ spgemm_status_t engine_symbolic(Engine* E) {
     }
     SG_TRY(read_back(ctx, nc, E->nctr, sizeof(nc)));
     SG_TRY(read_back(ctx, &nnz, E->Coff + U, sizeof(int64_t)));
-    SG_TRY(read_back(ctx, &err, E->ctr + 2 * NBIN + 3, sizeof(int)));
+    SG_TRY(read_back(ctx, &err, E->err_dev, sizeof(int)));
     // every product's first output, at the same synchronisation (batched calls)
     std::shared_ptr<DevBuf> pob;
     const int64_t np = E->it.nprod;

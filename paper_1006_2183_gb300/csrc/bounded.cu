@@ -93,7 +93,7 @@ spgemm_status_t engine_numeric_bounded(Engine* E, std::shared_ptr<DevBuf>* rbuf,
         }
         launch_exclusive_scan(st, cap, U, cap_off, stmp);
         SG_TRY(read_back(ctx, &total, cap_off + U, 8));
-        SG_TRY(read_back(ctx, &err, E->ctr + 2 * NBIN + 3, sizeof(int)));
+        SG_TRY(read_back(ctx, &err, E->err_dev, sizeof(int)));
         SG_TRY(sync_ctx(ctx));
     }
     if (err) return set_err(ctx, SPGEMM_ERR_INDEX_OVERFLOW, "slab tier capacity exceeded (code %d)", err);

@@ -88,8 +88,9 @@ struct Engine {
     int64_t* flops = nullptr;
     uint8_t* bin = nullptr;
     int32_t* item_prod = nullptr;
-    unsigned long long* ctr = nullptr;   // bin_count[NBIN], bin_cursor[NBIN], flops_total, slabs, store use, err,
-                                         // store bound, false-value flag
+    unsigned long long* ctr = nullptr;   // CTR_REP copies of bin counts and total flops, bin_cursor[NBIN], then
+                                         // the slab tier's counters, its error flag and the false-value flag
+    const int* err_dev = nullptr;        // the slab tier's error flag (device)
     int64_t* bin_off_dev = nullptr;
     int2* list = nullptr;
     sg::DenseWork dw;                    // slab-tier state

@@ -102,9 +102,30 @@ __device__ __forceinline__ int find_prod(const int64_t* __restrict__ base, int64
 __device__ __forceinline__ int64_t out_col(const DMat& B, int64_t p) { return B.jc ? __ldg(B.jc + p) : p; }
 
 // ------------------------------------------------------------------ analysis
-// Groups of LPI lanes per item (8, or 1 where B columns are short, as in the
-// block products): flops = sum_k nnz(A(:,k)) (Section 1's flops), the tier bin,
+// Groups of LPI lanes per item (8; 1 where B columns are short, as in the block
+// products; 32 where they hold 32 entries and more on average): flops = sum_k nnz(A(:,k)) (Section 1's flops), the tier bin,
 // the product id, and optionally the predictor inputs.
+// A lookup is a chain of dependent loads (B's row, A's column pointers), so a hub column
+// of B on its 8 lanes was the whole kernel's time (23,356 entries at R-MAT scale 20: a
+// chain of 2,900 lookups).  Columns longer than ANALYZE_LONG entries are walked by the
+// whole CTA, four lookups in flight per thread: R-MAT 20 flat 1.73 -> 0.29 ms, R-MAT of
+// 300,007 vertices 0.67 -> 0.16 ms.  Shorter ones stay on their lanes: up to 32 rounds of
+// 8 lanes cost less than a pass of the CTA of their own.  Items strided over the CTAs (the
+// hubs of an R-MAT graph sit side by side) took 0.42 ms at R-MAT 20: their pointers and
+// results no longer share sectors.
+constexpr int ANALYZE_LONG = 256;
+
+// lookup of A(:,k) for entry t of B(:,j): its length, stored in the A-column cache if there is one
+__device__ __forceinline__ long long analyze_entry(const Items& it, const DMat& A, int32_t k, int64_t cache_at) {
+    int64_t cs, ce;
+    col_range(A, k, cs, ce);
+    if (it.acs) {
+        it.acs[cache_at] = cs;
+        it.acl[cache_at] = (int32_t)(ce - cs);
+    }
+    return ce - cs;
+}
+
 template <int LPI>
 __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t* __restrict__ flops,
                                                  uint8_t* __restrict__ bin, int32_t* __restrict__ item_prod,
@@ -112,17 +133,23 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
                                                  const uint64_t* __restrict__ sketch,
                                                  const int64_t* __restrict__ sketch_base, float* __restrict__ feat,
                                                  int64_t* __restrict__ maxlen) {
+    constexpr int GRP = 256 / LPI;   // items of this CTA
     __shared__ unsigned long long s_cnt[NBIN];
     __shared__ unsigned long long s_fl;
+    __shared__ int s_nlong;
+    __shared__ int s_long[GRP];                                              // groups with a long column
+    __shared__ unsigned long long s_lf[GRP], s_lmx[GRP], s_lsk[GRP];         // their totals
     if (threadIdx.x < NBIN) s_cnt[threadIdx.x] = 0;
     if (threadIdx.x == 0) s_fl = 0;
+    if (threadIdx.x == 0) s_nlong = 0;
     __syncthreads();
-    const int sub = threadIdx.x & (LPI - 1);
-    const int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / LPI;
+    const int sub = threadIdx.x & (LPI - 1), grp = threadIdx.x / LPI;
+    const int64_t u = (int64_t)blockIdx.x * GRP + grp;
     long long f = 0, mx = 0;
     unsigned long long sk = 0;
     int64_t bs = 0, be = 0, am = 0;
     int prod = 0;
+    bool is_long = false;
     if (u < it.nitems) {
         prod = it.nprod == 1 ? 0 : __ldg(item_prod + u);   // filled per product beforehand
         const Prod* pr = it.prods + prod;
@@ -132,7 +159,13 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
         am = pr->A.m;
         const uint64_t* skp = sketch ? sketch + sketch_base[prod] : nullptr;
         const int64_t b0 = it.acs ? pr->bnz_base - __ldg(pr->B.cp) : 0;
-        if constexpr (LPI == 1) {
+        is_long = be - bs > ANALYZE_LONG;
+        if (is_long) {
+            if (sub == 0) {
+                s_lf[grp] = s_lmx[grp] = s_lsk[grp] = 0;
+                s_long[atomicAdd(&s_nlong, 1)] = grp;
+            }
+        } else if constexpr (LPI == 1) {
             // two entries of B(:,j) at a time, each step of their A-column lookups issued
             // for both before either is used (a lookup is a chain of dependent loads: B's
             // row, then AUX, then JC, then CP)
@@ -158,19 +191,61 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
             }
         } else {
             for (int64_t t = bs + sub; t < be; t += LPI) {
-                int32_t k = __ldg(pr->B.ir + t);
-                int64_t cs, ce;
-                col_range(pr->A, k, cs, ce);
-                long long len = ce - cs;
-                if (it.acs) {   // fill the A-column cache for the later passes
-                    it.acs[b0 + t] = cs;
-                    it.acl[b0 + t] = (int32_t)len;
-                }
+                const int32_t k = __ldg(pr->B.ir + t);
+                const long long len = analyze_entry(it, pr->A, k, b0 + t);
                 f += len;
                 mx = len > mx ? len : mx;
                 if (skp && k >= 0 && k < pr->A.n) sk |= __ldg(skp + k);
             }
         }
+    }
+    __syncthreads();
+    const int nlong = s_nlong;
+    for (int l = 0; l < nlong; ++l) {   // the CTA's long columns, one after another
+        const int g = s_long[l];
+        const int64_t ul = (int64_t)blockIdx.x * GRP + g;
+        const int lp = it.nprod == 1 ? 0 : __ldg(item_prod + ul);
+        const Prod* pr = it.prods + lp;
+        const int64_t p = ul - __ldg(it.item_base + lp);
+        const int64_t s0 = __ldg(pr->B.cp + p), e0 = __ldg(pr->B.cp + p + 1);
+        const uint64_t* skp = sketch ? sketch + sketch_base[lp] : nullptr;
+        const int64_t b0 = it.acs ? pr->bnz_base - __ldg(pr->B.cp) : 0;
+        long long lf = 0, lmx = 0;
+        unsigned long long lsk = 0;
+        constexpr int U = 4;
+        for (int64_t t0 = s0 + threadIdx.x; t0 < e0; t0 += 256 * U) {
+            int32_t k[U];
+            long long len[U];
+#pragma unroll
+            for (int i = 0; i < U; ++i) k[i] = t0 + 256 * i < e0 ? __ldg(pr->B.ir + t0 + 256 * i) : -1;
+#pragma unroll
+            for (int i = 0; i < U; ++i)
+                len[i] = t0 + 256 * i < e0 ? analyze_entry(it, pr->A, k[i], b0 + t0 + 256 * i) : 0;
+#pragma unroll
+            for (int i = 0; i < U; ++i) {
+                lf += len[i];
+                lmx = len[i] > lmx ? len[i] : lmx;
+                if (skp && k[i] >= 0 && k[i] < pr->A.n) lsk |= __ldg(skp + k[i]);
+            }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lf += __shfl_xor_sync(0xffffffffu, lf, o);
+            const long long om = __shfl_xor_sync(0xffffffffu, lmx, o);
+            lmx = om > lmx ? om : lmx;
+            lsk |= __shfl_xor_sync(0xffffffffu, lsk, o);
+        }
+        if ((threadIdx.x & 31) == 0) {
+            atomicAdd(&s_lf[g], (unsigned long long)lf);
+            atomicMax(&s_lmx[g], (unsigned long long)lmx);   // lengths are not negative
+            if (lsk) atomicOr(&s_lsk[g], lsk);
+        }
+    }
+    if (nlong > 0) __syncthreads();
+    if (is_long && sub == 0) {
+        f = (long long)s_lf[grp];
+        mx = (long long)s_lmx[grp];
+        sk = s_lsk[grp];
     }
 #pragma unroll
     for (int o = LPI / 2; o > 0; o >>= 1) {
@@ -216,8 +291,11 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
         }
     }
     __syncthreads();
-    if (threadIdx.x < NBIN && s_cnt[threadIdx.x]) atomicAdd(bin_count + threadIdx.x, s_cnt[threadIdx.x]);
-    if (threadIdx.x == 0 && flops_total) atomicAdd(flops_total, s_fl);
+    // the counters are kept in CTR_REP copies on lines of their own (32,768 CTAs adding to
+    // one line would queue in one L2 slice)
+    const int rep = (blockIdx.x & (CTR_REP - 1)) * CTR_STRIDE;
+    if (threadIdx.x < NBIN && s_cnt[threadIdx.x]) atomicAdd(bin_count + rep + threadIdx.x, s_cnt[threadIdx.x]);
+    if (threadIdx.x == 0 && flops_total) atomicAdd(flops_total + rep, s_fl);
 }
 
 // item_prod[u] = the product of item u: one CTA per product over its contiguous items.
@@ -239,6 +317,10 @@ void launch_analyze(cudaStream_t st, const Items& it, TierCfg cfg, int64_t* flop
         int grid = (int)ceil_div64(it.nitems, 256);
         k_analyze<1><<<grid, 256, 0, st>>>(it, cfg, flops, bin, item_prod, bin_count, flops_total, sketch,
                                            sketch_base, feat, maxlen);
+    } else if (it.total_bnz >= 32 * it.nitems) {
+        int grid = (int)ceil_div64(it.nitems * 32, 256);
+        k_analyze<32><<<grid, 256, 0, st>>>(it, cfg, flops, bin, item_prod, bin_count, flops_total, sketch,
+                                            sketch_base, feat, maxlen);
     } else {
         int grid = (int)ceil_div64(it.nitems * 8, 256);
         k_analyze<8><<<grid, 256, 0, st>>>(it, cfg, flops, bin, item_prod, bin_count, flops_total, sketch,
@@ -1015,40 +1097,53 @@ __host__ __device__ __forceinline__ int64_t slab_max_rows(int64_t m, int P) {
 // Slabs of the long columns: P per column, items[sbase[d] + q] = (d, q); the
 // storage bound of the slab row sets, sum over columns of min(flops, words),
 // accumulates in *store_bound (a slab stores min(words, rows) 4-byte entries and
-// rows <= flops).
+// rows <= flops).  The three global counters take one addition per warp (a column each
+// queued on one L2 line), and nothing here walks a column's slabs with 64-bit divisions:
+// R-MAT 20 flat 751 -> 27 us, R-MAT of 300,007 vertices 203 -> 10 us.
 __global__ void k_dense_items(Items it, const int2* __restrict__ dlist, int64_t nd, const int64_t* __restrict__ flops,
                               int part_flops, int RB, int2* items, unsigned long long* nitems, int8_t* nparts,
                               int32_t* sbase, unsigned long long* store_bound, int64_t* bbase,
                               unsigned long long* bnd_total) {
-    int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (d >= nd) return;
-    const int2 e = dlist[d];
-    const Prod* pr = it.prods + e.x;
-    const int64_t f = flops[__ldg(it.item_base + e.x) + e.y];
-    const int64_t deg = __ldg(pr->B.cp + e.y + 1) - __ldg(pr->B.cp + e.y);
-    const int64_t m = pr->A.m;
-    // slab rows stay <= RB: the fewest slabs whose 32-aligned cuts all fit (the host
-    // sized RB so that MAX_PARTS slabs always do)
-    int64_t pmin = m <= RB ? 1 : ceil_div64(m, (int64_t)RB);
-    while (pmin < MAX_PARTS && slab_max_rows(m, (int)pmin) > RB) ++pmin;
-    int64_t P = ceil_div64(f, part_flops);
-    const int64_t pdeg = f / (32 * (deg > 0 ? deg : 1));   // about 32 products per (slab, B entry) at least
-    P = P < pdeg ? P : pdeg;
-    P = P < pmin ? pmin : P;
-    P = P > MAX_PARTS ? MAX_PARTS : P;
-    P = P < 1 ? 1 : P;
-    nparts[d] = (int8_t)P;
-    int64_t words = 0;
-    for (int q = 0; q < P; ++q) {
-        int64_t R0, R1;
-        slab_rows(m, q, (int)P, R0, R1);
-        words += (R1 - R0 + 31) >> 5;
+    const int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    const bool ok = d < nd;
+    long long P = 0, bound = 0, bnd = 0;
+    if (ok) {
+        const int2 e = dlist[d];
+        const Prod* pr = it.prods + e.x;
+        const int64_t f = flops[__ldg(it.item_base + e.x) + e.y];
+        const int64_t deg = __ldg(pr->B.cp + e.y + 1) - __ldg(pr->B.cp + e.y);
+        const int64_t m = pr->A.m;
+        // slab rows stay <= RB: the fewest slabs whose 32-aligned cuts all fit (the host
+        // sized RB so that MAX_PARTS slabs always do); a cut moves a slab's ends by at
+        // most 31 rows
+        int64_t pmin = m <= RB ? 1 : ceil_div64(m, (int64_t)RB);
+        while (pmin > 1 && pmin < MAX_PARTS && ceil_div64(m, pmin) + 31 > RB && slab_max_rows(m, (int)pmin) > RB) ++pmin;
+        P = ceil_div64(f, part_flops);
+        const int64_t pdeg = f / (32 * (deg > 0 ? deg : 1));   // about 32 products per (slab, B entry) at least
+        P = P < pdeg ? P : pdeg;
+        P = P < pmin ? pmin : P;
+        P = P > MAX_PARTS ? MAX_PARTS : P;
+        P = P < 1 ? 1 : P;
+        const int64_t words = (m + 31) >> 5;   // of all its slabs: every inner cut is a multiple of 32
+        bound = f < words ? f : words;
+        // boundary table: P + 1 rows of deg positions (where each slab starts in every A(:,k)),
+        // then two rows with where every A(:,k) starts (low and high 32 bits)
+        bnd = (P + 3) * deg;
     }
-    atomicAdd(store_bound, (unsigned long long)(f < words ? f : words));
-    // boundary table: P + 1 rows of deg positions (where each slab starts in every A(:,k)),
-    // then two rows with where every A(:,k) starts (low and high 32 bits)
-    bbase[d] = (int64_t)atomicAdd(bnd_total, (unsigned long long)((P + 3) * deg));
-    unsigned long long base = atomicAdd(nitems, (unsigned long long)P);
+    const long long ip = warp_incl_scan64(P), ib = warp_incl_scan64(bnd), sb = warp_sum(bound);
+    unsigned long long bp = 0, bb = 0;
+    if (lane == 31) {
+        bp = atomicAdd(nitems, (unsigned long long)ip);
+        bb = atomicAdd(bnd_total, (unsigned long long)ib);
+        atomicAdd(store_bound, (unsigned long long)sb);
+    }
+    bp = __shfl_sync(0xffffffffu, bp, 31);
+    bb = __shfl_sync(0xffffffffu, bb, 31);
+    if (!ok) return;
+    const int64_t base = (int64_t)bp + ip - P;
+    nparts[d] = (int8_t)P;
+    bbase[d] = (int64_t)bb + ib - bnd;
     sbase[d] = (int32_t)base;
     for (int q = 0; q < P; ++q) items[base + q] = make_int2((int)d, q);
 }

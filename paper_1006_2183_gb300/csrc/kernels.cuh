@@ -39,6 +39,11 @@ constexpr int DEFAULT_SLAB_ROWS = 1 << 19;
 // 67.9 / 64.5 / 62.3 / 62.1 ms for the FP64 numeric pass)
 constexpr int DEFAULT_PART_FLOPS = 65536;
 
+// copies of the analysis counters (bin counts, then total flops), one 128-byte line each
+constexpr int CTR_REP = 16;
+constexpr int CTR_STRIDE = 16;
+static_assert(NBIN + 1 <= CTR_STRIDE, "one line per copy");
+
 struct TierCfg {
     int warp_max;     // cap <= warp_max -> warp tables (<= 512)
     int block_max;    // cap <= block_max -> CTA tables (<= 4096)
@@ -133,7 +138,8 @@ constexpr int64_t BM_MAX_ROWS = 262144;
 constexpr int64_t BM_WARP_MAX_ROWS = 32768;
 constexpr int BM_WARP_MIN_TBL = 256;   // smaller tables hold too few rows to prefer the bitmap
 
-// flops and bin per item, product id per item, bin counts and total flops.
+// flops and bin per item, product id per item, bin counts and total flops (CTR_REP partial
+// copies each, CTR_STRIDE entries apart: bin_count[r * CTR_STRIDE + b]).
 // With feat != nullptr also the 8 predictor inputs per item; `sketch` holds the
 // per-column row sketches of the A operands concatenated, product i's starting
 // at sketch_base[i].
