@@ -2,15 +2,11 @@
 // formulation, Section 2.1; accumulation in the spirit of the sparse
 // accumulator of Section 3.3), organised in accumulator tiers chosen per
 // output column from cap = min(flops, m):
-//   * one thread per column for flops <= 16 (insertion sort in registers),
-//   * warp-wide shared-memory hash tables (short columns),
+//   * up to 512 products: sorted in the registers of 8 to 32 lanes (sorttier.cu),
+//   * warp-wide shared-memory hash tables (short columns of many products),
 //   * CTA-wide shared-memory hash tables (medium columns),
-//   * the range tier (long columns): the symbolic pass marks the column's rows
-//     in a shared-memory bitmap per row slab and cuts the slab into row ranges
-//     of bounded output; the numeric pass walks the ranges in row order with
-//     per-(column, k) cursors into A(:,k), accumulates each range in a hash
-//     table (or a dense row array when the range is narrow) and writes it out
-//     in row order through the range's bitmap.
+//   * the slab tier (long columns): row slabs, each counted through a row bitmap in
+//     shared memory and accumulated at its rows' ranks.
 // The symbolic pass counts nnz per output column; the numeric pass fills rows
 // and values, in ascending row order without a sort wherever a row bitmap fits
 // in shared memory.  Every kernel works on items (product, stored column of B).
@@ -65,18 +61,16 @@ constexpr int WARP_BLOCK = 256;   // 8 warp groups per CTA
 __host__ __device__ __forceinline__ int bin_of(int64_t flops, int64_t cap, int warp_max, int block_max,
                                               int sort_max) {
     if (cap <= 0) return 0;
-    if (flops <= TINY_MAX) return BIN_TINY;
+    if (flops <= TINY_MAX) return BIN_SORT0;
+    if (cap <= warp_max && flops <= sort_max) {
+        int b = BIN_SORT0 + 1;
+        for (int64_t t = 2 * TINY_MAX; t < flops; t <<= 1) ++b;
+        return b;
+    }
     if (cap <= warp_max) {
-        // with sort_max, a column of more than sort_max products never lands in a bin
-        // whose table is for at most sort_max rows: bins 2 and 3 then also bound flops
-        int64_t c = cap;
-        if (sort_max > 0) {
-            const int64_t fl = flops < sort_max + 1 ? flops : sort_max + 1;
-            c = cap > fl ? cap : fl;
-        }
         int64_t t = WARP_TBL0;
         int b = BIN_WARP0;
-        while (t < 2 * c) { t <<= 1; ++b; }
+        while (t < 2 * cap) { t <<= 1; ++b; }
         return b;
     }
     if (cap <= block_max) {
@@ -365,7 +359,7 @@ __global__ void k_numeric_bins(Items it, TierCfg cfg, const uint8_t* __restrict_
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < it.nitems; u += (int64_t)gridDim.x * blockDim.x) {
         const int b = bin[u];
         int nb = 0;
-        if (b >= BIN_TINY && b < BIN_DENSE) nb = bin_of(flops[u], nnz_item[u], cfg.warp_max, cfg.block_max, cfg.sort_max);
+        if (b >= BIN_SORT0 && b < BIN_DENSE) nb = bin_of(flops[u], nnz_item[u], cfg.warp_max, cfg.block_max, cfg.sort_max);
         nbin[u] = (uint8_t)nb;
         if (nb) atomicAdd(&s_cnt[nb], 1ull);
     }
@@ -1012,11 +1006,23 @@ static void run_tiny(cudaStream_t st, const Items& it, const int2* list, int64_t
 // every A_i has at most BLOCK_TIER_MAX_ROWS rows: numeric passes run in the block tier
 static bool block_mode(const Items& it) { return it.max_m > 0 && it.max_m <= BLOCK_TIER_MAX_ROWS; }
 
+// Columns of few products, counting or numeric: the sort tier, or, where not even 16
+// products fit its keys (2^28 rows and more), a thread per column of at most 16.
+template <class SR, bool NUM>
+static void run_short(cudaStream_t st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
+                      int64_t* nnz_item, const int64_t* Coff, int32_t* Cir, typename SR::T* Cv, const int* vals_zero) {
+    if (sort_max_products(it.max_m) == 0)
+        run_tiny<SR, NUM>(st, it, list + off[BIN_SORT0], cnt[BIN_SORT0], nnz_item, Coff, Cir, Cv);
+    else if constexpr (NUM) launch_sort_tier<SR>(st, it, list, off, cnt, nnz_item, Coff, Cir, Cv, vals_zero);
+    else launch_sort_count(st, it, list, off, cnt, nnz_item);
+}
+
 template <class SR, bool NUM>
 static void run_hash_bins(cudaStream_t st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
-                          int64_t* nnz_item, const int64_t* Coff, int32_t* Cir, typename SR::T* Cv) {
+                          int64_t* nnz_item, const int64_t* Coff, int32_t* Cir, typename SR::T* Cv,
+                          const int* vals_zero = nullptr) {
     constexpr int W0 = BIN_WARP0, B0 = BIN_BLK0;
-    run_tiny<SR, NUM>(st, it, list + off[BIN_TINY], cnt[BIN_TINY], nnz_item, Coff, Cir, Cv);
+    run_short<SR, NUM>(st, it, list, off, cnt, nnz_item, Coff, Cir, Cv, vals_zero);
     run_hash<SR, 32, 64, NUM, WARP_BLOCK>(st, it, list + off[W0], cnt[W0], nnz_item, Coff, Cir, Cv);
     run_hash<SR, 32, 128, NUM, WARP_BLOCK>(st, it, list + off[W0 + 1], cnt[W0 + 1], nnz_item, Coff, Cir, Cv);
     if constexpr (!NUM) {
@@ -1840,11 +1846,11 @@ void launch_numeric_predicted(cudaStream_t st, const Items& it, const int2* list
                               const int64_t* bin_cnt, const DenseWork& dw, const int64_t* cap_off, int64_t* nnz_item,
                               int32_t* Cir, typename SR::T* Cv) {
     if (block_mode(it)) {
-        run_tiny<SR, true>(st, it, list + bin_off[BIN_TINY], bin_cnt[BIN_TINY], nnz_item, cap_off, Cir, Cv);
+        run_short<SR, true>(st, it, list, bin_off, bin_cnt, nnz_item, cap_off, Cir, Cv, dw.vals_zero);
         launch_block_tier<SR>(st, it, list, bin_off, bin_cnt, dw, nnz_item, cap_off, Cir, Cv, 1);
         return;
     }
-    run_hash_bins<SR, true>(st, it, list, bin_off, bin_cnt, nnz_item, cap_off, Cir, Cv);
+    run_hash_bins<SR, true>(st, it, list, bin_off, bin_cnt, nnz_item, cap_off, Cir, Cv, dw.vals_zero);
 }
 
 template <class SR>
@@ -1864,11 +1870,11 @@ void launch_numeric(cudaStream_t st, const Items& it, TierCfg cfg, const int2* l
                     typename SR::T* Cv, int which) {
     (void)cfg;
     if (block_mode(it)) {
-        if (which & 1) run_tiny<SR, true>(st, it, list + bin_off[BIN_TINY], bin_cnt[BIN_TINY], nullptr, Coff, Cir, Cv);
+        if (which & 1) run_short<SR, true>(st, it, list, bin_off, bin_cnt, nullptr, Coff, Cir, Cv, dw.vals_zero);
         launch_block_tier<SR>(st, it, list, bin_off, bin_cnt, dw, nullptr, Coff, Cir, Cv, which);
         return;
     }
-    if (which & 1) run_hash_bins<SR, true>(st, it, list, bin_off, bin_cnt, nullptr, Coff, Cir, Cv);
+    if (which & 1) run_hash_bins<SR, true>(st, it, list, bin_off, bin_cnt, nullptr, Coff, Cir, Cv, dw.vals_zero);
     if (which & 2) run_slabs<SR>(st, it, dw, true, Coff, Cir, Cv);
 }
 

@@ -14,16 +14,18 @@
 namespace sg {
 
 // Column tiers.  An item's capacity bound is cap = min(flops, m) >= nnz of its output.
-//   bin 0                  : cap == 0 (empty output column)
-//   bin 1                  : flops <= TINY_MAX: one thread, products sorted in registers
-//   bins 2 .. NWARP+1      : warp-wide hash tables of 64 .. 1024 slots (>= 2 cap)
-//   bins NWARP+2 .. +NBLK  : CTA-wide hash tables of 2048 .. 8192 slots (>= 2 cap)
-//   bin NBIN-1             : slab tier (long columns cut into row slabs)
+//   bin 0                          : cap == 0 (empty output column)
+//   bins BIN_SORT0 .. +NSORT-1     : at most 16, 32 .. 512 products (sort tier, up to
+//                                    TierCfg::sort_max products; 16 products always)
+//   bins BIN_WARP0 .. +NWARP-1     : warp-wide hash tables of 64 .. 1024 slots (>= 2 cap)
+//   bins BIN_BLK0 .. +NBLK-1       : CTA-wide hash tables of 2048 .. 8192 slots (>= 2 cap)
+//   bin NBIN-1                     : slab tier (long columns cut into row slabs)
+constexpr int NSORT = 6;
 constexpr int NWARP = 5;
 constexpr int NBLK = 3;
-constexpr int NBIN = 2 + NWARP + NBLK + 1;
-constexpr int BIN_TINY = 1;
-constexpr int BIN_WARP0 = 2;
+constexpr int NBIN = 1 + NSORT + NWARP + NBLK + 1;
+constexpr int BIN_SORT0 = 1;
+constexpr int BIN_WARP0 = BIN_SORT0 + NSORT;
 constexpr int BIN_BLK0 = BIN_WARP0 + NWARP;
 constexpr int BIN_DENSE = NBIN - 1;
 constexpr int TINY_MAX = 16;
@@ -39,16 +41,16 @@ constexpr int DEFAULT_SLAB_ROWS = 1 << 19;
 // 67.9 / 64.5 / 62.3 / 62.1 ms for the FP64 numeric pass)
 constexpr int DEFAULT_PART_FLOPS = 65536;
 
-// copies of the analysis counters (bin counts, then total flops), one 128-byte line each
+// copies of the analysis counters (bin counts, then total flops), two 128-byte lines each
 constexpr int CTR_REP = 16;
-constexpr int CTR_STRIDE = 16;
-static_assert(NBIN + 1 <= CTR_STRIDE, "one line per copy");
+constexpr int CTR_STRIDE = 32;
+static_assert(NBIN + 1 <= CTR_STRIDE, "a copy keeps to its lines");
 
 struct TierCfg {
     int warp_max;     // cap <= warp_max -> warp tables (<= 512)
     int block_max;    // cap <= block_max -> CTA tables (<= 4096)
-    int sort_max = 0; // > 0 (operands of at most BLOCK_TIER_MAX_ROWS rows): bins 2, 3 and 4
-                      // hold only columns of at most 32, 64 and 128 products (the sort tier)
+    int sort_max = 0; // columns of at most this many products (and cap <= warp_max) go to the
+                      // sort tier: sort_max_products(rows), less where another tier is faster
     int dense_rows;   // RB, most rows of one slab (bitmap bits in shared memory)
     int part_flops;   // target flops per slab of a long column
 };
@@ -104,6 +106,15 @@ struct DenseWork {
 // the block tier (two-level row bitmap per column, L2 reductions; blocktier.cu)
 // and count their columns with row bitmaps.
 constexpr int BLOCK_TIER_MAX_ROWS = 32768;
+
+// Most products of a column whose 32-bit keys in the sort tier (sorttier.cu) hold its rows:
+// a key is the row above log2(products) bits of slot, and all ones marks an empty slot.
+// 0: the rows leave no room even for 16 products.
+inline int sort_max_products(int64_t max_m) {
+    for (int n = 512, sb = 9; n >= TINY_MAX; n /= 2, --sb)
+        if (max_m <= (int64_t(1) << (32 - sb)) - 1) return n;
+    return 0;
+}
 
 struct Items {
     const Prod* prods = nullptr;        // device, nprod descriptors
@@ -185,6 +196,14 @@ template <class SR>
 void launch_block_tier(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
                        const int64_t* bin_cnt, const DenseWork& dw, int64_t* nnz_item, const int64_t* Coff,
                        int32_t* Cir, typename SR::T* Cv, int which);
+// numeric pass of the sort bins (sorttier.cu); nnz_item as for launch_block_tier
+template <class SR>
+void launch_sort_tier(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+                      const int64_t* bin_cnt, int64_t* nnz_item, const int64_t* Coff, int32_t* Cir,
+                      typename SR::T* Cv, const int* vals_zero);
+// counting pass of the sort bins
+void launch_sort_count(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+                       const int64_t* bin_cnt, int64_t* nnz_item);
 // nnz of long columns = sum of their slab counts (and each slab's start in its column)
 void launch_sum_parts(cudaStream_t st, const Items& it, const DenseWork& dw, int64_t* nnz_item);
 // per-product column pointers from item offsets: out[colbase_i + j] for j in [0, n_i]

@@ -1,0 +1,297 @@
+// Sort tier: columns of at most 512 products (TierCfg::sort_max), whatever the number
+// of rows that the keys hold.  A group of G lanes takes one output column
+// C(:,j) = (+)_{k in B(:,j)} A(:,k) (x) B(k,j) (Section 2.1), N = G K products at most:
+//   1. product p goes to lane p mod G as the key (row << log2 N) | p, its value to slot
+//      p of shared memory;
+//   2. a bitonic network sorts the keys, element i = K lane + r in register r of its
+//      lane: the steps at distances below K stay inside a lane, so a network over N
+//      elements takes log2 G (log2 G + 1) / 2 shuffled steps (6 for 64 products on 8
+//      lanes, where one register per lane on 32 lanes and 2 per lane would take 15);
+//   3. equal rows are adjacent: a lane adds its runs up in ascending k, runs that cross
+//      lanes go through a segmented scan, which is skipped where no run does (FP64
+//      additions are the slow pipe of this part, about two lanes per SM clock);
+//   4. rows and values are put in order in shared memory and stored coalesced.
+// No atomics, no tables to fill and empty, and several columns per warp share the
+// latency of the loads that a column starts with.  The counting form sorts rows alone.
+// Bound by instruction issue and the FP64 pipe, not by memory.  Against one warp per
+// column with 32-lane networks and, for operands of many rows, shared-memory hash tables
+// whose entries were then sorted: R*(A*P) on 128^3 FP64, 262,144 columns of 50 to 60
+// products and as many of about 32, 736 -> 310 us (counting 294 -> 168 us); 20 int64 pairs,
+// columns of up to 512 products, 1.25 -> 0.41 ms (counting 0.24 -> 0.18 ms).
+#include <algorithm>
+
+#include "internal.cuh"
+
+namespace sg {
+namespace {
+
+// threads per CTA: 8 warps, 4 where a column's slots take 6 KB
+constexpr int st_block(int K) { return K == 16 ? 128 : 256; }
+
+constexpr int ilog2(int x) { return x <= 1 ? 0 : 1 + ilog2(x / 2); }
+
+// shared-memory index of element i: one gap per 8 elements, so that lanes writing K
+// apart do not meet in a bank
+__device__ __forceinline__ int st_ph(int i) { return i + (i >> 3); }
+template <int N>
+constexpr int st_span() { return N + N / 8; }
+
+template <int G, class V>
+__device__ __forceinline__ V shflg(V x, int src) {
+    if constexpr (sizeof(V) == 1) return (V)__shfl_sync(0xffffffffu, (int)x, src, G);
+    else return __shfl_sync(0xffffffffu, x, src, G);
+}
+
+// a (x) b, where `one` says that b is the semiring's one: plus-times then leaves a as it is
+// without a multiplication (the merges' selector; FP64 multiplies at two lanes per clock)
+template <class SR>
+__device__ __forceinline__ typename SR::Acc mul_by(typename SR::T a, typename SR::T b, bool one) {
+    if constexpr (SR::id == SPGEMM_PLUS_TIMES_F64 || SR::id == SPGEMM_PLUS_TIMES_I64) {
+        if (one) return (typename SR::Acc)a;
+    }
+    return SR::mul(a, b);
+}
+
+// Ascending bitonic sort of the N = G K keys of a group (element i = K lane + r).
+template <int G, int K>
+__device__ __forceinline__ void sort_keys(uint32_t (&key)[K], int lane) {
+    constexpr int N = G * K;
+#pragma unroll
+    for (int k = 2; k <= N; k <<= 1) {
+#pragma unroll
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            if (j >= K) {
+                const int d = j / K;
+                const bool asc = k == N || (lane & (k / K)) == 0;
+                const bool take_min = asc == ((lane & d) == 0);
+#pragma unroll
+                for (int r = 0; r < K; ++r) {
+                    const uint32_t o = __shfl_xor_sync(0xffffffffu, key[r], d, G);
+                    key[r] = take_min ? min(key[r], o) : max(key[r], o);
+                }
+            } else {
+#pragma unroll
+                for (int r = 0; r < K; ++r) {
+                    if (r & j) continue;
+                    const bool asc = k == N || (k < K ? (r & k) == 0 : (lane & (k / K)) == 0);
+                    const uint32_t a = key[r], b = key[r | j];
+                    key[r] = asc ? min(a, b) : max(a, b);
+                    key[r | j] = asc ? max(a, b) : min(a, b);
+                }
+            }
+        }
+    }
+}
+
+// Inclusive scan over a group of G lanes.
+template <int G>
+__device__ __forceinline__ int scan_g(int v, int lane) {
+#pragma unroll
+    for (int o = 1; o < G; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, v, o, G);
+        if (lane >= o) v += t;
+    }
+    return v;
+}
+
+// NUM: rows and values to C (Coff as for launch_block_tier); otherwise counts to nnz_item.
+template <class SR, int G, int K, bool NUM>
+__global__ void __launch_bounds__(st_block(K)) k_sort(Items it, const int2* __restrict__ list, int64_t count,
+                                                   int64_t* __restrict__ nnz_item, const int64_t* __restrict__ Coff,
+                                                   int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv,
+                                                   const int* __restrict__ vals_zero) {
+    using T = typename SR::T;
+    using Acc = typename SR::Acc;
+    constexpr int N = G * K, SB = ilog2(N), NG = st_block(K) / G, SPAN = st_span<N>();
+    constexpr uint32_t NONE = 0xffffffffu;
+    constexpr uint32_t NOROW = NONE >> SB;   // no stored row (the host bounds the rows)
+    __shared__ Acc s_val[NUM ? NG * SPAN : 1];
+    __shared__ int32_t s_row[NUM ? NG * SPAN : 1];
+    const int lane = threadIdx.x & (G - 1), grp = threadIdx.x / G;
+    Acc* sv = s_val + (NUM ? grp * SPAN : 0);
+    int32_t* sr = s_row + (NUM ? grp * SPAN : 0);
+    // boolean products whose operands hold no false value: every output value is true
+    const bool walk = NUM && (SR::id != SPGEMM_OR_AND_BOOL || vals_zero == nullptr || *vals_zero != 0);
+    // the groups of a warp go round together (their shuffles name the whole warp)
+    const int64_t step = (int64_t)gridDim.x * NG;
+    for (int64_t w0 = (int64_t)blockIdx.x * NG + (grp & ~(32 / G - 1)); w0 < count; w0 += step) {
+        const int64_t w = w0 + (grp & (32 / G - 1));
+        const bool act = w < count;
+        int2 e = make_int2(0, 0);
+        if (act) e = __ldg(list + w);
+        const Prod* pr = it.prods + e.x;
+        const int64_t u = __ldg(it.item_base + e.x) + e.y;
+        int64_t bs = 0, be = 0;
+        if (act) {
+            bs = __ldg(pr->B.cp + e.y);
+            be = __ldg(pr->B.cp + e.y + 1);
+        }
+        const uint32_t m = (uint32_t)pr->A.m;
+        const bool b_one = __all_sync(0xffffffffu, pr->B.num == nullptr);   // of every group of the warp
+        uint32_t key[K];
+#pragma unroll
+        for (int r = 0; r < K; ++r) key[r] = NONE;
+        // 1. products: the entries of B(:,j) G at a time (the bin bounds their products by N)
+        int base = 0;
+        for (int64_t b0 = bs; __any_sync(0xffffffffu, b0 < be && base < N); b0 += G) {
+            const int64_t t = b0 + lane;
+            int len = 0;
+            int64_t a0 = 0;
+            T bv = T(0);
+            if (t < be) {
+                const int32_t k = __ldg(pr->B.ir + t);
+                int64_t sa, ea;
+                a_col(it, pr, t, k, sa, ea);
+                a0 = sa;
+                len = (int)(ea - sa);
+                if (walk) bv = load_val<SR>(pr->B, t);
+            }
+            const int inc = scan_g<G>(len, lane);
+            const int tot = __shfl_sync(0xffffffffu, inc, G - 1, G);
+            a0 -= inc - len;   // product p of the chunk is at a0 + p of its entry
+#pragma unroll
+            for (int r = 0; r < K; ++r) {
+                const int p = r * G + lane - base;   // the slot's product within this chunk
+                if (!__any_sync(0xffffffffu, p >= 0 && p < tot)) continue;
+                int src = 0;                         // entries that end at or before product p
+#pragma unroll
+                for (int st = G / 2; st > 0; st >>= 1)
+                    if (__shfl_sync(0xffffffffu, inc, src + st - 1, G) <= p) src += st;
+                const int64_t as = __shfl_sync(0xffffffffu, a0, src, G);
+                T bvs = T(0);
+                if constexpr (NUM) bvs = shflg<G>(bv, src);
+                if (p >= 0 && p < tot) {
+                    const int32_t row = __ldg(pr->A.ir + as + p);
+                    if ((uint32_t)row < m) {   // else malformed input: skipped
+                        key[r] = ((uint32_t)row << SB) | (uint32_t)(r * G + lane);
+                        if constexpr (NUM)
+                            sv[st_ph(r * G + lane)] = walk ? mul_by<SR>(load_val<SR>(pr->A, as + p), bvs, b_one) : SR::one();
+                    }
+                }
+            }
+            base += tot;
+        }
+        // 2. order
+        sort_keys<G, K>(key, lane);
+        // 3. runs of equal rows: the last element of a run holds its sum
+        const uint32_t first = key[0] >> SB, last = key[K - 1] >> SB;
+        uint32_t before = __shfl_up_sync(0xffffffffu, last, 1, G), after = __shfl_down_sync(0xffffffffu, first, 1, G);
+        if (lane == 0) before = NOROW;
+        if (lane == G - 1) after = NOROW;
+        uint32_t end = 0;   // bit r: element r is the last of its run
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            const uint32_t nx = r + 1 < K ? key[r + 1 < K ? r + 1 : r] >> SB : after;
+            if (key[r] != NONE && nx != (key[r] >> SB)) end |= 1u << r;
+        }
+        const int c = __popc(end);
+        const int inc = scan_g<G>(c, lane);
+        const int cnt = __shfl_sync(0xffffffffu, inc, G - 1, G);
+        if constexpr (!NUM) {
+            if (act && lane == 0) nnz_item[u] = cnt;
+        } else {
+            __syncwarp();
+            Acc v[K];
+#pragma unroll
+            for (int r = 0; r < K; ++r) v[r] = key[r] != NONE ? sv[st_ph((int)(key[r] & (N - 1)))] : SR::zero();
+#pragma unroll
+            for (int r = 1; r < K; ++r) {
+                const bool same = key[r] != NONE && (key[r] >> SB) == (key[r - 1] >> SB);
+                if (__any_sync(0xffffffffu, same)) v[r] = same ? SR::add(v[r - 1], v[r]) : v[r];
+            }
+            // a run that continues the lane before's last one takes that lane's sum
+            const bool cont = key[0] != NONE && before == first;
+            if (__any_sync(0xffffffffu, cont)) {
+                Acc s = v[K - 1];
+                int through = cont && last == first && key[K - 1] != NONE;   // one run, from the lane before's
+#pragma unroll
+                for (int d = 1; d < G; d <<= 1) {
+                    const Acc sp = shflg<G>(s, lane >= d ? lane - d : lane);
+                    const int tp = __shfl_up_sync(0xffffffffu, through, d, G);
+                    if (lane >= d && through) {
+                        s = SR::add(sp, s);
+                        through = tp;
+                    }
+                }
+                const Acc carry = shflg<G>(s, lane > 0 ? lane - 1 : 0);
+#pragma unroll
+                for (int r = 0; r < K; ++r) {
+                    const bool take = cont && ((end >> r) & 1u) && (key[r] >> SB) == first;
+                    if (__any_sync(0xffffffffu, take)) v[r] = take ? SR::add(carry, v[r]) : v[r];
+                }
+            }
+            __syncwarp();   // every value is out of its slot
+            // 4. the column in order, then coalesced stores
+            int pos = inc - c;
+#pragma unroll
+            for (int r = 0; r < K; ++r)
+                if ((end >> r) & 1u) {
+                    sr[st_ph(pos)] = (int32_t)(key[r] >> SB);
+                    sv[st_ph(pos)] = v[r];
+                    ++pos;
+                }
+            __syncwarp();
+            if (act) {
+                const int64_t out0 = __ldg(Coff + u);
+                const int64_t capn = __ldg(Coff + u + 1) - out0;
+                if (nnz_item && lane == 0) nnz_item[u] = cnt;
+                // exact offsets always fit; with nnz_item a column that does not fit its
+                // slots is only counted
+                if (cnt <= capn) {
+                    const int32_t rb = out_row_base(pr, e.y);
+                    for (int i = lane; i < cnt; i += G) {
+                        __stcs(Cir + out0 + i, sr[st_ph(i)] + rb);
+                        Cv[out0 + i] = SR::out(sv[st_ph(i)]);
+                    }
+                }
+            }
+            __syncwarp();   // the slots are free for the next column
+        }
+    }
+}
+
+template <class SR, int G, int K, bool NUM>
+void run(cudaStream_t st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item, const int64_t* Coff,
+         int32_t* Cir, typename SR::T* Cv, const int* vals_zero) {
+    if (count <= 0) return;
+    const int grid = (int)std::min<int64_t>(ceil_div64(count, st_block(K) / G), (int64_t)sm_count() * 32);
+    k_sort<SR, G, K, NUM><<<grid, st_block(K), 0, st>>>(it, list, count, nnz_item, Coff, Cir, Cv, vals_zero);
+    note_launch();
+}
+
+template <class SR, bool NUM>
+void run_bins(cudaStream_t st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
+              int64_t* nnz_item, const int64_t* Coff, int32_t* Cir, typename SR::T* Cv, const int* vz) {
+    constexpr int S = BIN_SORT0;
+    run<SR, 8, 2, NUM>(st, it, list + off[S], cnt[S], nnz_item, Coff, Cir, Cv, vz);
+    run<SR, 8, 4, NUM>(st, it, list + off[S + 1], cnt[S + 1], nnz_item, Coff, Cir, Cv, vz);
+    run<SR, 8, 8, NUM>(st, it, list + off[S + 2], cnt[S + 2], nnz_item, Coff, Cir, Cv, vz);
+    run<SR, 16, 8, NUM>(st, it, list + off[S + 3], cnt[S + 3], nnz_item, Coff, Cir, Cv, vz);
+    run<SR, 32, 8, NUM>(st, it, list + off[S + 4], cnt[S + 4], nnz_item, Coff, Cir, Cv, vz);
+    run<SR, 32, 16, NUM>(st, it, list + off[S + 5], cnt[S + 5], nnz_item, Coff, Cir, Cv, vz);
+}
+
+}  // namespace
+
+template <class SR>
+void launch_sort_tier(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+                      const int64_t* bin_cnt, int64_t* nnz_item, const int64_t* Coff, int32_t* Cir,
+                      typename SR::T* Cv, const int* vals_zero) {
+    run_bins<SR, true>(st, it, list, bin_off, bin_cnt, nnz_item, Coff, Cir, Cv, vals_zero);
+}
+
+void launch_sort_count(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+                       const int64_t* bin_cnt, int64_t* nnz_item) {
+    run_bins<MP32, false>(st, it, list, bin_off, bin_cnt, nnz_item, nullptr, nullptr, nullptr, nullptr);
+}
+
+#define SG_INST(SR)                                                                                             \
+    template void launch_sort_tier<SR>(cudaStream_t, const Items&, const int2*, const int64_t*, const int64_t*, \
+                                       int64_t*, const int64_t*, int32_t*, typename SR::T*, const int*);
+SG_INST(PT64)
+SG_INST(MP32)
+SG_INST(BOOL8)
+SG_INST(PTI64)
+#undef SG_INST
+
+}  // namespace sg
