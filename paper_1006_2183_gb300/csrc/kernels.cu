@@ -1684,12 +1684,19 @@ __global__ void __launch_bounds__(RT_BLOCK, 2) k_slab_num(Items it, DenseWork dw
         } else {
             for (int x = tid; x < ng * 4; x += RT_BLOCK) bitmap[x] = 0u;
             __syncthreads();
-            for (int i0 = 0; i0 < cnt; i0 += RT_BLOCK) {
-                const int i = i0 + tid;
-                const int32_t r = i < cnt ? (int32_t)__ldcs(rs + i) : -1;
-                const int lr = (int)(r - R0);
-                if (i < cnt) {
-                    __stcs(Cir + ob + i, r + rb);    // C's rows: the row list itself
+            // four rows per thread in flight: the list comes from DRAM, and one load at a
+            // time left this loop waiting for it (R-MAT 20 flat FP64: 55.0 -> 51.6 ms)
+            constexpr int U = 4;
+            for (int i0 = tid; i0 < cnt; i0 += RT_BLOCK * U) {
+                int32_t r[U];
+#pragma unroll
+                for (int x = 0; x < U; ++x)
+                    r[x] = i0 + x * RT_BLOCK < cnt ? (int32_t)__ldcs(rs + i0 + x * RT_BLOCK) : -1;
+#pragma unroll
+                for (int x = 0; x < U; ++x) {
+                    if (i0 + x * RT_BLOCK >= cnt) break;
+                    const int lr = (int)(r[x] - R0);
+                    __stcs(Cir + ob + i0 + x * RT_BLOCK, r[x] + rb);    // C's rows: the row list itself
                     atomicOr(&bitmap[lr >> 5], 1u << (lr & 31));
                 }
             }
