@@ -19,7 +19,7 @@ spgemm_status_t set_err(spgemm_ctx* ctx, spgemm_status_t s, const char* fmt, ...
         if (s != SPGEMM_OK) {
             // queued reads whose destinations the failing call is about to abandon
             ctx->rb_pending.clear();
-            ctx->rb_used = 0;
+            ctx->rb_used = ctx->rb_launched = 0;
         }
     }
     return s;
@@ -65,21 +65,19 @@ size_t sr_size(spgemm_semiring_t sr) {
     return 0;
 }
 
-spgemm_status_t sync_ctx(spgemm_ctx* ctx) {
-    const cudaError_t e = cudaStreamSynchronize(ctx->stream);
-    if (e == cudaSuccess) {
-        for (const auto& r : ctx->rb_pending) std::memcpy(r.dst, ctx->rb_host + r.off, r.bytes);
-    }
-    ctx->rb_pending.clear();
-    ctx->rb_used = 0;
-    SG_CUDA(ctx, e);
-    SG_CUDA(ctx, cudaGetLastError());
-    return SPGEMM_OK;
-}
-
 namespace {
-// dst (mapped host memory) <- src (device), 8 bytes per thread when both are aligned
-__global__ void k_read_back(unsigned char* __restrict__ dst, const unsigned char* __restrict__ src, size_t bytes) {
+// Device-to-host reads of one wait, in one launch: dst[i] (mapped host memory) <- src[i],
+// 8 bytes per thread where both are aligned.
+constexpr int RB_MAX = 8;
+struct ReadList {
+    unsigned char* dst[RB_MAX];
+    const unsigned char* src[RB_MAX];
+    size_t bytes[RB_MAX];
+};
+__global__ void k_read_back(ReadList l) {
+    unsigned char* __restrict__ dst = l.dst[blockIdx.y];
+    const unsigned char* __restrict__ src = l.src[blockIdx.y];
+    const size_t bytes = l.bytes[blockIdx.y];
     const size_t i0 = (size_t)blockIdx.x * blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
     if ((((uintptr_t)src | (uintptr_t)dst | bytes) & 7) == 0) {
         for (size_t i = i0; i < bytes / 8; i += step)
@@ -88,7 +86,42 @@ __global__ void k_read_back(unsigned char* __restrict__ dst, const unsigned char
         for (size_t i = i0; i < bytes; i += step) dst[i] = src[i];
     }
 }
+
+// launches the reads queued since the last flush
+spgemm_status_t flush_reads(spgemm_ctx* ctx) {
+    const size_t n = ctx->rb_pending.size();
+    if (ctx->rb_launched >= n) return SPGEMM_OK;
+    ReadList l;
+    int k = 0;
+    size_t most = 0;
+    for (size_t i = ctx->rb_launched; i < n; ++i, ++k) {
+        const auto& r = ctx->rb_pending[i];
+        l.dst[k] = ctx->rb_dev + r.off;
+        l.src[k] = (const unsigned char*)r.src;
+        l.bytes[k] = r.bytes;
+        most = std::max(most, r.bytes);
+    }
+    const dim3 grid((unsigned)std::min<size_t>((most + 2047) / 2048, 256), (unsigned)k);
+    k_read_back<<<grid, 256, 0, ctx->stream>>>(l);
+    note_launch();
+    ctx->rb_launched = n;
+    SG_CUDA(ctx, cudaGetLastError());
+    return SPGEMM_OK;
+}
 }  // namespace
+
+spgemm_status_t sync_ctx(spgemm_ctx* ctx) {
+    SG_TRY(flush_reads(ctx));
+    const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+    if (e == cudaSuccess) {
+        for (const auto& r : ctx->rb_pending) std::memcpy(r.dst, ctx->rb_host + r.off, r.bytes);
+    }
+    ctx->rb_pending.clear();
+    ctx->rb_used = ctx->rb_launched = 0;
+    SG_CUDA(ctx, e);
+    SG_CUDA(ctx, cudaGetLastError());
+    return SPGEMM_OK;
+}
 
 spgemm_status_t read_back(spgemm_ctx* ctx, void* dst, const void* src, size_t bytes) {
     if (bytes == 0) return SPGEMM_OK;
@@ -117,12 +150,9 @@ spgemm_status_t read_back(spgemm_ctx* ctx, void* dst, const void* src, size_t by
             ctx->rb_cap = cap;
         }
     }
-    const int grid = (int)std::min<size_t>((bytes + 2047) / 2048, 256);
-    k_read_back<<<grid, 256, 0, ctx->stream>>>(ctx->rb_dev + off, (const unsigned char*)src, bytes);
-    note_launch();
-    SG_CUDA(ctx, cudaGetLastError());
-    ctx->rb_pending.push_back({dst, off, bytes});
+    ctx->rb_pending.push_back({dst, src, off, bytes});
     ctx->rb_used = off + bytes;
+    if (ctx->rb_pending.size() - ctx->rb_launched == RB_MAX) SG_TRY(flush_reads(ctx));
     return SPGEMM_OK;
 }
 
@@ -401,20 +431,23 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         return o;
     };
     const int64_t U1 = std::max<int64_t>(U, 1);
+    // uploaded in one copy: products, item offsets, zeroed counters (counter copies of the
+    // analysis, the scatter cursors, the slab tier's counters, numeric counts and cursors)
+    constexpr int NCTR = CTR_REP * CTR_STRIDE + NBIN + 8;
     size_t o_prods = take(sizeof(Prod) * std::max<int64_t>(np, 1));
     size_t o_base = take(8 * (np + 1));
+    size_t o_ctr = take(8 * NCTR);
+    size_t o_nctr = take(8 * 2 * NBIN);
+    const size_t up_bytes = off;
     size_t o_flops = take(8 * U1);
     size_t o_bin = take(U1);
     size_t o_iprod = take(4 * U1);
-    size_t o_ctr = take(8 * (CTR_REP * CTR_STRIDE + NBIN + 8));
     size_t o_binoff = take(8 * NBIN);
     size_t o_list = take(sizeof(int2) * U1);
     size_t o_nnz = take(8 * U1);
     size_t o_scan = take(scan_tmp_bytes(U1));
     size_t o_nbin = take(U1);
     size_t o_nlist = take(sizeof(int2) * U1);
-    size_t o_nctr = take(8 * 2 * NBIN);
-    size_t o_nbinoff = take(8 * NBIN);
     size_t o_feat = want_features ? take(32 * U1) : 0;
     size_t o_sk = want_features ? take(8 * std::max<int64_t>(amax_n, 1)) : 0;
     size_t o_skb = want_features ? take(8 * (np + 1)) : 0;
@@ -441,10 +474,14 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
     E->nbin = (uint8_t*)(base + o_nbin);
     E->nlist = (int2*)(base + o_nlist);
     E->nctr = (unsigned long long*)(base + o_nctr);
-    E->nbin_off_dev = (int64_t*)(base + o_nbinoff);
     E->numeric_bins = false;
-    SG_CUDA(ctx, cudaMemcpyAsync(dprods, E->hprods.data(), sizeof(Prod) * np, cudaMemcpyHostToDevice, st));
-    SG_CUDA(ctx, cudaMemcpyAsync(dbase, E->hitem_base.data(), 8 * (np + 1), cudaMemcpyHostToDevice, st));
+    {
+        std::vector<char> up(up_bytes, 0);
+        if (np > 0) std::memcpy(up.data() + o_prods, E->hprods.data(), sizeof(Prod) * np);
+        std::memcpy(up.data() + o_base, E->hitem_base.data(), 8 * (np + 1));
+        // from pageable memory: the call returns once the bytes are out of `up`
+        SG_CUDA(ctx, cudaMemcpyAsync(base, up.data(), up_bytes, cudaMemcpyHostToDevice, st));
+    }
     E->it.prods = dprods;
     E->it.item_base = dbase;
     E->it.nprod = np;
@@ -475,12 +512,11 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         }
         SG_CUDA(ctx, cudaMemcpyAsync(skbase, hb.data(), 8 * (np + 1), cudaMemcpyHostToDevice, st));
     }
-    // counter copies of the analysis, then the scatter cursors and the slab tier's counters
     unsigned long long* const cur = E->ctr + CTR_REP * CTR_STRIDE;
     unsigned long long* const slab_ctr = cur + NBIN;
-    SG_CUDA(ctx, cudaMemsetAsync(E->ctr, 0, 8 * (CTR_REP * CTR_STRIDE + NBIN + 8), st));
     launch_analyze(st, E->it, E->cfg, E->flops, E->bin, E->item_prod, E->ctr, E->ctr + NBIN, sketch, skbase,
-                   E->feat, E->maxlen);
+                   E->feat, E->maxlen, E->nnz_item);
+    launch_bin_scatter(st, E->it, E->bin, E->item_prod, E->ctr, CTR_REP, cur, E->bin_off_dev, E->list);
     unsigned long long hc[CTR_REP * CTR_STRIDE];
     SG_TRY(read_back(ctx, hc, E->ctr, sizeof(hc)));
     SG_TRY(sync_ctx(ctx));
@@ -494,8 +530,6 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         acc += E->bin_cnt[b];
     }
     E->flops_total = (int64_t)hc[NBIN];
-    SG_CUDA(ctx, cudaMemcpyAsync(E->bin_off_dev, E->bin_off, sizeof(int64_t) * NBIN, cudaMemcpyHostToDevice, st));
-    launch_bin_scatter(st, E->it, E->bin, E->item_prod, E->bin_off_dev, cur, E->list);
     const int64_t nd = E->bin_cnt[BIN_DENSE];
     E->dw = DenseWork();
     if (nd > 0 && E->it.max_m <= BLOCK_TIER_MAX_ROWS) {
@@ -596,7 +630,6 @@ spgemm_status_t engine_symbolic(Engine* E) {
     spgemm_ctx* ctx = E->ctx;
     cudaStream_t st = ctx->stream;
     const int64_t U = E->it.nitems;
-    SG_CUDA(ctx, cudaMemsetAsync(E->nnz_item, 0, 8 * std::max<int64_t>(U, 1), st));
     switch (E->sr) {
     case SPGEMM_PLUS_TIMES_F64: dispatch_symbolic<PT64>(E); break;
     case SPGEMM_MIN_PLUS_F32: dispatch_symbolic<MP32>(E); break;
@@ -610,16 +643,12 @@ spgemm_status_t engine_symbolic(Engine* E) {
     E->Coff = (int64_t*)E->Coff_buf->p;
     {
         PhaseTimer t(ctx, SPGEMM_PHASE_SCAN, E->sr);
-        launch_exclusive_scan(st, E->nnz_item, U, E->Coff, E->scan_tmp);
+        launch_count_scan(st, E->it, E->cfg, E->bin, E->flops, E->item_prod, E->nnz_item, E->Coff, E->scan_tmp,
+                          E->nbin, E->nctr, E->nlist);
     }
     int64_t nnz = 0;
     int err = 0;
     unsigned long long nc[NBIN];
-    {
-        PhaseTimer t(ctx, SPGEMM_PHASE_SCAN, E->sr);
-        SG_CUDA(ctx, cudaMemsetAsync(E->nctr, 0, 8 * 2 * NBIN, st));
-        launch_numeric_bins(st, E->it, E->cfg, E->bin, E->flops, E->nnz_item, E->nbin, E->nctr);
-    }
     SG_TRY(read_back(ctx, nc, E->nctr, sizeof(nc)));
     SG_TRY(read_back(ctx, &nnz, E->Coff + U, sizeof(int64_t)));
     SG_TRY(read_back(ctx, &err, E->err_dev, sizeof(int)));
@@ -642,11 +671,6 @@ spgemm_status_t engine_symbolic(Engine* E) {
         E->nbin_cnt[b] = (int64_t)nc[b];
         E->nbin_off[b] = acc;
         acc += E->nbin_cnt[b];
-    }
-    {
-        PhaseTimer t(ctx, SPGEMM_PHASE_SCAN, E->sr);
-        SG_CUDA(ctx, cudaMemcpyAsync(E->nbin_off_dev, E->nbin_off, sizeof(int64_t) * NBIN, cudaMemcpyHostToDevice, st));
-        launch_bin_scatter(st, E->it, E->nbin, E->item_prod, E->nbin_off_dev, E->nctr + NBIN, E->nlist);
     }
     E->numeric_bins = true;
     E->symbolic_done = true;

@@ -43,9 +43,9 @@ struct spgemm_ctx {
     // already queued on the copy engine (from any stream, the caller's included).
     unsigned char* rb_host = nullptr;   // cudaHostAlloc(..., cudaHostAllocMapped)
     unsigned char* rb_dev = nullptr;    // its device address
-    size_t rb_cap = 0, rb_used = 0;
-    struct Readback { void* dst; size_t off, bytes; };
-    std::vector<Readback> rb_pending;
+    size_t rb_cap = 0, rb_used = 0, rb_launched = 0;
+    struct Readback { void* dst; const void* src; size_t off, bytes; };
+    std::vector<Readback> rb_pending;   // the first rb_launched of them are on the stream already
 };
 
 // Shared ownership of an allocation (batch outputs share one buffer).
@@ -106,7 +106,6 @@ struct Engine {
     uint8_t* nbin = nullptr;
     int2* nlist = nullptr;
     unsigned long long* nctr = nullptr;   // count[NBIN], cursor[NBIN]
-    int64_t* nbin_off_dev = nullptr;
     int64_t nbin_cnt[sg::NBIN] = {0};
     int64_t nbin_off[sg::NBIN] = {0};
     bool numeric_bins = false;
@@ -165,8 +164,9 @@ size_t sr_size(spgemm_semiring_t sr);
 sg::DMat dmat_of(const spgemm_mat* M);
 spgemm_status_t check_cuda(spgemm_ctx* ctx, cudaError_t e, const char* what);
 spgemm_status_t sync_ctx(spgemm_ctx* ctx);
-// Queues a read of `bytes` at device address src into host memory dst, on the context
-// stream; dst holds the bytes after the next sync_ctx (not before).
+// Queues a read of `bytes` at device address src into host memory dst; the reads queued
+// before a sync_ctx go to the context stream together, in one launch at that sync_ctx (or
+// before), so src has to keep its bytes until then; dst holds them after it (not before).
 spgemm_status_t read_back(spgemm_ctx* ctx, void* dst, const void* src, size_t bytes);
 
 // formats.cu

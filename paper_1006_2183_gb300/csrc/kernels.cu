@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
                                                  unsigned long long* bin_count, unsigned long long* flops_total,
                                                  const uint64_t* __restrict__ sketch,
                                                  const int64_t* __restrict__ sketch_base, float* __restrict__ feat,
-                                                 int64_t* __restrict__ maxlen) {
+                                                 int64_t* __restrict__ maxlen, int64_t* __restrict__ nnz_item) {
     constexpr int GRP = 256 / LPI;   // items of this CTA
     __shared__ unsigned long long s_cnt[NBIN];
     __shared__ unsigned long long s_fl;
@@ -266,6 +266,7 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
         flops[u] = f;
         if (it.nprod == 1) item_prod[u] = 0;
         bin[u] = (uint8_t)b;
+        nnz_item[u] = 0;   // of the empty columns; the counting passes write the others
         if (maxlen) maxlen[u] = mx;
         if (feat) {
             // predictor inputs (definitions in predictor.cu)
@@ -301,7 +302,7 @@ __global__ void k_item_prod(Items it, int32_t* __restrict__ item_prod) {
 
 void launch_analyze(cudaStream_t st, const Items& it, TierCfg cfg, int64_t* flops, uint8_t* bin, int32_t* item_prod,
                     unsigned long long* bin_count, unsigned long long* flops_total, const uint64_t* sketch,
-                    const int64_t* sketch_base, float* feat, int64_t* maxlen) {
+                    const int64_t* sketch_base, float* feat, int64_t* maxlen, int64_t* nnz_item) {
     if (it.nitems == 0) return;
     if (it.nprod > 1) {
         k_item_prod<<<(unsigned)it.nprod, 256, 0, st>>>(it, item_prod);
@@ -310,15 +311,15 @@ void launch_analyze(cudaStream_t st, const Items& it, TierCfg cfg, int64_t* flop
     if (it.total_bnz < 4 * it.nitems) {   // about one B entry per item: one lane each
         int grid = (int)ceil_div64(it.nitems, 256);
         k_analyze<1><<<grid, 256, 0, st>>>(it, cfg, flops, bin, item_prod, bin_count, flops_total, sketch,
-                                           sketch_base, feat, maxlen);
+                                           sketch_base, feat, maxlen, nnz_item);
     } else if (it.total_bnz >= 32 * it.nitems) {
         int grid = (int)ceil_div64(it.nitems * 32, 256);
         k_analyze<32><<<grid, 256, 0, st>>>(it, cfg, flops, bin, item_prod, bin_count, flops_total, sketch,
-                                            sketch_base, feat, maxlen);
+                                            sketch_base, feat, maxlen, nnz_item);
     } else {
         int grid = (int)ceil_div64(it.nitems * 8, 256);
         k_analyze<8><<<grid, 256, 0, st>>>(it, cfg, flops, bin, item_prod, bin_count, flops_total, sketch,
-                                           sketch_base, feat, maxlen);
+                                           sketch_base, feat, maxlen, nnz_item);
     }
     note_launch();
 }
@@ -347,58 +348,64 @@ void launch_row_sketch(cudaStream_t st, const DMat& A, uint64_t* sketch) {
     note_launch();
 }
 
-// Numeric bins of the hash-tier items from their exact counts: the table needs
-// only 2 nnz slots, not 2 min(flops, m).  Range-tier and empty items get bin 0
-// (not listed).
-__global__ void k_numeric_bins(Items it, TierCfg cfg, const uint8_t* __restrict__ bin,
-                               const int64_t* __restrict__ flops, const int64_t* __restrict__ nnz_item,
-                               uint8_t* __restrict__ nbin, unsigned long long* __restrict__ cnt) {
-    __shared__ unsigned long long s_cnt[NBIN];
-    for (int b = threadIdx.x; b < NBIN; b += blockDim.x) s_cnt[b] = 0;
-    __syncthreads();
-    for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < it.nitems; u += (int64_t)gridDim.x * blockDim.x) {
-        const int b = bin[u];
-        int nb = 0;
-        if (b >= BIN_SORT0 && b < BIN_DENSE) nb = bin_of(flops[u], nnz_item[u], cfg.warp_max, cfg.block_max, cfg.sort_max);
-        nbin[u] = (uint8_t)nb;
-        if (nb) atomicAdd(&s_cnt[nb], 1ull);
+// Where every bin's list starts (s_off, NBIN entries) from the bins' counts, kept in `rep`
+// copies CTR_STRIDE apart.  Called by all threads of a CTA; ends with a barrier.
+__device__ __forceinline__ void bin_offsets(const unsigned long long* cnt, int rep, int64_t* s_off) {
+    if (threadIdx.x < 32) {
+        const int b = threadIdx.x;
+        long long c = 0;
+        if (b < NBIN)
+            for (int r = 0; r < rep; ++r) c += (long long)__ldcg(cnt + r * CTR_STRIDE + b);
+        const long long inc = warp_incl_scan64(c);
+        if (b < NBIN) s_off[b] = inc - c;
     }
     __syncthreads();
-    for (int b = threadIdx.x; b < NBIN; b += blockDim.x)
-        if (s_cnt[b]) atomicAdd(cnt + b, s_cnt[b]);
 }
 
-void launch_numeric_bins(cudaStream_t st, const Items& it, TierCfg cfg, const uint8_t* bin, const int64_t* flops,
-                         const int64_t* nnz_item, uint8_t* nbin, unsigned long long* cnt) {
-    if (it.nitems == 0) return;
-    const int grid = (int)std::min<int64_t>(ceil_div64(it.nitems, 256), sm_count() * 8);
-    k_numeric_bins<<<grid, 256, 0, st>>>(it, cfg, bin, flops, nnz_item, nbin, cnt);
-    note_launch();
+// One bin per thread (b <= 0: not listed): its place in the list of bin b, whose entries
+// before this CTA's come from one global addition per bin.  All threads call it.
+__device__ __forceinline__ int64_t list_place(int b, unsigned long long* cursor, const int64_t* s_off, int* s_n,
+                                              int64_t* s_base) {
+    if (threadIdx.x < NBIN) s_n[threadIdx.x] = 0;
+    __syncthreads();
+    const unsigned peers = __match_any_sync(0xffffffffu, b);
+    const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
+    int at = 0;
+    if (b > 0 && lane == leader) at = atomicAdd(&s_n[b], __popc(peers));
+    at = __shfl_sync(0xffffffffu, at, leader) + __popc(peers & ((1u << lane) - 1));
+    __syncthreads();
+    if (threadIdx.x < NBIN && threadIdx.x > 0 && s_n[threadIdx.x] > 0)
+        s_base[threadIdx.x] = s_off[threadIdx.x] +
+                              (int64_t)atomicAdd(cursor + threadIdx.x, (unsigned long long)s_n[threadIdx.x]);
+    __syncthreads();
+    return b > 0 ? s_base[b] + at : 0;
 }
 
-// Scatter of items into per-bin lists (warp-aggregated atomics).
-__global__ void k_bin_scatter(Items it, const uint8_t* __restrict__ bin, const int32_t* __restrict__ item_prod,
-                              const int64_t* __restrict__ bin_off, unsigned long long* cursor, int2* __restrict__ list) {
-    int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int b = u < it.nitems ? bin[u] : -1;
-    unsigned mask = __match_any_sync(0xffffffffu, b);
-    int lane = threadIdx.x & 31;
-    int leader = __ffs(mask) - 1;
-    unsigned long long base = 0;
-    if (b > 0 && lane == leader) base = atomicAdd(cursor + b, (unsigned long long)__popc(mask));
-    base = __shfl_sync(0xffffffffu, base, leader);
+// Scatter of items into per-bin lists, whose offsets every CTA makes from the counts (and
+// CTA 0 leaves in off_out), so that the launch waits for no host.
+__global__ void __launch_bounds__(256) k_bin_scatter(Items it, const uint8_t* __restrict__ bin,
+                                                     const int32_t* __restrict__ item_prod,
+                                                     const unsigned long long* __restrict__ cnt, int rep,
+                                                     unsigned long long* cursor, int64_t* __restrict__ off_out,
+                                                     int2* __restrict__ list) {
+    __shared__ int64_t s_off[NBIN], s_base[NBIN];
+    __shared__ int s_n[NBIN];
+    bin_offsets(cnt, rep, s_off);
+    if (blockIdx.x == 0 && threadIdx.x < NBIN) off_out[threadIdx.x] = s_off[threadIdx.x];
+    const int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int b = u < it.nitems ? bin[u] : -1;
+    const int64_t at = list_place(b, cursor, s_off, s_n, s_base);
     if (b > 0) {
-        int rank = __popc(mask & ((1u << lane) - 1));
-        int prod = item_prod[u];
-        int p = (int)(u - __ldg(it.item_base + prod));
-        list[bin_off[b] + base + rank] = make_int2(prod, p);
+        const int prod = item_prod[u];
+        list[at] = make_int2(prod, (int)(u - __ldg(it.item_base + prod)));
     }
 }
 
 void launch_bin_scatter(cudaStream_t st, const Items& it, const uint8_t* bin, const int32_t* item_prod,
-                        const int64_t* bin_off, unsigned long long* bin_cursor, int2* list) {
+                        const unsigned long long* cnt, int rep, unsigned long long* cursor, int64_t* off_out,
+                        int2* list) {
     if (it.nitems == 0) return;
-    k_bin_scatter<<<(int)ceil_div64(it.nitems, 256), 256, 0, st>>>(it, bin, item_prod, bin_off, bin_cursor, list);
+    k_bin_scatter<<<(int)ceil_div64(it.nitems, 256), 256, 0, st>>>(it, bin, item_prod, cnt, rep, cursor, off_out, list);
     note_launch();
 }
 
@@ -1216,6 +1223,25 @@ __global__ void __launch_bounds__(256) k_slab_bounds(Items it, DenseWork dw) {
     }
 }
 
+// Any zero byte in v[0, n), 16 at a time between the aligned ends, the work spread over
+// `stride` threads of which this is thread t0.  (A byte per load took 115 us for the 16 MB
+// of an R-MAT scale 20 graph.)
+__device__ __forceinline__ bool any_zero_byte(const uint8_t* __restrict__ v, int64_t n, int64_t t0, int64_t stride) {
+    int64_t head = (int64_t)((16 - ((uintptr_t)v & 15)) & 15);
+    head = head < n ? head : n;
+    const int64_t nq = (n - head) >> 4;
+    const uint4* __restrict__ q = reinterpret_cast<const uint4*>(v + head);
+    bool f = false;
+    auto zero = [](uint32_t x) { return ((x - 0x01010101u) & ~x & 0x80808080u) != 0u; };
+    for (int64_t i = t0; i < nq; i += stride) {
+        const uint4 x = __ldg(q + i);
+        f |= zero(x.x) || zero(x.y) || zero(x.z) || zero(x.w);
+    }
+    for (int64_t i = t0; i < head; i += stride) f |= __ldg(v + i) == 0;
+    for (int64_t i = head + 16 * nq + t0; i < n; i += stride) f |= __ldg(v + i) == 0;
+    return f;
+}
+
 // flag = 1 when some stored value of an operand is false (boolean semiring): then
 // the numeric pass must evaluate the products; else every output value is true.
 __global__ void k_false_values(Items it, int* flag) {
@@ -1233,7 +1259,7 @@ __global__ void k_false_values(Items it, int* flag) {
                     for (int64_t i = __ldg(M.cp + c); i < __ldg(M.ce + c); ++i) f |= __ldg(v + i) == 0;
             } else {
                 const int64_t s = __ldg(M.cp), e = __ldg(M.cp + M.nzc);
-                for (int64_t i = s + t0; i < e; i += stride) f |= __ldg(v + i) == 0;
+                f = any_zero_byte(v + s, e - s, t0, stride);
             }
             if (f) *flag = 1;
         }
@@ -1241,15 +1267,12 @@ __global__ void k_false_values(Items it, int* flag) {
 }
 
 __global__ void k_any_false(const uint8_t* __restrict__ v, int64_t n, int* flag) {
-    bool f = false;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        f |= __ldg(v + i) == 0;
-    if (f) *flag = 1;
+    if (any_zero_byte(v, n, (int64_t)blockIdx.x * blockDim.x + threadIdx.x, (int64_t)gridDim.x * blockDim.x)) *flag = 1;
 }
 
 void launch_any_false(cudaStream_t st, const void* vals, int64_t n, int* flag) {
     if (!vals || n <= 0) return;
-    k_any_false<<<(int)std::min<int64_t>(ceil_div64(n, 256), sm_count() * 8), 256, 0, st>>>((const uint8_t*)vals, n,
+    k_any_false<<<(int)std::min<int64_t>(ceil_div64(n, 16 * 256), sm_count() * 8), 256, 0, st>>>((const uint8_t*)vals, n,
                                                                                           flag);
     note_launch();
 }
@@ -1257,7 +1280,7 @@ void launch_any_false(cudaStream_t st, const void* vals, int64_t n, int* flag) {
 void launch_false_values(cudaStream_t st, const Items& it, int* flag) {
     if (it.nprod <= 0) return;
     const int gy = (int)std::min<int64_t>(it.nprod, 65535);
-    const int gx = std::max(1, std::min(256, 4096 / gy));
+    const int gx = std::max(1, std::min(sm_count() * 4, 4096 / gy));
     k_false_values<<<dim3(gx, gy), 256, 0, st>>>(it, flag);
     note_launch();
 }
@@ -2014,6 +2037,9 @@ void launch_tier_stats(cudaStream_t st, const Items& it, const uint8_t* bin, con
 constexpr int SCAN_BLOCK = 1024;
 constexpr int SCAN_ITEMS = 4;
 constexpr int SCAN_TILE = SCAN_BLOCK * SCAN_ITEMS;
+// up to this many tiles every CTA of the second pass adds the earlier tiles' sums itself
+// (two 8-byte loads per thread at most); more tiles take a launch of their own for that
+constexpr int64_t SCAN_SELF_TILES = 2 * SCAN_BLOCK;
 
 __device__ __forceinline__ long long block_excl_scan64(long long v, long long* ws, long long& total) {
     long long x = warp_incl_scan64(v);
@@ -2032,17 +2058,67 @@ __device__ __forceinline__ long long block_excl_scan64(long long v, long long* w
     return x + add - v;
 }
 
+// The end of the counting pass was five launches, two uploads and a memset: three scan
+// launches, the bins from the counts (every thread adding to the same shared counters, 15 us
+// for 4,096 columns), their offsets through the host, and the lists.  It is one launch up to
+// 4,096 columns (11 us) and two up to 8 million: ER 4096^2 flat, a whole call, 137 -> 95 us.
+// What the scan of the exact counts does besides: the numeric bin of every item (hash tables
+// need only 2 nnz slots, not 2 min(flops, m); slab-tier and empty items get bin 0, not
+// listed), the bins' counts, and their lists.
+struct CountBins {
+    Items it;
+    TierCfg cfg;
+    const uint8_t* bin;
+    const int64_t* flops;
+    const int32_t* item_prod;
+    uint8_t* nbin;
+    unsigned long long* cnt;      // NBIN counts (zeroed by the caller)
+    unsigned long long* cursor;   // NBIN cursors (zeroed by the caller)
+    int2* list;
+};
+
+__device__ __forceinline__ int numeric_bin(const CountBins& nb, int64_t u, int64_t nnz) {
+    const int b = nb.bin[u];
+    if (b < BIN_SORT0 || b >= BIN_DENSE) return 0;
+    return bin_of(nb.flops[u], nnz, nb.cfg.warp_max, nb.cfg.block_max, nb.cfg.sort_max);
+}
+
+// adds one thread's bin (b <= 0: none) to the CTA's counts; whole warps call it
+__device__ __forceinline__ void count_bin(int b, int* s_n) {
+    const unsigned peers = __match_any_sync(0xffffffffu, b);
+    if (b > 0 && (int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&s_n[b], __popc(peers));
+}
+
+// First pass: the sum of every tile, and with BINS the numeric bins and their counts.
+template <bool BINS>
 __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_reduce(const int64_t* __restrict__ in, int64_t n,
-                                                             long long* __restrict__ sums) {
+                                                             long long* __restrict__ sums, CountBins nb) {
     __shared__ long long ws[32];
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
+    __shared__ int s_n[NBIN];
+    if constexpr (BINS) {
+        if (threadIdx.x < NBIN) s_n[threadIdx.x] = 0;
+        __syncthreads();
+    }
+    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     long long s = 0;
 #pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i)
-        if (base + i < n) s += in[base + i];
+    for (int i = 0; i < SCAN_ITEMS; ++i) {
+        const int64_t u = base + i * SCAN_BLOCK + threadIdx.x;
+        const long long v = u < n ? in[u] : 0;
+        s += v;
+        if constexpr (BINS) {
+            const int b = u < n ? numeric_bin(nb, u, v) : 0;
+            if (u < n) nb.nbin[u] = (uint8_t)b;
+            count_bin(b, s_n);
+        }
+    }
     long long total;
     block_excl_scan64(s, ws, total);
     if (threadIdx.x == 0) sums[blockIdx.x] = total;
+    if constexpr (BINS) {
+        if (threadIdx.x < NBIN && s_n[threadIdx.x])
+            atomicAdd(nb.cnt + threadIdx.x, (unsigned long long)s_n[threadIdx.x]);
+    }
 }
 
 __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_sums(long long* sums, int64_t nb) {
@@ -2058,11 +2134,25 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_sums(long long* sums, int64
     }
 }
 
+// Second pass: out[u + 1] for the CTA's tile, after the earlier tiles (`summed`: sums already
+// holds their exclusive scan).  With BINS also the numeric lists; a single tile makes its own
+// bins and counts first, so that the whole step is this one launch.
+template <bool BINS>
 __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_apply(const int64_t* __restrict__ in, int64_t n,
-                                                            const long long* __restrict__ sums,
-                                                            int64_t* __restrict__ out) {
+                                                            const long long* __restrict__ sums, bool summed,
+                                                            int64_t* __restrict__ out, CountBins nb) {
     __shared__ long long ws[32];
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
+    __shared__ int64_t s_off[NBIN], s_base[NBIN];
+    __shared__ int s_n[NBIN];
+    long long before = 0;
+    if (summed) {
+        before = sums[blockIdx.x];
+    } else if (blockIdx.x > 0) {
+        long long s = 0;
+        for (int64_t t = threadIdx.x; t < blockIdx.x; t += SCAN_BLOCK) s += sums[t];
+        block_excl_scan64(s, ws, before);
+    }
+    const int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
     long long v[SCAN_ITEMS];
     long long s = 0;
 #pragma unroll
@@ -2071,28 +2161,79 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_apply(const int64_t* __rest
         s += v[i];
     }
     long long total;
-    long long ex = block_excl_scan64(s, ws, total) + sums[blockIdx.x];
+    long long ex = block_excl_scan64(s, ws, total) + before;
     if (blockIdx.x == 0 && threadIdx.x == 0) out[0] = 0;
 #pragma unroll
     for (int i = 0; i < SCAN_ITEMS; ++i) {
         ex += v[i];
         if (base + i < n) out[base + i + 1] = ex;
     }
+    if constexpr (BINS) {
+        int b[SCAN_ITEMS];
+        if (gridDim.x == 1) {
+            if (threadIdx.x < NBIN) s_n[threadIdx.x] = 0;
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < SCAN_ITEMS; ++i) {
+                b[i] = base + i < n ? numeric_bin(nb, base + i, v[i]) : 0;
+                if (base + i < n) nb.nbin[base + i] = (uint8_t)b[i];
+                count_bin(b[i], s_n);
+            }
+            __syncthreads();
+            if (threadIdx.x < NBIN) nb.cnt[threadIdx.x] = (unsigned long long)s_n[threadIdx.x];
+            __threadfence();
+            __syncthreads();
+        } else {
+#pragma unroll
+            for (int i = 0; i < SCAN_ITEMS; ++i) b[i] = base + i < n ? nb.nbin[base + i] : 0;
+        }
+        bin_offsets(nb.cnt, 1, s_off);
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; ++i) {
+            const int64_t at = list_place(b[i], nb.cursor, s_off, s_n, s_base);
+            if (b[i] > 0) {
+                const int prod = nb.item_prod[base + i];
+                nb.list[at] = make_int2(prod, (int)(base + i - __ldg(nb.it.item_base + prod)));
+            }
+        }
+    }
 }
 
 size_t scan_tmp_bytes(int64_t n) { return (size_t)(ceil_div64(std::max<int64_t>(n, 1), SCAN_TILE) + 1) * 8; }
+
+template <bool BINS>
+static void run_scan(cudaStream_t st, const int64_t* in, int64_t n, int64_t* out, void* tmp, const CountBins& nb) {
+    const int64_t nt = ceil_div64(n, SCAN_TILE);
+    long long* sums = reinterpret_cast<long long*>(tmp);
+    const bool summed = nt > SCAN_SELF_TILES;
+    if (nt > 1) {
+        k_scan_reduce<BINS><<<(int)nt, SCAN_BLOCK, 0, st>>>(in, n, sums, nb);
+        note_launch();
+    }
+    if (summed) {
+        k_scan_sums<<<1, SCAN_BLOCK, 0, st>>>(sums, nt);
+        note_launch();
+    }
+    k_scan_apply<BINS><<<(int)nt, SCAN_BLOCK, 0, st>>>(in, n, sums, summed, out, nb);
+    note_launch();
+}
 
 void launch_exclusive_scan(cudaStream_t st, const int64_t* in, int64_t n, int64_t* out, void* tmp) {
     if (n <= 0) {
         cudaMemsetAsync(out, 0, sizeof(int64_t), st);
         return;
     }
-    int64_t nb = ceil_div64(n, SCAN_TILE);
-    long long* sums = reinterpret_cast<long long*>(tmp);
-    k_scan_reduce<<<(int)nb, SCAN_BLOCK, 0, st>>>(in, n, sums);
-    k_scan_sums<<<1, SCAN_BLOCK, 0, st>>>(sums, nb);
-    k_scan_apply<<<(int)nb, SCAN_BLOCK, 0, st>>>(in, n, sums, out);
-    note_launch(3);
+    run_scan<false>(st, in, n, out, tmp, CountBins());
+}
+
+void launch_count_scan(cudaStream_t st, const Items& it, TierCfg cfg, const uint8_t* bin, const int64_t* flops,
+                       const int32_t* item_prod, const int64_t* nnz_item, int64_t* out, void* tmp, uint8_t* nbin,
+                       unsigned long long* cnt, int2* list) {
+    if (it.nitems <= 0) {
+        cudaMemsetAsync(out, 0, sizeof(int64_t), st);
+        return;
+    }
+    run_scan<true>(st, nnz_item, it.nitems, out, tmp, CountBins{it, cfg, bin, flops, item_prod, nbin, cnt, cnt + NBIN, list});
 }
 
 }  // namespace sg

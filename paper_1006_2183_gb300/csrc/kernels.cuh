@@ -149,20 +149,25 @@ constexpr int64_t BM_MAX_ROWS = 262144;
 constexpr int64_t BM_WARP_MAX_ROWS = 32768;
 constexpr int BM_WARP_MIN_TBL = 256;   // smaller tables hold too few rows to prefer the bitmap
 
-// flops and bin per item, product id per item, bin counts and total flops (CTR_REP partial
+// flops and bin per item, product id per item, nnz_item = 0, bin counts and total flops (CTR_REP partial
 // copies each, CTR_STRIDE entries apart: bin_count[r * CTR_STRIDE + b]).
 // With feat != nullptr also the 8 predictor inputs per item; `sketch` holds the
 // per-column row sketches of the A operands concatenated, product i's starting
 // at sketch_base[i].
 void launch_analyze(cudaStream_t st, const Items& it, TierCfg cfg, int64_t* flops, uint8_t* bin, int32_t* item_prod,
                     unsigned long long* bin_count, unsigned long long* flops_total, const uint64_t* sketch,
-                    const int64_t* sketch_base, float* feat, int64_t* maxlen = nullptr);
+                    const int64_t* sketch_base, float* feat, int64_t* maxlen, int64_t* nnz_item);
 void launch_row_sketch(cudaStream_t st, const DMat& A, uint64_t* sketch);
+// per-bin lists of the items; cnt holds the bins' counts in `rep` copies CTR_STRIDE apart,
+// cursor NBIN zeros; off_out gets where every list starts
 void launch_bin_scatter(cudaStream_t st, const Items& it, const uint8_t* bin, const int32_t* item_prod,
-                        const int64_t* bin_off, unsigned long long* bin_cursor, int2* list);
-// hash-tier bins from exact counts (after the symbolic pass); cnt[NBIN] accumulates
-void launch_numeric_bins(cudaStream_t st, const Items& it, TierCfg cfg, const uint8_t* bin, const int64_t* flops,
-                         const int64_t* nnz_item, uint8_t* nbin, unsigned long long* cnt);
+                        const unsigned long long* cnt, int rep, unsigned long long* cursor, int64_t* off_out,
+                        int2* list);
+// out = exclusive scan of the exact counts nnz_item (out[nitems] the total), the items' numeric
+// bins nbin, the bins' counts cnt[NBIN] and lists; cnt[0, 2 NBIN) is zero before
+void launch_count_scan(cudaStream_t st, const Items& it, TierCfg cfg, const uint8_t* bin, const int64_t* flops,
+                       const int32_t* item_prod, const int64_t* nnz_item, int64_t* out, void* tmp, uint8_t* nbin,
+                       unsigned long long* cnt, int2* list);
 // slabs of the long columns (position d in the dense list, slab q); P_d slabs of at
 // most RB rows each; *store_bound accumulates the entries their row sets can need
 void launch_dense_items(cudaStream_t st, const Items& it, const int2* dense_list, int64_t ndense,
