@@ -237,6 +237,7 @@ spgemm_status_t spgemm_ctx_destroy(spgemm_ctx_t ctx) {
     ctx_free(ctx, ctx->adam_v);
     ctx_free(ctx, ctx->grad);
     cudaStreamSynchronize(ctx->stream);
+    ctx->lanes.destroy();
     if (ctx->rb_host) cudaFreeHost(ctx->rb_host);
     delete ctx;
     return SPGEMM_OK;
@@ -606,22 +607,41 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
     return SPGEMM_OK;
 }
 
+// Timed, the hash and sort tiers and the long columns run one after the other, each under
+// its phase; otherwise all launches of the pass share its lanes, the longest first.
 template <class SR>
 static void dispatch_symbolic(Engine* E) {
+    spgemm_ctx* ctx = E->ctx;
+    auto launch = [&](const Lanes& l, int which) {
+        launch_symbolic<SR>(l, E->it, E->cfg, E->list, E->bin_off, E->bin_cnt, E->dw, E->nnz_item, which);
+    };
+    if (!ctx->timing) {
+        launch(Lanes(ctx->stream, pass_lanes(ctx, E->bin_cnt, E->dw.ndense)), 3);
+        return;
+    }
     for (int which = 1; which <= 2; ++which) {
-        PhaseTimer t(E->ctx, which == 1 ? SPGEMM_PHASE_SYMBOLIC_HASH : SPGEMM_PHASE_SYMBOLIC_DENSE, E->sr);
-        launch_symbolic<SR>(E->ctx->stream, E->it, E->cfg, E->list, E->bin_off, E->bin_cnt, E->dw, E->nnz_item,
-                            which);
+        PhaseTimer t(ctx, which == 1 ? SPGEMM_PHASE_SYMBOLIC_HASH : SPGEMM_PHASE_SYMBOLIC_DENSE, E->sr);
+        launch(Lanes(ctx->stream), which);
     }
 }
 
 template <class SR>
 static void dispatch_numeric(Engine* E, int32_t* Cir, void* Cv) {
-    for (int which = 1; which <= 2; ++which) {
-        PhaseTimer t(E->ctx, which == 1 ? SPGEMM_PHASE_NUMERIC_HASH : SPGEMM_PHASE_NUMERIC_DENSE, E->sr);
+    spgemm_ctx* ctx = E->ctx;
+    auto launch = [&](const Lanes& l, int which) {
         const bool nb = which == 1 && E->numeric_bins;
-        launch_numeric<SR>(E->ctx->stream, E->it, E->cfg, nb ? E->nlist : E->list, nb ? E->nbin_off : E->bin_off,
+        launch_numeric<SR>(l, E->it, E->cfg, nb ? E->nlist : E->list, nb ? E->nbin_off : E->bin_off,
                            nb ? E->nbin_cnt : E->bin_cnt, E->dw, E->Coff, Cir, (typename SR::T*)Cv, which);
+    };
+    if (!ctx->timing) {
+        Lanes l(ctx->stream, pass_lanes(ctx, E->numeric_bins ? E->nbin_cnt : E->bin_cnt, E->dw.ndense));
+        launch(l, 2);
+        launch(l, 1);
+        return;
+    }
+    for (int which = 1; which <= 2; ++which) {
+        PhaseTimer t(ctx, which == 1 ? SPGEMM_PHASE_NUMERIC_HASH : SPGEMM_PHASE_NUMERIC_DENSE, E->sr);
+        launch(Lanes(ctx->stream), which);
     }
 }
 

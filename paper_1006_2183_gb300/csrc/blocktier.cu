@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 4 : 1) k_block_tier(Item
 }
 
 template <class SR, int GS, int BLOCK>
-void run_bt(cudaStream_t st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item, const int64_t* Coff,
+void run_bt(const Lanes& st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item, const int64_t* Coff,
             int32_t* Cir, typename SR::T* Cv, const int* vals_zero) {
     if (count <= 0) return;
     constexpr int NG = BLOCK / GS;
@@ -339,14 +339,14 @@ void run_bt(cudaStream_t st, const Items& it, const int2* list, int64_t count, i
         per_sm = 1;
     }
     const int grid = (int)std::min<int64_t>(ceil_div64(count, NG), (int64_t)per_sm * sm_count());
-    kern<<<grid, BLOCK, smem, st>>>(it, list, count, nnz_item, Coff, Cir, Cv, vals_zero);
+    kern<<<grid, BLOCK, smem, st.next()>>>(it, list, count, nnz_item, Coff, Cir, Cv, vals_zero);
     note_launch();
 }
 
 }  // namespace
 
 template <class SR>
-void launch_block_tier(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+void launch_block_tier(const Lanes& st, const Items& it, const int2* list, const int64_t* bin_off,
                        const int64_t* bin_cnt, const DenseWork& dw, int64_t* nnz_item, const int64_t* Coff,
                        int32_t* Cir, typename SR::T* Cv, int which) {
     if (which & 1) {
@@ -380,7 +380,7 @@ void launch_block_tier(cudaStream_t st, const Items& it, const int2* list, const
 }
 
 #define SG_INST(SR)                                                                                               \
-    template void launch_block_tier<SR>(cudaStream_t, const Items&, const int2*, const int64_t*, const int64_t*, \
+    template void launch_block_tier<SR>(const Lanes&, const Items&, const int2*, const int64_t*, const int64_t*, \
                                         const DenseWork&, int64_t*, const int64_t*, int32_t*, typename SR::T*, int);
 SG_INST(PT64)
 SG_INST(MP32)

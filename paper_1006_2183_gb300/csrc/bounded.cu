@@ -38,7 +38,16 @@ __global__ void k_col_ends(const int64_t* __restrict__ start, const int64_t* __r
 
 template <class SR>
 void numeric_launches(Engine* E, const int64_t* cap_off, int32_t* rows, void* vals) {
-    cudaStream_t st = E->ctx->stream;
+    spgemm_ctx* ctx = E->ctx;
+    if (!ctx->timing) {   // all launches share the lanes, the longest first
+        Lanes l(ctx->stream, pass_lanes(ctx, E->bin_cnt, E->dw.ndense));
+        launch_numeric<SR>(l, E->it, E->cfg, E->list, E->bin_off, E->bin_cnt, E->dw, cap_off, rows,
+                           (typename SR::T*)vals, 2);
+        launch_numeric_predicted<SR>(l, E->it, E->list, E->bin_off, E->bin_cnt, E->dw, cap_off, E->nnz_item, rows,
+                                     (typename SR::T*)vals);
+        return;
+    }
+    cudaStream_t st = ctx->stream;
     {
         PhaseTimer t(E->ctx, SPGEMM_PHASE_NUMERIC_HASH, E->sr);
         launch_numeric_predicted<SR>(st, E->it, E->list, E->bin_off, E->bin_cnt, E->dw, cap_off, E->nnz_item, rows,

@@ -34,6 +34,7 @@ struct spgemm_ctx {
     // boolean semiring, set by a call that already knows it for every product it runs
     // (SUMMA checks its two operands once): -1 unknown, 0 no stored false value, 1 some
     int bool_hint = -1;
+    sg::LanePool lanes;                  // side streams of passes of several launches
     // statistics of the last SUMMA call
     std::vector<int64_t> summa_stage_flops;
     int64_t summa_nonempty = 0;
@@ -195,6 +196,13 @@ spgemm_status_t engine_numeric_bounded(Engine* E, std::shared_ptr<DevBuf>* rbuf,
                                        const int64_t** col_end);
 // esc.cu: all products of E by expand-sort-compress (local rows); sets Coff and nnz_total
 spgemm_status_t engine_esc(Engine* E, std::shared_ptr<DevBuf>* rbuf, std::shared_ptr<DevBuf>* vbuf);
+// The lanes of a pass over the lists counted in cnt[NBIN] and the ndense long columns: the
+// context's side streams where it has more than one launch.
+inline sg::LanePool* pass_lanes(spgemm_ctx* ctx, const int64_t* cnt, int64_t ndense) {
+    int n = ndense > 0;
+    for (int b = sg::BIN_SORT0; b < sg::BIN_DENSE; ++b) n += cnt[b] > 0;
+    return n > 1 ? &ctx->lanes : nullptr;
+}
 // output arrays sized by the engine's nnz_total, values of the semiring width
 spgemm_status_t engine_alloc_out(Engine* E, std::shared_ptr<DevBuf>* rbuf, std::shared_ptr<DevBuf>* vbuf);
 sg::DMat csc_view(int64_t m, int64_t n, int64_t nnz, const int64_t* cp, const int32_t* ir, const void* num);

@@ -42,6 +42,58 @@ int sm_count() {
     return n;
 }
 
+bool LanePool::init() {
+    if (ready || failed) return ready;
+    failed = cudaEventCreateWithFlags(&start, cudaEventDisableTiming) != cudaSuccess;
+    for (int i = 0; i < NSIDE && !failed; ++i)
+        failed = cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking) != cudaSuccess ||
+                 cudaEventCreateWithFlags(&done[i], cudaEventDisableTiming) != cudaSuccess;
+    if (failed) {
+        cudaGetLastError();   // passes then stay on one stream
+        destroy();
+        failed = true;
+    }
+    ready = !failed;
+    return ready;
+}
+
+void LanePool::destroy() {
+    if (start) cudaEventDestroy(start);
+    for (int i = 0; i < NSIDE; ++i) {
+        if (done[i]) cudaEventDestroy(done[i]);
+        if (side[i]) cudaStreamDestroy(side[i]);
+        done[i] = nullptr;
+        side[i] = nullptr;
+    }
+    start = nullptr;
+    ready = failed = false;
+}
+
+Lanes::Lanes(cudaStream_t main, LanePool* pool) : main_(main) {
+    if (pool && pool->init() && cudaEventRecord(pool->start, main) == cudaSuccess) pool_ = pool;
+}
+
+cudaStream_t Lanes::next() const {
+    const int t = turn_++ % (LanePool::NSIDE + 1);
+    if (!pool_ || t == 0) return main_;
+    const int i = t - 1;
+    if (!used_[i]) {
+        if (cudaStreamWaitEvent(pool_->side[i], pool_->start, 0) != cudaSuccess) return main_;
+        used_[i] = true;
+    }
+    return pool_->side[i];
+}
+
+Lanes::~Lanes() {
+    for (int i = 0; i < LanePool::NSIDE; ++i)
+        if (used_[i]) {
+            // should the join fail, the host waits instead: later work must not start early
+            if (cudaEventRecord(pool_->done[i], pool_->side[i]) != cudaSuccess ||
+                cudaStreamWaitEvent(main_, pool_->done[i], 0) != cudaSuccess)
+                cudaStreamSynchronize(pool_->side[i]);
+        }
+}
+
 // Raises a kernel's dynamic shared-memory limit on the current device to at least
 // `bytes`; never lowers it (the limit belongs to the kernel, whichever launcher
 // asks).  A refused request is not remembered, so the launch reports the error.
@@ -768,7 +820,7 @@ __global__ void __launch_bounds__(BLOCK, hash_min_blocks(BLOCK, TBL)) k_hash(Ite
 }
 
 template <class SR, int GS, int TBL, bool NUM, int BLOCK>
-static void run_hash(cudaStream_t st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item,
+static void run_hash(const Lanes& st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item,
                      const int64_t* Coff, int32_t* Cir, typename SR::T* Cv) {
     if (count <= 0) return;
     using L = HashLayout<SR, GS, TBL, NUM>;
@@ -782,7 +834,7 @@ static void run_hash(cudaStream_t st, const Items& it, const int2* list, int64_t
     smem_at_least((const void*)kern, smem);
     int64_t want = ceil_div64(count, NG);
     int grid = (int)std::min<int64_t>(want, sm_count() * 32);
-    kern<<<grid, BLOCK, smem, st>>>(it, list, count, nnz_item, Coff, Cir, Cv, bm_words);
+    kern<<<grid, BLOCK, smem, st.next()>>>(it, list, count, nnz_item, Coff, Cir, Cv, bm_words);
     note_launch();
 }
 
@@ -920,7 +972,7 @@ __global__ void __launch_bounds__(BLOCK, 2048 / BLOCK) k_bitcount(Items it, cons
 }
 
 template <int GS, int BLOCK>
-static void run_bitcount(cudaStream_t st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item) {
+static void run_bitcount(const Lanes& st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item) {
     if (count <= 0) return;
     constexpr int NG = BLOCK / GS;
     constexpr size_t GROUP = bitcount_group_bytes<GS>();
@@ -929,7 +981,7 @@ static void run_bitcount(cudaStream_t st, const Items& it, const int2* list, int
     auto kern = k_bitcount<GS, BLOCK>;
     smem_at_least((const void*)kern, smem);
     const int grid = (int)std::min<int64_t>(ceil_div64(count, NG), sm_count() * 32);
-    kern<<<grid, BLOCK, smem, st>>>(it, list, count, nnz_item, bm_words);
+    kern<<<grid, BLOCK, smem, st.next()>>>(it, list, count, nnz_item, bm_words);
     note_launch();
 }
 
@@ -1002,11 +1054,11 @@ __global__ void __launch_bounds__(256) k_tiny(Items it, const int2* __restrict__
 }
 
 template <class SR, bool NUM>
-static void run_tiny(cudaStream_t st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item,
+static void run_tiny(const Lanes& st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item,
                      const int64_t* Coff, int32_t* Cir, typename SR::T* Cv) {
     if (count <= 0) return;
     const int grid = (int)std::min<int64_t>(ceil_div64(count, 256), sm_count() * 16);
-    k_tiny<SR, NUM><<<grid, 256, 0, st>>>(it, list, count, nnz_item, Coff, Cir, Cv);
+    k_tiny<SR, NUM><<<grid, 256, 0, st.next()>>>(it, list, count, nnz_item, Coff, Cir, Cv);
     note_launch();
 }
 
@@ -1016,7 +1068,7 @@ static bool block_mode(const Items& it) { return it.max_m > 0 && it.max_m <= BLO
 // Columns of few products, counting or numeric: the sort tier, or, where not even 16
 // products fit its keys (2^28 rows and more), a thread per column of at most 16.
 template <class SR, bool NUM>
-static void run_short(cudaStream_t st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
+static void run_short(const Lanes& st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
                       int64_t* nnz_item, const int64_t* Coff, int32_t* Cir, typename SR::T* Cv, const int* vals_zero) {
     if (sort_max_products(it.max_m) == 0)
         run_tiny<SR, NUM>(st, it, list + off[BIN_SORT0], cnt[BIN_SORT0], nnz_item, Coff, Cir, Cv);
@@ -1025,7 +1077,7 @@ static void run_short(cudaStream_t st, const Items& it, const int2* list, const 
 }
 
 template <class SR, bool NUM>
-static void run_hash_bins(cudaStream_t st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
+static void run_hash_bins(const Lanes& st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
                           int64_t* nnz_item, const int64_t* Coff, int32_t* Cir, typename SR::T* Cv,
                           const int* vals_zero = nullptr) {
     constexpr int W0 = BIN_WARP0, B0 = BIN_BLK0;
@@ -1849,9 +1901,10 @@ static int resident_grid(const void* fn, int block, size_t smem) {
 }
 
 template <class SR>
-static void run_slabs(cudaStream_t st, const Items& it, const DenseWork& dw, bool numeric, const int64_t* Coff,
+static void run_slabs(const Lanes& lanes, const Items& it, const DenseWork& dw, bool numeric, const int64_t* Coff,
                       int32_t* Cir, typename SR::T* Cv) {
     if (dw.ndense <= 0) return;
+    const cudaStream_t st = lanes.next();
     const int64_t nslab_max = dw.nslabs > 0 ? dw.nslabs : dw.ndense * MAX_PARTS;
     if (!numeric) {
         k_slab_bounds<<<(int)std::min<int64_t>(nslab_max, sm_count() * 8), 256, 0, st>>>(it, dw);
@@ -1872,7 +1925,7 @@ static void run_slabs(cudaStream_t st, const Items& it, const DenseWork& dw, boo
 }
 
 template <class SR>
-void launch_numeric_predicted(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+void launch_numeric_predicted(const Lanes& st, const Items& it, const int2* list, const int64_t* bin_off,
                               const int64_t* bin_cnt, const DenseWork& dw, const int64_t* cap_off, int64_t* nnz_item,
                               int32_t* Cir, typename SR::T* Cv) {
     if (block_mode(it)) {
@@ -1884,18 +1937,18 @@ void launch_numeric_predicted(cudaStream_t st, const Items& it, const int2* list
 }
 
 template <class SR>
-void launch_symbolic(cudaStream_t st, const Items& it, TierCfg cfg, const int2* list, const int64_t* bin_off,
+void launch_symbolic(const Lanes& st, const Items& it, TierCfg cfg, const int2* list, const int64_t* bin_off,
                      const int64_t* bin_cnt, const DenseWork& dw, int64_t* nnz_item, int which) {
     (void)cfg;
-    if (which & 1) run_hash_bins<SR, false>(st, it, list, bin_off, bin_cnt, nnz_item, nullptr, nullptr, nullptr);
-    if (which & 2) {
+    if (which & 2) {   // the longest launches first
         if (dw.dcol) run_bitcount<256, 256>(st, it, dw.dlist, dw.ndense, nnz_item);   // rows fit the bitmap
         else run_slabs<SR>(st, it, dw, false, nullptr, nullptr, nullptr);
     }
+    if (which & 1) run_hash_bins<SR, false>(st, it, list, bin_off, bin_cnt, nnz_item, nullptr, nullptr, nullptr);
 }
 
 template <class SR>
-void launch_numeric(cudaStream_t st, const Items& it, TierCfg cfg, const int2* list, const int64_t* bin_off,
+void launch_numeric(const Lanes& st, const Items& it, TierCfg cfg, const int2* list, const int64_t* bin_off,
                     const int64_t* bin_cnt, const DenseWork& dw, const int64_t* Coff, int32_t* Cir,
                     typename SR::T* Cv, int which) {
     (void)cfg;
@@ -1909,12 +1962,12 @@ void launch_numeric(cudaStream_t st, const Items& it, TierCfg cfg, const int2* l
 }
 
 #define SG_INST(SR)                                                                                              \
-    template void launch_symbolic<SR>(cudaStream_t, const Items&, TierCfg, const int2*, const int64_t*,          \
+    template void launch_symbolic<SR>(const Lanes&, const Items&, TierCfg, const int2*, const int64_t*,          \
                                       const int64_t*, const DenseWork&, int64_t*, int);                          \
-    template void launch_numeric<SR>(cudaStream_t, const Items&, TierCfg, const int2*, const int64_t*,           \
+    template void launch_numeric<SR>(const Lanes&, const Items&, TierCfg, const int2*, const int64_t*,           \
                                      const int64_t*, const DenseWork&, const int64_t*, int32_t*, typename SR::T*, \
                                      int);                                                                       \
-    template void launch_numeric_predicted<SR>(cudaStream_t, const Items&, const int2*, const int64_t*,          \
+    template void launch_numeric_predicted<SR>(const Lanes&, const Items&, const int2*, const int64_t*,          \
                                                const int64_t*, const DenseWork&, const int64_t*, int64_t*, int32_t*, \
                                                typename SR::T*);
 SG_INST(PT64)

@@ -149,6 +149,41 @@ constexpr int64_t BM_MAX_ROWS = 262144;
 constexpr int64_t BM_WARP_MAX_ROWS = 32768;
 constexpr int BM_WARP_MIN_TBL = 256;   // smaller tables hold too few rows to prefer the bitmap
 
+// Side streams and events of a context (created at its first pass of several launches).
+struct LanePool {
+    static constexpr int NSIDE = 3;
+    cudaStream_t side[NSIDE] = {nullptr};
+    cudaEvent_t start = nullptr, done[NSIDE] = {nullptr};
+    bool ready = false, failed = false;
+    bool init();
+    void destroy();
+};
+
+// The streams that the launches of one pass go to.  The tiers of a pass work on columns of
+// their own, so their launches may overlap: they take turns on the context's stream and the
+// pool's side streams, which start after everything queued on the context's stream before
+// this object and are joined into it when the object goes (a stream capture of the
+// context's stream captures the fork and the join with it).  From a plain stream: one lane.
+// A pass has up to 16 launches whose last CTAs leave most of the chip idle, 10 to 25 us each
+// even for a handful of columns.  Whole calls, one lane against four: BFS step 343 -> 276 us,
+// restriction products 2057 -> 1572 us, 20 int64 pairs 1830 -> 1524 us, R-MAT 18 SUMMA FP64
+// 26.2 -> 24.7 ms.  The fork and the join cost about 8 us, so a pass of one launch has none.
+class Lanes {
+  public:
+    Lanes(cudaStream_t main) : main_(main) {}
+    Lanes(cudaStream_t main, LanePool* pool);   // pool null or unusable: one lane
+    ~Lanes();
+    Lanes(const Lanes&) = delete;
+    Lanes& operator=(const Lanes&) = delete;
+    cudaStream_t next() const;
+
+  private:
+    cudaStream_t main_;
+    LanePool* pool_ = nullptr;
+    mutable int turn_ = 0;
+    mutable bool used_[LanePool::NSIDE] = {false};
+};
+
 // flops and bin per item, product id per item, nnz_item = 0, bin counts and total flops (CTR_REP partial
 // copies each, CTR_STRIDE entries apart: bin_count[r * CTR_STRIDE + b]).
 // With feat != nullptr also the 8 predictor inputs per item; `sketch` holds the
@@ -181,33 +216,33 @@ void launch_any_false(cudaStream_t st, const void* vals, int64_t n, int* flag);
 
 // which: 1 = hash-table tiers, 2 = long columns (slab tier, or the block tier in block mode), 3 = both
 template <class SR>
-void launch_symbolic(cudaStream_t st, const Items& it, TierCfg cfg, const int2* list, const int64_t* bin_off,
+void launch_symbolic(const Lanes& st, const Items& it, TierCfg cfg, const int2* list, const int64_t* bin_off,
                      const int64_t* bin_cnt, const DenseWork& dw, int64_t* nnz_item, int which = 3);
 template <class SR>
-void launch_numeric(cudaStream_t st, const Items& it, TierCfg cfg, const int2* list, const int64_t* bin_off,
+void launch_numeric(const Lanes& st, const Items& it, TierCfg cfg, const int2* list, const int64_t* bin_off,
                     const int64_t* bin_cnt, const DenseWork& dw, const int64_t* Coff, int32_t* Cir,
                     typename SR::T* Cv, int which = 3);
 
 // numeric pass of the hash tiers into a predicted layout: cap_off are capacity offsets;
 // every item's exact count goes to nnz_item, items that do not fit are not written
 template <class SR>
-void launch_numeric_predicted(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+void launch_numeric_predicted(const Lanes& st, const Items& it, const int2* list, const int64_t* bin_off,
                               const int64_t* bin_cnt, const DenseWork& dw, const int64_t* cap_off, int64_t* nnz_item,
                               int32_t* Cir, typename SR::T* Cv);
 
 // numeric pass of the block tier (blocktier.cu); with nnz_item the counts are recorded and
 // a column is written only when it fits its slots Coff[u+1] - Coff[u]
 template <class SR>
-void launch_block_tier(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+void launch_block_tier(const Lanes& st, const Items& it, const int2* list, const int64_t* bin_off,
                        const int64_t* bin_cnt, const DenseWork& dw, int64_t* nnz_item, const int64_t* Coff,
                        int32_t* Cir, typename SR::T* Cv, int which);
 // numeric pass of the sort bins (sorttier.cu); nnz_item as for launch_block_tier
 template <class SR>
-void launch_sort_tier(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+void launch_sort_tier(const Lanes& st, const Items& it, const int2* list, const int64_t* bin_off,
                       const int64_t* bin_cnt, int64_t* nnz_item, const int64_t* Coff, int32_t* Cir,
                       typename SR::T* Cv, const int* vals_zero);
 // counting pass of the sort bins
-void launch_sort_count(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+void launch_sort_count(const Lanes& st, const Items& it, const int2* list, const int64_t* bin_off,
                        const int64_t* bin_cnt, int64_t* nnz_item);
 // nnz of long columns = sum of their slab counts (and each slab's start in its column)
 void launch_sum_parts(cudaStream_t st, const Items& it, const DenseWork& dw, int64_t* nnz_item);

@@ -251,16 +251,16 @@ __global__ void __launch_bounds__(st_block(K)) k_sort(Items it, const int2* __re
 }
 
 template <class SR, int G, int K, bool NUM>
-void run(cudaStream_t st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item, const int64_t* Coff,
+void run(const Lanes& st, const Items& it, const int2* list, int64_t count, int64_t* nnz_item, const int64_t* Coff,
          int32_t* Cir, typename SR::T* Cv, const int* vals_zero) {
     if (count <= 0) return;
     const int grid = (int)std::min<int64_t>(ceil_div64(count, st_block(K) / G), (int64_t)sm_count() * 32);
-    k_sort<SR, G, K, NUM><<<grid, st_block(K), 0, st>>>(it, list, count, nnz_item, Coff, Cir, Cv, vals_zero);
+    k_sort<SR, G, K, NUM><<<grid, st_block(K), 0, st.next()>>>(it, list, count, nnz_item, Coff, Cir, Cv, vals_zero);
     note_launch();
 }
 
 template <class SR, bool NUM>
-void run_bins(cudaStream_t st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
+void run_bins(const Lanes& st, const Items& it, const int2* list, const int64_t* off, const int64_t* cnt,
               int64_t* nnz_item, const int64_t* Coff, int32_t* Cir, typename SR::T* Cv, const int* vz) {
     constexpr int S = BIN_SORT0;
     run<SR, 8, 2, NUM>(st, it, list + off[S], cnt[S], nnz_item, Coff, Cir, Cv, vz);
@@ -274,19 +274,19 @@ void run_bins(cudaStream_t st, const Items& it, const int2* list, const int64_t*
 }  // namespace
 
 template <class SR>
-void launch_sort_tier(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+void launch_sort_tier(const Lanes& st, const Items& it, const int2* list, const int64_t* bin_off,
                       const int64_t* bin_cnt, int64_t* nnz_item, const int64_t* Coff, int32_t* Cir,
                       typename SR::T* Cv, const int* vals_zero) {
     run_bins<SR, true>(st, it, list, bin_off, bin_cnt, nnz_item, Coff, Cir, Cv, vals_zero);
 }
 
-void launch_sort_count(cudaStream_t st, const Items& it, const int2* list, const int64_t* bin_off,
+void launch_sort_count(const Lanes& st, const Items& it, const int2* list, const int64_t* bin_off,
                        const int64_t* bin_cnt, int64_t* nnz_item) {
     run_bins<MP32, false>(st, it, list, bin_off, bin_cnt, nnz_item, nullptr, nullptr, nullptr, nullptr);
 }
 
 #define SG_INST(SR)                                                                                             \
-    template void launch_sort_tier<SR>(cudaStream_t, const Items&, const int2*, const int64_t*, const int64_t*, \
+    template void launch_sort_tier<SR>(const Lanes&, const Items&, const int2*, const int64_t*, const int64_t*, \
                                        int64_t*, const int64_t*, int32_t*, typename SR::T*, const int*);
 SG_INST(PT64)
 SG_INST(MP32)
