@@ -1131,6 +1131,7 @@ static void run_hash_bins(const Lanes& st, const Items& it, const int2* list, co
 // atomics are the slow path on this part), no hashing and no sort, and a slab's
 // products are spread evenly over the CTA's warps.
 constexpr int RT_BLOCK = 512;
+constexpr int RT_WARPS = RT_BLOCK / 32;
 
 __device__ __forceinline__ int32_t lower_bound_rows(const int32_t* __restrict__ r, int64_t len, int64_t v) {
     int64_t lo = 0, hi = len;
@@ -1227,7 +1228,10 @@ void launch_dense_items(cudaStream_t st, const Items& it, const int2* dense_list
 // entry t of B(:,j), where slab q starts inside A(:,k) (relative to the column's
 // start); row P holds A(:,k)'s length.  One CTA per slab, every search of the slab
 // in flight at once (the passes that read them no longer wait on search chains at
-// their barriers).
+// their barriers).  A slab is one chain of loads whatever its entries (29 on average at
+// R-MAT 20): half as many threads per CTA where there are very many slabs put twice as many
+// in flight (R-MAT 20 flat 3.7 -> 2.3 ms), but leave longer columns of B to fewer threads
+// (restriction, 20,000 slabs: 93 -> 173 us).
 __global__ void __launch_bounds__(256) k_slab_bounds(Items it, DenseWork dw) {
     const int64_t nsym = (int64_t)*dw.nitems;
     for (int64_t w = blockIdx.x; w < nsym; w += gridDim.x) {
@@ -1337,63 +1341,20 @@ void launch_false_values(cudaStream_t st, const Items& it, int* flag) {
     note_launch();
 }
 
-// Inclusive scan of a 64-bit value over the CTA (RT_BLOCK threads).
-__device__ __forceinline__ unsigned long long rt_block_incl_scan64(unsigned long long v, unsigned long long* ws,
-                                                                   unsigned long long& total) {
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    unsigned long long x = v;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) ws[w] = x;
-    __syncthreads();
-    if (w == 0) {
-        unsigned long long s = lane < RT_BLOCK / 32 ? ws[lane] : 0ull;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            unsigned long long y = __shfl_up_sync(0xffffffffu, s, o);
-            if (lane >= o) s += y;
-        }
-        if (lane < RT_BLOCK / 32) ws[lane] = s;
-    }
-    __syncthreads();
-    const unsigned long long add = w > 0 ? ws[w - 1] : 0ull;
-    total = ws[RT_BLOCK / 32 - 1];
-    __syncthreads();
-    return x + add;
-}
-
-struct RangeSmem {   // per-batch segments of the flattened expansion (compacted: all nonempty)
-    int end[RT_BLOCK];        // inclusive prefix of segment lengths (exclusive end in flattened space)
-    int64_t start[RT_BLOCK];  // first position of the segment in A.ir
+// The segments of one batch of RT_BLOCK entries of B(:,j), the nonempty ones in order: part a
+// .. b of the arrays of A, and where it ends in the batch's flattened products (QUADS: in
+// aligned quads of A's arrays, so that quad x of the batch is quad q + x of the array).
+struct SegSmem {
+    union {
+        int4 seg[RT_BLOCK];       // QUADS: q, a, b
+        int64_t start[RT_BLOCK];  // otherwise: a minus the products before the segment
+    };
     int64_t bv[RT_BLOCK];     // B value bits (read back as SR::T)
-    int64_t stop[RT_BLOCK];   // one past the segment's last position (quad walks)
-    unsigned long long ws[32];
-    int wc[RT_BLOCK / 32 + 1];
+    int end[RT_BLOCK];
+    int2 tot[RT_WARPS];       // per warp: segments and products of its entries
 };
-// shared-memory offset of what follows a RangeSmem (16-byte aligned for vector access)
-constexpr size_t RS_BYTES = (sizeof(RangeSmem) + 15) / 16 * 16;
-
-// Compacts the active (k, segment) pairs of this batch into sc and returns
-// (number of segments, number of products).  Called by all threads.
-__device__ __forceinline__ void rt_compact(RangeSmem* sc, bool active, int len, int64_t a, int64_t bvbits, int& ns,
-                                           int& T, int64_t stop = 0) {
-    const unsigned long long packed = active && len > 0 ? ((1ull << 32) | (unsigned)len) : 0ull;
-    unsigned long long tot;
-    const unsigned long long inc = rt_block_incl_scan64(packed, sc->ws, tot);
-    if (packed) {
-        const int pos = (int)(inc >> 32) - 1;
-        sc->end[pos] = (int)(inc & 0xffffffffull);
-        sc->start[pos] = a;
-        sc->bv[pos] = bvbits;
-        sc->stop[pos] = stop;
-    }
-    ns = (int)(tot >> 32);
-    T = (int)(tot & 0xffffffffull);
-    __syncthreads();
-}
+// shared-memory offset of what follows a SegSmem (16-byte aligned for vector access)
+constexpr size_t RS_BYTES = (sizeof(SegSmem) + 15) / 16 * 16;
 
 // Where A(:,k) starts for entry i of B(:,j) (deg entries): two int32 rows of the
 // column's boundary table, low and high 32 bits, written by the boundary pre-pass.
@@ -1401,72 +1362,49 @@ __device__ __forceinline__ int64_t seg_start(const int32_t* __restrict__ sab, in
     return (int64_t)(uint32_t)__ldg(sab + i) | ((int64_t)__ldg(sab + deg + i) << 32);
 }
 
-// Flattened walk over the products of rows [R0, R1) of column bs..be of B: B's
-// entries in chunks of RT_BLOCK; per entry the part of A(:,k) inside the rows
-// (two binary searches), compacted into segments; each warp takes a contiguous
-// slice of the chunk's products, four 32-product windows per step with every load
-// issued before the updates.  f(valid, row, a, b) is called by all 32 lanes of a
-// warp for each window of products (a and b, the A and B values, only when NUM;
-// row is INT_MIN on lanes without a product).  Ends with a CTA barrier.
-template <class SR, bool NUM, class F>
-__device__ __forceinline__ void slab_walk(const Items& it, const Prod* pr, int64_t bs, int64_t be,
-                                          const int32_t* __restrict__ brow0, const int32_t* __restrict__ brow1,
-                                          const int32_t* __restrict__ sab, RangeSmem* sc, F&& f) {
-    using T = typename SR::T;
-    constexpr int U = 4, NWARP = RT_BLOCK / 32;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int32_t* __restrict__ air = pr->A.ir;
-    for (int64_t b0 = bs; b0 < be; b0 += RT_BLOCK) {
-        const int64_t t = b0 + tid;
-        int len = 0;
-        int64_t a = 0, bvbits = 0;
+// The segments of entries [b0, b0 + RT_BLOCK) of B(:,j) inside rows [R0, R1): brow0 / brow1 are
+// the boundary rows of R0 and R1.  With VALS also B's values.  Returns the number of segments
+// and of products (quads).  A warp without entries only meets the two barriers, the second of
+// which publishes the segments.
+template <class SR, bool VALS, bool QUADS>
+__device__ __forceinline__ void slab_segments(const Prod* pr, int64_t b0, int64_t bs, int64_t be,
+                                              const int32_t* __restrict__ brow0, const int32_t* __restrict__ brow1,
+                                              const int32_t* __restrict__ sab, SegSmem* sc, int& ns, int& T) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t t = b0 + threadIdx.x;
+    int len = 0, inc = 0, rank = 0;
+    int64_t a = 0, b = 0, bvbits = 0;
+    if (b0 + warp * 32 < be) {
         if (t < be) {
             const int64_t s = seg_start(sab, t - bs, be - bs);
             a = s + __ldg(brow0 + (t - bs));
-            const int64_t b = s + __ldg(brow1 + (t - bs));
-            len = (int)(b - a);
-            if constexpr (NUM) *reinterpret_cast<T*>(&bvbits) = load_val<SR>(pr->B, t);
+            b = s + __ldg(brow1 + (t - bs));
+            if constexpr (QUADS) len = b > a ? (int)(((b - 1) >> 2) - (a >> 2) + 1) : 0;
+            else len = (int)(b - a);
+            if constexpr (VALS) *reinterpret_cast<typename SR::T*>(&bvbits) = load_val<SR>(pr->B, t);
         }
-        int ns, Tn;
-        rt_compact(sc, t < be, len, a, bvbits, ns, Tn);
-        const int C = (Tn + NWARP * 32 - 1) / (NWARP * 32) * 32;
-        const int xb = warp * C, xe = min(Tn, xb + C);
-        if (xb < xe) {
-            int lo = 0, hi = ns;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (sc->end[mid] <= xb) lo = mid + 1;
-                else hi = mid;
-            }
-            int o0 = lo;
-            for (int x0 = xb; x0 < xe; x0 += 32 * U) {
-                int64_t idx[U];
-                bool ok[U];
-                int ob[U];
-#pragma unroll
-                for (int uu = 0; uu < U; ++uu) {
-                    const int xw = x0 + 32 * uu;
-                    const int oi = warp_window_segment(sc->end, ns, xw, o0);
-                    ok[uu] = xw + lane < xe;
-                    ob[uu] = oi;
-                    idx[uu] = ok[uu] ? sc->start[oi] + (xw + lane - (oi ? sc->end[oi - 1] : 0)) : 0;
-                }
-                int32_t row[U];
-                T av[U];
-#pragma unroll
-                for (int uu = 0; uu < U; ++uu) {
-                    row[uu] = ok[uu] ? __ldg(air + idx[uu]) : INT_MIN;
-                    if constexpr (NUM) av[uu] = ok[uu] ? load_val<SR>(pr->A, idx[uu]) : T(0);
-                }
-#pragma unroll
-                for (int uu = 0; uu < U; ++uu) {
-                    if constexpr (NUM) f(ok[uu], row[uu], av[uu], ok[uu] ? *reinterpret_cast<const T*>(&sc->bv[ob[uu]]) : T(0));
-                    else f(ok[uu], row[uu], T(0), T(0));
-                }
-            }
-        }
-        __syncthreads();
+        inc = warp_incl_scan(len);
+        const unsigned some = __ballot_sync(0xffffffffu, len > 0);
+        rank = __popc(some & ((1u << lane) - 1u));
+        if (lane == 31) sc->tot[warp] = make_int2(__popc(some), inc);
+    } else if (lane == 31) {
+        sc->tot[warp] = make_int2(0, 0);
     }
+    __syncthreads();
+    const int2 w = lane < RT_WARPS ? sc->tot[lane] : make_int2(0, 0);
+    ns = __reduce_add_sync(0xffffffffu, w.x);
+    T = __reduce_add_sync(0xffffffffu, w.y);
+    if (b0 + warp * 32 < be) {
+        const int i = rank + __reduce_add_sync(0xffffffffu, lane < warp ? w.x : 0);
+        const int e = inc + __reduce_add_sync(0xffffffffu, lane < warp ? w.y : 0);
+        if (len > 0) {
+            sc->end[i] = e;
+            if constexpr (QUADS) sc->seg[i] = make_int4((int)(a >> 2) - (e - len), (int)a, (int)b, 0);
+            else sc->start[i] = a - (e - len);
+            if constexpr (VALS) sc->bv[i] = bvbits;
+        }
+    }
+    __syncthreads();
 }
 
 // Four consecutive values of A at an aligned position p (16-byte loads: one for
@@ -1491,115 +1429,149 @@ __device__ __forceinline__ void load4(const T* __restrict__ p, T v[4]) {
     }
 }
 
-// slab_walk over aligned quads: a segment [a, b) of A(:,k) covers the quads
-// q = a/4 .. (b-1)/4, and each lane takes one quad per window, loading its four
-// rows with one 16-byte load (and its values with one or two) and masking the
-// positions outside [a, b).  U windows per step, every load issued before the
-// updates.  Needs A.ir and A.num 16-byte aligned and A a CSC whose arrays hold
-// nnz_end entries (a quad past the end is read one by one).
-// f(valid, row, a, b) as in slab_walk, four times per window.
-template <class SR, bool NUM, int U, class F>
-__device__ __forceinline__ void slab_walk_quads(const Items& it, const Prod* pr, int64_t bs, int64_t be,
-                                                const int32_t* __restrict__ brow0,
-                                                const int32_t* __restrict__ brow1, const int32_t* __restrict__ sab,
-                                                int64_t nnz_end, RangeSmem* sc, F&& f) {
-    using T = typename SR::T;
-    constexpr int NWARP = RT_BLOCK / 32;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// Positions p0 .. p0 + 3 of A (an aligned quad): rows, and values with NUM.  A quad past the
+// arrays' end (nnz_end entries) is read one by one.
+template <class SR, bool NUM>
+__device__ __forceinline__ void load_quad(const Prod* pr, int p0, int nnz_end, int32_t (&row)[4],
+                                          typename SR::T (&av)[4]) {
+    using V = typename SR::T;
     const int32_t* __restrict__ air = pr->A.ir;
-    const T* __restrict__ anum = reinterpret_cast<const T*>(pr->A.num);
+    const V* __restrict__ anum = reinterpret_cast<const V*>(pr->A.num);
+    if (p0 + 4 <= nnz_end) {
+        const int4 r4 = __ldg(reinterpret_cast<const int4*>(air + p0));
+        row[0] = r4.x;
+        row[1] = r4.y;
+        row[2] = r4.z;
+        row[3] = r4.w;
+        if constexpr (NUM) {
+            if (anum) load4<V>(anum + p0, av);
+            else av[0] = av[1] = av[2] = av[3] = (V)SR::one();
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            if (p0 + j < nnz_end) {
+                row[j] = __ldg(air + p0 + j);
+                if constexpr (NUM) av[j] = load_val<SR>(pr->A, p0 + j);
+            }
+    }
+}
+
+// bit j: position p0 + j lies in [a, b), which meets the quad
+__device__ __forceinline__ unsigned quad_mask(int p0, int a, int b) {
+    return (0xfu << max(a - p0, 0)) & (0xfu >> (4 - min(b - p0, 4)));
+}
+
+// Walk over the products of the batch in sc: each warp takes a contiguous slice, U windows of
+// 32 per step with every load issued before the updates.  With QUADS a lane takes an aligned
+// quad per window (rows by one 16-byte load, values by one or two); positions are 32-bit and
+// A.ir and A.num 16-byte aligned.  f(row, a, b) is called for every product of the lane (a and
+// b, the A and B values, only with NUM).  A window inside one segment needs no search for its
+// segments, and a window of whole quads no masks.  One quad per lane and step: the passes are
+// bound by instructions and their latency, so registers go to warps (four CTAs of 512 threads
+// per SM at 32 registers, where two at 64 kept two quads in flight).  Counting pass, R-MAT 18
+// 3.2 -> 2.3 ms, 300,007 vertices 3.6 -> 2.6 ms, R-MAT 20 (slabs of 2^18 rows) 32.7 -> 25.4 ms;
+// numeric pass, boolean 3.0 -> 2.7 ms, int64 623 -> 532 us, FP64 at R-MAT 20 52.4 -> 51.1 ms.
+template <class SR, bool NUM, bool QUADS, class F>
+__device__ __forceinline__ void slab_walk(const Prod* pr, const SegSmem* sc, int ns, int T, F&& f) {
+    using V = typename SR::T;
+    constexpr int U = QUADS ? 1 : 4, J = QUADS ? 4 : 1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int C = (T + RT_BLOCK - 1) / RT_BLOCK * 32;
+    const int xb = warp * C, xe = min(T, xb + C);
+    if (xb >= xe) return;
+    int lo = 0, hi = xb > 0 ? ns : 0;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (sc->end[mid] <= xb) lo = mid + 1;
+        else hi = mid;
+    }
+    int o0 = lo, cend = sc->end[lo];   // the segment that the next window starts in
+    [[maybe_unused]] const int nnz_end = QUADS ? (int)pr->A.nnz : 0;
+    [[maybe_unused]] const int32_t* __restrict__ air = pr->A.ir;
+    for (int x0 = xb; x0 < xe; x0 += 32 * U) {
+        int32_t row[U][J];
+        V av[U][J];
+        V bv[U];
+        unsigned vm[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int xw = x0 + 32 * u, x = xw + lane;
+            int oi = o0;
+            if (xw + 32 >= cend) {
+                oi = warp_window_segment(sc->end, ns, xw, o0);
+                cend = o0 < ns ? sc->end[o0] : INT_MAX;
+            }
+            vm[u] = 0u;
+            bv[u] = V(0);
+            if (x < xe) {
+                if constexpr (NUM) bv[u] = *reinterpret_cast<const V*>(&sc->bv[oi]);
+                if constexpr (QUADS) {
+                    const int4 sg = sc->seg[oi];
+                    const int p0 = (sg.x + x) << 2;
+                    vm[u] = quad_mask(p0, sg.y, sg.z);
+                    load_quad<SR, NUM>(pr, p0, nnz_end, row[u], av[u]);
+                } else {
+                    const int64_t p = sc->start[oi] + x;
+                    vm[u] = 1u;
+                    row[u][0] = __ldg(air + p);
+                    if constexpr (NUM) av[u][0] = load_val<SR>(pr->A, p);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (QUADS && __all_sync(0xffffffffu, vm[u] == 0xfu)) {
+#pragma unroll
+                for (int j = 0; j < J; ++j) f(row[u][j], av[u][j], bv[u]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < J; ++j)
+                    if ((vm[u] >> j) & 1u) f(row[u][j], av[u][j], bv[u]);
+            }
+        }
+    }
+}
+
+// The products of column B(:,j) inside the slab, batch after batch; ends with a CTA barrier.
+template <class SR, bool NUM, bool QUADS, class F>
+__device__ __forceinline__ void slab_products(const Prod* pr, int64_t bs, int64_t be, const int32_t* __restrict__ brow0,
+                                              const int32_t* __restrict__ brow1, const int32_t* __restrict__ sab,
+                                              SegSmem* sc, F&& f) {
     for (int64_t b0 = bs; b0 < be; b0 += RT_BLOCK) {
-        const int64_t t = b0 + tid;
-        int nq = 0;
-        int64_t a = 0, b = 0, bvbits = 0;
-        if (t < be) {
-            const int64_t s = seg_start(sab, t - bs, be - bs);
-            a = s + __ldg(brow0 + (t - bs));
-            b = s + __ldg(brow1 + (t - bs));
-            nq = b > a ? (int)(((b - 1) >> 2) - (a >> 2) + 1) : 0;
-            if constexpr (NUM) *reinterpret_cast<T*>(&bvbits) = load_val<SR>(pr->B, t);
-        }
-        int ns, Tq;
-        rt_compact(sc, t < be, nq, a, bvbits, ns, Tq, b);
-        const int C = (Tq + NWARP * 32 - 1) / (NWARP * 32) * 32;
-        const int xb = warp * C, xe = min(Tq, xb + C);
-        if (xb < xe) {
-            int lo = 0, hi = xb > 0 ? ns : 0;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (sc->end[mid] <= xb) lo = mid + 1;
-                else hi = mid;
-            }
-            int o0 = lo;
-            for (int x0 = xb; x0 < xe; x0 += 32 * U) {
-                int4 rq[U];
-                T av[U][4];
-                T bv[U];
-                unsigned vm[U];   // bit j: position p0 + j lies in the segment
-#pragma unroll
-                for (int uu = 0; uu < U; ++uu) {
-                    const int xw = x0 + 32 * uu;
-                    const int oi = warp_window_segment(sc->end, ns, xw, o0);
-                    rq[uu] = make_int4(INT_MIN, INT_MIN, INT_MIN, INT_MIN);
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) av[uu][j] = T(0);
-                    bv[uu] = T(0);
-                    vm[uu] = 0u;
-                    if (xw + lane < xe) {
-                        const int64_t sa = sc->start[oi], sb = sc->stop[oi];
-                        const int64_t p0 = ((sa >> 2) + (xw + lane - (oi ? sc->end[oi - 1] : 0))) << 2;
-                        // sa - p0 is in [-inf, 3] and sb - p0 in [1, inf): the quad holds
-                        // positions lo .. hi-1 of the segment
-                        const int qlo = (int)max(sa - p0, (int64_t)0);
-                        const int qhi = (int)min(sb - p0, (int64_t)4);
-                        vm[uu] = (0xfu << qlo) & (0xfu >> (4 - qhi));
-                        if (p0 + 4 <= nnz_end) {
-                            rq[uu] = __ldg(reinterpret_cast<const int4*>(air + p0));
-                            if constexpr (NUM) {
-                                if (anum) load4<T>(anum + p0, av[uu]);
-                                else av[uu][0] = av[uu][1] = av[uu][2] = av[uu][3] = (T)SR::one();
-                            }
-                        } else {   // the array's last, partial quad
-                            int32_t r4[4] = {INT_MIN, INT_MIN, INT_MIN, INT_MIN};
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-                                if (p0 + j < nnz_end) {
-                                    r4[j] = __ldg(air + p0 + j);
-                                    if constexpr (NUM) av[uu][j] = load_val<SR>(pr->A, p0 + j);
-                                }
-                            rq[uu] = make_int4(r4[0], r4[1], r4[2], r4[3]);
-                        }
-                        if constexpr (NUM) bv[uu] = *reinterpret_cast<const T*>(&sc->bv[oi]);
-                    }
-                }
-#pragma unroll
-                for (int uu = 0; uu < U; ++uu) {
-                    const int32_t r4[4] = {rq[uu].x, rq[uu].y, rq[uu].z, rq[uu].w};
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const bool v = (vm[uu] >> j) & 1u;
-                        f(v, v ? r4[j] : INT_MIN, av[uu][j], bv[uu]);
-                    }
-                }
-            }
-        }
+        int ns, T;
+        slab_segments<SR, NUM, QUADS>(pr, b0, bs, be, brow0, brow1, sab, sc, ns, T);
+        slab_walk<SR, NUM, QUADS>(pr, sc, ns, T, f);
         __syncthreads();
     }
 }
 
-// the quad walk applies to a product whose A is a CSC (no DCSC index, no gaps) with
-// 16-byte aligned row and value arrays
-__device__ __forceinline__ bool quads_ok(const Prod* pr) {
-    return pr->A.jc == nullptr && pr->A.ce == nullptr && ((uintptr_t)pr->A.ir & 15) == 0 &&
+// the quad walk applies to a product whose A is a CSC (no DCSC index, no gaps) of fewer than
+// 2^31 entries with 16-byte aligned row and value arrays
+__host__ __device__ __forceinline__ bool quads_ok(const Prod* pr) {
+    return pr->A.jc == nullptr && pr->A.ce == nullptr && pr->A.nnz < INT_MAX - 8 && ((uintptr_t)pr->A.ir & 15) == 0 &&
            ((uintptr_t)pr->A.num & 15) == 0;
 }
 
+// the semiring whose slabs add up in shared memory
+constexpr bool slab_local(int sr) { return sr == SPGEMM_MIN_PLUS_F32; }
+// shared memory of the numeric pass before its accumulators
+__host__ __device__ constexpr size_t slab_num_bytes(int RB) { return (RS_BYTES + (size_t)(RB / 128 + 1) * 20 + 15) / 16 * 16; }
+// accumulators that leave room for two CTAs per SM beside slabs of RB rows
+constexpr size_t SLAB_SMEM = 113152;
+
+int slab_acc_entries(int sr, int RB) {
+    if (!slab_local(sr) || slab_num_bytes(RB) >= SLAB_SMEM) return 0;
+    return (int)((SLAB_SMEM - slab_num_bytes(RB)) / sizeof(MP32::Acc));
+}
+
 // Symbolic slab kernel: mark, count, store the row set.
-__global__ void __launch_bounds__(RT_BLOCK, 2) k_slab_sym(Items it, DenseWork dw) {
+template <bool QUADS>
+__global__ void __launch_bounds__(RT_BLOCK, 4) k_slab_sym(Items it, DenseWork dw) {
     extern __shared__ __align__(16) unsigned char smem[];
-    RangeSmem* sc = reinterpret_cast<RangeSmem*>(smem);
+    SegSmem* sc = reinterpret_cast<SegSmem*>(smem);
     uint32_t* bitmap = reinterpret_cast<uint32_t*>(smem + RS_BYTES);
-    int* s_scan = sc->wc;
+    int* s_scan = reinterpret_cast<int*>(sc->tot);
     __shared__ long long s_off;
     __shared__ SlabRec s_rec[2];   // this slab's record and the next one's, in flight
     constexpr int RC = sizeof(SlabRec) / 16;
@@ -1626,22 +1598,21 @@ __global__ void __launch_bounds__(RT_BLOCK, 2) k_slab_sym(Items it, DenseWork dw
         const int32_t r0 = (int32_t)R0;
         // one shared atomic per product: R-MAT rows of one window mostly fall in different
         // words, so folding lanes per word first (shuffles) measured slower
-        auto mark = [&](bool ok, int32_t row, uint8_t, uint8_t) {
+        auto mark = [&](int32_t row, uint8_t, uint8_t) {
             const int lr = row - r0;
-            if (ok && (unsigned)lr < (unsigned)span) atomicOr(&bitmap[lr >> 5], 1u << (lr & 31));
+            if ((unsigned)lr < (unsigned)span) atomicOr(&bitmap[lr >> 5], 1u << (lr & 31));
         };
         const int32_t* brow0 = dw.bnd + rc.bnd;
         const int32_t* brow1 = brow0 + (be - bs);
         const int32_t* sab = dw.bnd + rc.sab;
-        if (quads_ok(pr)) slab_walk_quads<BOOL8, false, 2>(it, pr, bs, be, brow0, brow1, sab, pr->A.nnz, sc, mark);
-        else slab_walk<BOOL8, false>(it, pr, bs, be, brow0, brow1, sab, sc, mark);
+        slab_products<BOOL8, false, QUADS>(pr, bs, be, brow0, brow1, sab, sc, mark);
         // count per chunk of 32 groups (lane l reads group 32 c + l with one 16-byte load:
         // no bank conflicts); a thread owns cpt consecutive chunks for the CTA scan
         constexpr int NWARP = RT_BLOCK / 32;
         const int lane = tid & 31, warp = tid >> 5;
         const int nch = (ng + 31) >> 5;
         const uint4* __restrict__ grp4 = reinterpret_cast<const uint4*>(bitmap);
-        int* s_cc = reinterpret_cast<int*>(sc->start);   // the walk's segment arrays are free now
+        int* s_cc = reinterpret_cast<int*>(sc->seg);   // the walk's segment arrays are free now
         for (int cc = warp; cc < nch; cc += NWARP) {
             const int g = cc * 32 + lane;
             int c = 0;
@@ -1711,16 +1682,24 @@ __global__ void __launch_bounds__(RT_BLOCK, 2) k_slab_sym(Items it, DenseWork dw
     }
 }
 
-// Numeric slab kernel: row set -> ranks -> C's rows, zero values, L2 reductions.
-template <class SR>
-__global__ void __launch_bounds__(RT_BLOCK, 2) k_slab_num(Items it, DenseWork dw, const int64_t* __restrict__ Coff,
-                                                          int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv) {
+// Numeric slab kernel: row set -> ranks -> C's rows, zero values, products added at their
+// ranks.  Min-plus slabs of at most acc_cap entries add up in shared memory, whose 32-bit
+// atomics are native (the L2 takes 2.1e11 random reductions a second whatever their width),
+// and store their values once: R-MAT 18 7.0 -> 6.0 ms.  Longer ones and the other semirings
+// add into C by L2 reductions: a shared FP64 addition is a compare-and-swap loop (three
+// times slower than the L2 at R-MAT 20), an int64 one two atomics (20 pairs 623 -> 726 us).
+template <class SR, bool QUADS>
+__global__ void __launch_bounds__(RT_BLOCK, slab_local(SR::id) ? 2 : 4) k_slab_num(Items it, DenseWork dw, const int64_t* __restrict__ Coff,
+                                                          int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv,
+                                                          int acc_cap) {
     using T = typename SR::T;
+    using Acc = typename SR::Acc;
+    constexpr bool LOCAL = slab_local(SR::id);
     extern __shared__ __align__(16) unsigned char smem[];
-    RangeSmem* sc = reinterpret_cast<RangeSmem*>(smem);
+    SegSmem* sc = reinterpret_cast<SegSmem*>(smem);
     uint32_t* bitmap = reinterpret_cast<uint32_t*>(smem + RS_BYTES);              // groups * 4 words
     int* gp = reinterpret_cast<int*>(bitmap + (size_t)(dw.RB / 128 + 1) * 4);    // rows before each group
-    int* s_scan = sc->wc;
+    Acc* acc = reinterpret_cast<Acc*>(smem + slab_num_bytes(dw.RB));
     const int tid = threadIdx.x;
     // boolean products whose operands hold no false value: every output is true
     const bool walk = SR::id != SPGEMM_OR_AND_BOOL || dw.vals_zero == nullptr || *dw.vals_zero != 0;
@@ -1777,39 +1756,36 @@ __global__ void __launch_bounds__(RT_BLOCK, 2) k_slab_num(Items it, DenseWork dw
             }
         }
         __syncthreads();
-        // 2. rows before every group: a warp per chunk of 32 groups (lane l reads group
-        //    32 c + l: no bank conflicts), chunk totals scanned by the CTA, then added
-        constexpr int NWARP = RT_BLOCK / 32;
+        // 2. rows before every group: chunk totals (a warp per chunk of 32 groups, lane l reads
+        //    group 32 c + l: no bank conflicts), their scan by one warp, then every group's
         const int lane = tid & 31, warp = tid >> 5;
         const int nch = (ng + 31) >> 5;
-        int* s_cc = reinterpret_cast<int*>(sc->start);   // free until the walk
-        for (int cc = warp; cc < nch; cc += NWARP) {
+        int* s_cc = reinterpret_cast<int*>(sc->seg);   // free until the walk
+        for (int cc = warp; cc < nch; cc += RT_WARPS) {
             const int g = cc * 32 + lane;
-            int c = 0;
-            if (g < ng) {
-                const uint4 grp = reinterpret_cast<const uint4*>(bitmap)[g];
-                c = __popc(grp.x) + __popc(grp.y) + __popc(grp.z) + __popc(grp.w);
-            }
-            const int inc = warp_incl_scan(c);
-            if (g < ng) gp[g] = inc - c;
-            if (lane == 31) s_cc[cc] = inc;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (g < ng) v = reinterpret_cast<const uint4*>(bitmap)[g];
+            const int c = __reduce_add_sync(0xffffffffu, __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w));
+            if (lane == 0) s_cc[cc] = c;
         }
         __syncthreads();
-        {
-            const int cpt = (nch + RT_BLOCK - 1) / RT_BLOCK;
-            const int c0 = min(tid * cpt, nch), c1 = min(c0 + cpt, nch);
-            int c = 0;
-            for (int cc = c0; cc < c1; ++cc) c += s_cc[cc];
-            int total;
-            int excl = group_incl_scan<RT_BLOCK>(c, s_scan, total) - c;
-            for (int cc = c0; cc < c1; ++cc) {
-                const int v = s_cc[cc];
-                s_cc[cc] = excl;
-                excl += v;
+        if (warp == 0) {
+            int run = 0;
+            for (int c0 = 0; c0 < nch; c0 += 32) {
+                const int v = c0 + lane < nch ? s_cc[c0 + lane] : 0, inc = warp_incl_scan(v);
+                if (c0 + lane < nch) s_cc[c0 + lane] = run + inc - v;
+                run += __shfl_sync(0xffffffffu, inc, 31);
             }
         }
         __syncthreads();
-        for (int g = tid; g < ng; g += RT_BLOCK) gp[g] += s_cc[g >> 5];
+        for (int cc = warp; cc < nch; cc += RT_WARPS) {
+            const int g = cc * 32 + lane;
+            uint4 v = make_uint4(0u, 0u, 0u, 0u);
+            if (g < ng) v = reinterpret_cast<const uint4*>(bitmap)[g];
+            const int c = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+            const int r = s_cc[cc] + warp_incl_scan(c) - c;
+            if (g < ng) gp[g] = r;
+        }
         __syncthreads();
         // 3. C's rows of a bitmap slab: a warp per chunk of 32 groups; lanes write their
         //    group's rows from its rank base, or, for chunks of at least 16 rows a word,
@@ -1817,7 +1793,7 @@ __global__ void __launch_bounds__(RT_BLOCK, 2) k_slab_num(Items it, DenseWork dw
         //    covers neighbouring addresses
         if (dense) {
             const uint4* __restrict__ grp4 = reinterpret_cast<const uint4*>(bitmap);
-            for (int cc = warp; cc < nch; cc += NWARP) {
+            for (int cc = warp; cc < nch; cc += RT_WARPS) {
                 const int g = cc * 32 + lane;
                 uint4 v = make_uint4(0u, 0u, 0u, 0u);
                 if (g < ng) v = grp4[g];
@@ -1852,31 +1828,44 @@ __global__ void __launch_bounds__(RT_BLOCK, 2) k_slab_num(Items it, DenseWork dw
             }
         }
         // 4. values: the semiring zero (all true for the boolean shortcut)
-        for (int i = tid; i < cnt; i += RT_BLOCK) Cv[ob + i] = init;
-        __syncthreads();   // the stores above come before this CTA's reductions
+        const bool local = LOCAL && cnt <= acc_cap;
+        if (local)
+            for (int i = tid; i < cnt; i += RT_BLOCK) acc[i] = SR::zero();
+        else
+            for (int i = tid; i < cnt; i += RT_BLOCK) Cv[ob + i] = init;
+        __syncthreads();   // the stores above come before this CTA's additions
         // 5. every product, added at its row's rank
         if (walk) {
             const int span = (int)(R1 - R0);
             const int32_t r0 = (int32_t)R0;
-            auto add = [&](bool ok, int32_t row, T a, T b) {
-                if (!ok) return;
+            // rank of a row in the slab's set; -1 for rows outside it (malformed input only)
+            auto rank_of = [&](int32_t row) {
                 const int lr = row - r0;
-                if ((unsigned)lr >= (unsigned)span) return;   // malformed input only
+                if ((unsigned)lr >= (unsigned)span) return -1;
                 const int wd = lr >> 5, g = wd >> 2, y = wd & 3;
                 const uint4 grp = reinterpret_cast<const uint4*>(bitmap)[g];
                 const uint32_t wv = y == 0 ? grp.x : y == 1 ? grp.y : y == 2 ? grp.z : grp.w;
                 const uint32_t bit = 1u << (lr & 31);
-                if (!(wv & bit)) return;                      // malformed input only
-                const int rank = gp[g] + __popc(wv & (bit - 1u)) + (y > 0 ? __popc(grp.x) : 0) +
-                                 (y > 1 ? __popc(grp.y) : 0) + (y > 2 ? __popc(grp.z) : 0);
-                red_out<SR>(Cv, ob + rank, SR::mul(a, b));
+                if (!(wv & bit)) return -1;
+                return gp[g] + __popc(wv & (bit - 1u)) + (y > 0 ? __popc(grp.x) : 0) + (y > 1 ? __popc(grp.y) : 0) +
+                       (y > 2 ? __popc(grp.z) : 0);
             };
             const int64_t bs = rc.bs, be = rc.be;
             const int32_t* brow0 = dw.bnd + rc.bnd;
             const int32_t* brow1 = brow0 + (be - bs);
             const int32_t* sab = dw.bnd + rc.sab;
-            if (quads_ok(pr)) slab_walk_quads<SR, true, 2>(it, pr, bs, be, brow0, brow1, sab, pr->A.nnz, sc, add);
-            else slab_walk<SR, true>(it, pr, bs, be, brow0, brow1, sab, sc, add);
+            if (LOCAL && local) {
+                slab_products<SR, true, QUADS>(pr, bs, be, brow0, brow1, sab, sc, [&](int32_t row, T a, T b) {
+                    const int rank = rank_of(row);
+                    if (rank >= 0 && rank < cnt) SR::atomic_add(acc + rank, SR::mul(a, b));
+                });
+                for (int i = tid; i < cnt; i += RT_BLOCK) __stcs(Cv + ob + i, SR::out(acc[i]));
+            } else {
+                slab_products<SR, true, QUADS>(pr, bs, be, brow0, brow1, sab, sc, [&](int32_t row, T a, T b) {
+                    const int rank = rank_of(row);
+                    if (rank >= 0) red_out<SR>(Cv, ob + rank, SR::mul(a, b));
+                });
+            }
         } else {
             __syncthreads();
         }
@@ -1889,6 +1878,8 @@ __global__ void k_slab_fin(DenseWork dw, const int64_t* __restrict__ Coff) {
     for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nsym; w += (int64_t)gridDim.x * blockDim.x)
         dw.rec[w].ob = __ldg(Coff + dw.rec[w].u) + dw.spref[w];
 }
+
+bool slab_quads(const Prod& pr) { return quads_ok(&pr); }
 
 // CTAs per SM the kernel can keep resident with `smem` bytes, times the SM count
 static int resident_grid(const void* fn, int block, size_t smem) {
@@ -1907,19 +1898,23 @@ static void run_slabs(const Lanes& lanes, const Items& it, const DenseWork& dw, 
     const cudaStream_t st = lanes.next();
     const int64_t nslab_max = dw.nslabs > 0 ? dw.nslabs : dw.ndense * MAX_PARTS;
     if (!numeric) {
-        k_slab_bounds<<<(int)std::min<int64_t>(nslab_max, sm_count() * 8), 256, 0, st>>>(it, dw);
+        const int bnd_block = nslab_max >= (1 << 19) ? 128 : 256;
+        k_slab_bounds<<<(int)std::min<int64_t>(nslab_max, sm_count() * (2048 / bnd_block)), bnd_block, 0, st>>>(it, dw);
         note_launch();
         const size_t smem = RS_BYTES + (size_t)(dw.RB / 128 + 1) * 16;
-        smem_at_least((const void*)k_slab_sym, smem);
-        const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)k_slab_sym, RT_BLOCK, smem));
-        k_slab_sym<<<grid, RT_BLOCK, smem, st>>>(it, dw);
+        auto kern = dw.quads ? k_slab_sym<true> : k_slab_sym<false>;
+        smem_at_least((const void*)kern, smem);
+        const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)kern, RT_BLOCK, smem));
+        kern<<<grid, RT_BLOCK, smem, st>>>(it, dw);
     } else {
         k_slab_fin<<<(int)std::min<int64_t>(ceil_div64(nslab_max, 256), sm_count() * 8), 256, 0, st>>>(dw, Coff);
         note_launch();
-        const size_t smem = RS_BYTES + (size_t)(dw.RB / 128 + 1) * 16 + (size_t)(dw.RB / 128 + 1) * 4;
-        smem_at_least((const void*)k_slab_num<SR>, smem);
-        const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)k_slab_num<SR>, RT_BLOCK, smem));
-        k_slab_num<SR><<<grid, RT_BLOCK, smem, st>>>(it, dw, Coff, Cir, Cv);
+        const int acc_cap = slab_acc_entries(SR::id, dw.RB);
+        const size_t smem = slab_num_bytes(dw.RB) + (size_t)acc_cap * sizeof(typename SR::Acc);
+        auto kern = dw.quads ? k_slab_num<SR, true> : k_slab_num<SR, false>;
+        smem_at_least((const void*)kern, smem);
+        const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)kern, RT_BLOCK, smem));
+        kern<<<grid, RT_BLOCK, smem, st>>>(it, dw, Coff, Cir, Cv, acc_cap);
     }
     note_launch();
 }

@@ -33,8 +33,11 @@ constexpr int WARP_TBL0 = 64;
 constexpr int BLK_TBL0 = 2048;
 // most row slabs of one long column
 constexpr int MAX_PARTS = 64;
-// default most rows of one slab: a 64 KB row bitmap keeps two CTAs per SM
-constexpr int DEFAULT_SLAB_ROWS = 1 << 19;
+// default most rows of one slab: its row bitmap (and ranks) then leave room for four CTAs of
+// the counting pass per SM and three or four of the numeric pass.  R-MAT 20 flat FP64 with
+// one column cut at 2^19 / 2^18 / 2^17 rows: counting 31.3 / 25.3 / 32.3 ms, numeric 55.3 /
+// 51.2 / 56.2 ms; 300,007 rows are better whole than in two slabs (boolean 2.6 against 3.1 ms)
+constexpr int DEFAULT_SLAB_ROWS = 327680;
 // default target flops per slab: every slab repeats its binary searches per entry of
 // B(:,j) and its bitmap set-up, so larger slabs pay up to about this size (R-MAT
 // scale 20 flat: 8192 / 16384 / 32768 / 65536 / 131072 flops per slab give 74.8 /
@@ -97,6 +100,7 @@ struct DenseWork {
     SlabRec* rec = nullptr;               // per slab: its record
     int* err = nullptr;                   // nonzero: a capacity was exceeded
     int RB = 1 << 19;                     // most rows per slab
+    bool quads = false;                   // every A_i can be read in aligned quads (slab_quads)
     // block mode (every A_i has at most BLOCK_TIER_MAX_ROWS rows): long columns
     // are counted with row bitmaps and computed by the block tier; no slabs
     bool dcol = false;
@@ -209,6 +213,10 @@ void launch_dense_items(cudaStream_t st, const Items& it, const int2* dense_list
                         const int64_t* flops, int part_flops, int RB, int2* items, unsigned long long* nitems,
                         int8_t* nparts, int32_t* sbase, unsigned long long* store_bound, int64_t* bbase,
                         unsigned long long* bnd_total);
+// entries that a slab of at most RB rows can add up in shared memory (0: semirings without)
+int slab_acc_entries(int sr, int RB);
+// whether A of the product can be read in aligned quads by the slab passes
+bool slab_quads(const Prod& pr);
 // *flag = 1 when an operand of some product stores a false value (boolean semiring)
 void launch_false_values(cudaStream_t st, const Items& it, int* flag);
 // *flag = 1 when one of the n bytes at vals is 0 (vals == nullptr: nothing)
