@@ -25,18 +25,22 @@ constexpr int L2W = BLOCK_TIER_MAX_ROWS / 32;   // row-bitmap words
 constexpr int L1W = L2W / 32;                   // words of the bitmap of nonempty L2 words
 static_assert(L1W == 32, "one warp owns the first-level bitmap");
 
+// Shared memory of one group, sized by the words `nw` of the row bitmap (a multiple of 32) that
+// the operands of this launch need: the fewer bytes a group takes, the more warps an SM holds.
 template <class SR, int GS>
 struct BtLayout {
     using T = typename SR::T;
-    static constexpr size_t l2 = (size_t)L2W * 4;
-    static constexpr size_t l1 = (size_t)L1W * 4;
-    static constexpr size_t wp = (size_t)L2W * 2;   // rows before each nonempty word (< 2^16)
-    static constexpr size_t gp = (size_t)L2W * 2;   // the nonempty words, ascending
-    static constexpr size_t incl = (size_t)GS * 4;
-    static constexpr size_t a0 = (size_t)GS * 8;
-    static constexpr size_t bv = (size_t)GS * 8;
-    static constexpr size_t ws = 32 * 8;
-    static constexpr size_t group = (l2 + l1 + wp + gp + incl + a0 + bv + ws + 15) / 16 * 16;
+    size_t l1, wp, gp, a0, bv, incl, ws, group;   // the row bitmap is at 0
+    __host__ __device__ explicit BtLayout(int nw) {
+        l1 = (size_t)nw * 4;
+        wp = l1 + (size_t)L1W * 4;             // rows before each nonempty word (< 2^16)
+        gp = wp + (size_t)nw * 2;              // the nonempty words, ascending
+        a0 = gp + (size_t)nw * 2;
+        bv = a0 + (size_t)GS * 8;
+        incl = bv + (size_t)GS * (sizeof(T) < 4 ? 4 : sizeof(T));
+        ws = incl + (size_t)GS * 4;
+        group = (ws + (GS == 32 ? 16 : 32 * 8) + 15) / 16 * 16;
+    }
 };
 
 template <int GS>
@@ -178,33 +182,38 @@ __device__ __forceinline__ int row_word(bool ok, int32_t r, int m) { return ok &
 // offsets are exact.  With nnz_item the column's count is recorded there and the
 // column is written only when it fits its capacity Coff[u+1] - Coff[u] (the
 // predicted and the upper-bound layouts).
+// A warp group's shared memory follows the operands' rows (4.9 KB at 16,384 rows where a
+// fixed 32,768 took 9.2), and its registers are held to 48, so that five CTAs (40 warps) stay
+// resident where three did: both FP64 launches of the 16 x 16 SUMMA at R-MAT 18 together 11.6
+// -> 9.0 ms, min-plus on 100,003 vertices 2.7 -> 2.0 ms (four CTAs 9.6, six at 40 registers
+// 10.3 ms).  The time left is mostly the L2 reductions'.
 // The 512-thread form is held to 32 registers, so that four CTAs (64 warps) stay resident
 // per SM: its time is the walk of L2 reductions, which more warps keep in flight.  In the
 // FP64 32 x 32 SUMMA at R-MAT scale 20, two CTAs per SM (59 registers) took 3.4 ms longer
 // in the stage products and 7.8 ms longer in the merge; three CTAs took 0.4 and 2.0 ms longer.
 template <class SR, int GS, int BLOCK>
-__global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 4 : 1) k_block_tier(Items it, const int2* __restrict__ list, int64_t count,
+__global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 4 : 5) k_block_tier(Items it, const int2* __restrict__ list, int64_t count,
                                                      int64_t* __restrict__ nnz_item, const int64_t* __restrict__ Coff,
                                                      int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv,
-                                                     const int* __restrict__ vals_zero) {
+                                                     const int* __restrict__ vals_zero, int nwords_max) {
     using T = typename SR::T;
-    using L = BtLayout<SR, GS>;
+    const BtLayout<SR, GS> L(nwords_max);
     constexpr int NG = BLOCK / GS;
     extern __shared__ __align__(16) unsigned char smem[];
     const int g = (threadIdx.x / GS), lane = threadIdx.x % GS;
-    unsigned char* base = smem + (size_t)g * L::group;
+    unsigned char* base = smem + (size_t)g * L.group;
     uint32_t* l2 = reinterpret_cast<uint32_t*>(base);
-    uint32_t* l1 = reinterpret_cast<uint32_t*>(base + L::l2);
-    uint16_t* wp = reinterpret_cast<uint16_t*>(base + L::l2 + L::l1);
-    uint16_t* wl = reinterpret_cast<uint16_t*>(base + L::l2 + L::l1 + L::wp);
-    int* s_incl = reinterpret_cast<int*>(base + L::l2 + L::l1 + L::wp + L::gp);
-    int64_t* s_a0 = reinterpret_cast<int64_t*>(base + L::l2 + L::l1 + L::wp + L::gp + L::incl);
-    T* s_bv = reinterpret_cast<T*>(base + L::l2 + L::l1 + L::wp + L::gp + L::incl + L::a0);
-    long long* ws = reinterpret_cast<long long*>(base + L::l2 + L::l1 + L::wp + L::gp + L::incl + L::a0 + L::bv);
+    uint32_t* l1 = reinterpret_cast<uint32_t*>(base + L.l1);
+    uint16_t* wp = reinterpret_cast<uint16_t*>(base + L.wp);
+    uint16_t* wl = reinterpret_cast<uint16_t*>(base + L.gp);
+    int* s_incl = reinterpret_cast<int*>(base + L.incl);
+    int64_t* s_a0 = reinterpret_cast<int64_t*>(base + L.a0);
+    T* s_bv = reinterpret_cast<T*>(base + L.bv);
+    long long* ws = reinterpret_cast<long long*>(base + L.ws);
     // boolean products whose operands hold no false value: every output value is true
     const bool walk = SR::id != SPGEMM_OR_AND_BOOL || vals_zero == nullptr || *vals_zero != 0;
     const T init = walk ? SR::out(SR::zero()) : T(1);
-    for (int x = lane; x < L2W; x += GS) l2[x] = 0u;
+    for (int x = lane; x < nwords_max; x += GS) l2[x] = 0u;
     for (int x = lane; x < L1W; x += GS) l1[x] = 0u;
     gsync<GS>();
     for (int64_t w = (int64_t)blockIdx.x * NG + g; w < count; w += (int64_t)gridDim.x * NG) {
@@ -215,6 +224,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 4 : 1) k_block_tier(Item
         const int m = (int)pr->A.m;   // <= BLOCK_TIER_MAX_ROWS
         const int nw = (m + 31) >> 5;
         const bool one_chunk = be - bs <= GS;
+        const bool b_one = pr->B.num == nullptr;   // a merge: the selector's ones
         int ns = 0, total = 0;
         // 1. marks
         for (int64_t b0 = bs; b0 < be; b0 += GS) {
@@ -307,7 +317,7 @@ __global__ void __launch_bounds__(BLOCK, BLOCK == 512 ? 4 : 1) k_block_tier(Item
                         const uint32_t wv = l2[wd];
                         const uint32_t bit = 1u << (r & 31);
                         const int rank = wp[wd] + __popc(wv & (bit - 1u));
-                        red_out<SR>(Cv, out0 + rank, SR::mul(a, b));
+                        red_out<SR>(Cv, out0 + rank, b_one ? mul_by<SR>(a, b, true) : SR::mul(a, b));
                     });
                     if (!one_chunk) gsync<GS>();
                 }
@@ -326,20 +336,17 @@ void run_bt(const Lanes& st, const Items& it, const int2* list, int64_t count, i
             int32_t* Cir, typename SR::T* Cv, const int* vals_zero) {
     if (count <= 0) return;
     constexpr int NG = BLOCK / GS;
-    const size_t smem = BtLayout<SR, GS>::group * NG;
+    const int nw = (int)ceil_div64(std::max<int64_t>(it.max_m, 1), 32 * 32) * 32;   // <= L2W
+    const size_t smem = BtLayout<SR, GS>(nw).group * NG;
     auto kern = k_block_tier<SR, GS, BLOCK>;
-    static bool attr = false;   // per process: the limit belongs to the kernel
-    if (!attr) {
-        cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        attr = true;
-    }
+    smem_at_least((const void*)kern, smem);
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BLOCK, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         per_sm = 1;
     }
     const int grid = (int)std::min<int64_t>(ceil_div64(count, NG), (int64_t)per_sm * sm_count());
-    kern<<<grid, BLOCK, smem, st.next()>>>(it, list, count, nnz_item, Coff, Cir, Cv, vals_zero);
+    kern<<<grid, BLOCK, smem, st.next()>>>(it, list, count, nnz_item, Coff, Cir, Cv, vals_zero, nw);
     note_launch();
 }
 

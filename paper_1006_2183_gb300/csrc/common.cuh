@@ -68,6 +68,16 @@ struct PTI64 {
     __device__ static T out(Acc a) { return (T)a; }
 };
 
+// a (x) b, where `one` says that b is the semiring's one: plus-times then leaves a as it is
+// without a multiplication (the merges' selector; FP64 multiplies at two lanes per clock)
+template <class SR>
+__device__ __forceinline__ typename SR::Acc mul_by(typename SR::T a, typename SR::T b, bool one) {
+    if constexpr (SR::id == SPGEMM_PLUS_TIMES_F64 || SR::id == SPGEMM_PLUS_TIMES_I64) {
+        if (one) return (typename SR::Acc)a;
+    }
+    return SR::mul(a, b);
+}
+
 // ------------------------------------------------------------------ matrix view
 // CSC when jc == nullptr; DCSC (Section 2.3) otherwise: cp[p], jc[p] describe the
 // p-th nonempty column, aux indexes chunks of `chunk` columns.
@@ -326,23 +336,6 @@ __device__ __forceinline__ void red_out(typename SR::T* Cv, int64_t pos, typenam
     } else {
         SR::atomic_add(Cv + pos, v);   // double add; float min through integer min / max
     }
-}
-
-// bitmap[wd] |= bit for every lane with wd >= 0; lanes that hit the same word
-// combine their bits first, so each run of equal words takes one shared atomic.
-// Called by all 32 lanes of the warp.
-__device__ __forceinline__ void or_bits_warp(uint32_t* bitmap, int wd, uint32_t bit) {
-    const int lane = threadIdx.x & 31;
-    const int wprev = __shfl_up_sync(0xffffffffu, wd, 1);
-    const bool head = lane == 0 || wprev != wd;
-    uint32_t acc = bit;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t b2 = __shfl_down_sync(0xffffffffu, acc, o);
-        const int w2 = __shfl_down_sync(0xffffffffu, wd, o);
-        if (lane + o < 32 && w2 == wd) acc |= b2;
-    }
-    if (wd >= 0 && head) atomicOr(&bitmap[wd], acc);
 }
 
 __host__ __device__ __forceinline__ int64_t ceil_div64(int64_t a, int64_t b) { return (a + b - 1) / b; }

@@ -97,7 +97,7 @@ Lanes::~Lanes() {
 // Raises a kernel's dynamic shared-memory limit on the current device to at least
 // `bytes`; never lowers it (the limit belongs to the kernel, whichever launcher
 // asks).  A refused request is not remembered, so the launch reports the error.
-static void smem_at_least(const void* fn, size_t bytes) {
+void smem_at_least(const void* fn, size_t bytes) {
     static std::mutex mu;
     static std::map<std::pair<int, const void*>, size_t> limit;
     int dev = 0;

@@ -268,6 +268,8 @@ void launch_tier_stats(cudaStream_t st, const Items& it, const uint8_t* bin, con
                        const int64_t* flops, const int64_t* nnz_item, unsigned long long* out);
 
 
+// raises a kernel's dynamic shared-memory limit on the current device to at least `bytes`
+void smem_at_least(const void* fn, size_t bytes);
 // streaming multiprocessors of the current device (queried once per device)
 int sm_count();
 

@@ -42,16 +42,6 @@ __device__ __forceinline__ V shflg(V x, int src) {
     else return __shfl_sync(0xffffffffu, x, src, G);
 }
 
-// a (x) b, where `one` says that b is the semiring's one: plus-times then leaves a as it is
-// without a multiplication (the merges' selector; FP64 multiplies at two lanes per clock)
-template <class SR>
-__device__ __forceinline__ typename SR::Acc mul_by(typename SR::T a, typename SR::T b, bool one) {
-    if constexpr (SR::id == SPGEMM_PLUS_TIMES_F64 || SR::id == SPGEMM_PLUS_TIMES_I64) {
-        if (one) return (typename SR::Acc)a;
-    }
-    return SR::mul(a, b);
-}
-
 // Ascending bitonic sort of the N = G K keys of a group (element i = K lane + r).
 template <int G, int K>
 __device__ __forceinline__ void sort_keys(uint32_t (&key)[K], int lane) {
