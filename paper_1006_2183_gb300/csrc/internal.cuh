@@ -178,6 +178,8 @@ spgemm_status_t check_handles(spgemm_ctx* ctx, const std::vector<spgemm_mat*>& m
 spgemm_status_t transpose_csc(spgemm_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const int64_t* cp,
                               const int32_t* ir, const void* num, size_t w, spgemm_mat_t out_handle);
 spgemm_status_t make_dcsc(spgemm_ctx* ctx, const spgemm_mat* csc, bool aux, spgemm_mat* out);
+// col[t] = the column of entry t of a CSC array
+void launch_expand_cols(cudaStream_t st, const int64_t* cp, int64_t n, int64_t nnz, int32_t* col);
 size_t radix_tmp_bytes(int64_t n);
 void radix_sort_pairs(cudaStream_t st, uint32_t* k0, uint32_t* v0, uint32_t* k1, uint32_t* v1, int64_t n, int bits,
                       void* tmp, bool* in_second);
