@@ -503,7 +503,7 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
     E->it.acl = any_dcsc ? (int32_t*)(base + o_acl) : nullptr;
     E->it.max_m = 0;
     for (auto& pr : E->hprods) E->it.max_m = std::max<int64_t>(E->it.max_m, pr.A.m);
-    // the sort tier takes the columns that its keys hold (512 products up to 2^23 rows);
+    // the sort tier takes the columns that its keys hold (1024 products up to 2^22 rows);
     // where the block tier can take the columns of 257 .. 512 products it is as fast for
     // them and faster for the merges' long runs (R-MAT 18, 16 x 16 SUMMA, FP64: 26.8 ms
     // with the line at 256 products, 27.0 at 128, 28.9 at 512)

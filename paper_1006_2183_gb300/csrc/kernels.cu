@@ -2,7 +2,7 @@
 // formulation, Section 2.1; accumulation in the spirit of the sparse
 // accumulator of Section 3.3), organised in accumulator tiers chosen per
 // output column from cap = min(flops, m):
-//   * up to 512 products: sorted in the registers of 8 to 32 lanes (sorttier.cu),
+//   * up to 1024 products: sorted in the registers of 8 to 32 lanes (sorttier.cu),
 //   * warp-wide shared-memory hash tables (short columns of many products),
 //   * CTA-wide shared-memory hash tables (medium columns),
 //   * the slab tier (long columns): row slabs, each counted through a row bitmap in
@@ -114,7 +114,7 @@ __host__ __device__ __forceinline__ int bin_of(int64_t flops, int64_t cap, int w
                                               int sort_max) {
     if (cap <= 0) return 0;
     if (flops <= TINY_MAX) return BIN_SORT0;
-    if (cap <= warp_max && flops <= sort_max) {
+    if (flops <= sort_max && cap <= (flops <= 512 ? warp_max : block_max)) {
         int b = BIN_SORT0 + 1;
         for (int64_t t = 2 * TINY_MAX; t < flops; t <<= 1) ++b;
         return b;

@@ -15,12 +15,12 @@ namespace sg {
 
 // Column tiers.  An item's capacity bound is cap = min(flops, m) >= nnz of its output.
 //   bin 0                          : cap == 0 (empty output column)
-//   bins BIN_SORT0 .. +NSORT-1     : at most 16, 32 .. 512 products (sort tier, up to
+//   bins BIN_SORT0 .. +NSORT-1     : at most 16, 32 .. 1024 products (sort tier, up to
 //                                    TierCfg::sort_max products; 16 products always)
 //   bins BIN_WARP0 .. +NWARP-1     : warp-wide hash tables of 64 .. 1024 slots (>= 2 cap)
 //   bins BIN_BLK0 .. +NBLK-1       : CTA-wide hash tables of 2048 .. 8192 slots (>= 2 cap)
 //   bin NBIN-1                     : slab tier (long columns cut into row slabs)
-constexpr int NSORT = 6;
+constexpr int NSORT = 7;
 constexpr int NWARP = 5;
 constexpr int NBLK = 3;
 constexpr int NBIN = 1 + NSORT + NWARP + NBLK + 1;
@@ -52,8 +52,9 @@ static_assert(NBIN + 1 <= CTR_STRIDE, "a copy keeps to its lines");
 struct TierCfg {
     int warp_max;     // cap <= warp_max -> warp tables (<= 512)
     int block_max;    // cap <= block_max -> CTA tables (<= 4096)
-    int sort_max = 0; // columns of at most this many products (and cap <= warp_max) go to the
-                      // sort tier: sort_max_products(rows), less where another tier is faster
+    int sort_max = 0; // columns of at most this many products (and cap <= warp_max, or
+                      // <= block_max beyond 512 products) go to the sort tier:
+                      // sort_max_products(rows), less where another tier is faster
     int dense_rows;   // RB, most rows of one slab (bitmap bits in shared memory)
     int part_flops;   // target flops per slab of a long column
 };
@@ -115,7 +116,7 @@ constexpr int BLOCK_TIER_MAX_ROWS = 32768;
 // a key is the row above log2(products) bits of slot, and all ones marks an empty slot.
 // 0: the rows leave no room even for 16 products.
 inline int sort_max_products(int64_t max_m) {
-    for (int n = 512, sb = 9; n >= TINY_MAX; n /= 2, --sb)
+    for (int n = 1024, sb = 10; n >= TINY_MAX; n /= 2, --sb)
         if (max_m <= (int64_t(1) << (32 - sb)) - 1) return n;
     return 0;
 }

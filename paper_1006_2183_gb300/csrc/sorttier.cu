@@ -1,4 +1,4 @@
-// Sort tier: columns of at most 512 products (TierCfg::sort_max), whatever the number
+// Sort tier: columns of at most 1024 products (TierCfg::sort_max), whatever the number
 // of rows that the keys hold.  A group of G lanes takes one output column
 // C(:,j) = (+)_{k in B(:,j)} A(:,k) (x) B(k,j) (Section 2.1), N = G K products at most:
 //   1. product p goes to lane p mod G as the key (row << log2 N) | p, its value to slot
@@ -13,11 +13,13 @@
 //   4. rows and values are put in order in shared memory and stored coalesced.
 // No atomics, no tables to fill and empty, and several columns per warp share the
 // latency of the loads that a column starts with.  The counting form sorts rows alone.
-// Bound by instruction issue and the FP64 pipe, not by memory.  Against one warp per
-// column with 32-lane networks and, for operands of many rows, shared-memory hash tables
-// whose entries were then sorted: R*(A*P) on 128^3 FP64, 262,144 columns of 50 to 60
-// products and as many of about 32, 736 -> 310 us (counting 294 -> 168 us); 20 int64 pairs,
-// columns of up to 512 products, 1.25 -> 0.41 ms (counting 0.24 -> 0.18 ms).
+// Bound by instruction issue and the FP64 pipe, not by memory: what the registers and the
+// slots leave resident decides (the caps below).  Against one warp per column with 32-lane
+// networks and, for operands of many rows, shared-memory hash tables whose entries were
+// then sorted: R*(A*P) on 128^3 FP64, 262,144 columns of 50 to 60 products and as many of
+// about 32, 736 -> 265 us (counting 294 -> 155 us); 20 int64 pairs, columns of up to 1024
+// products, 1.35 -> 0.40 ms (counting 0.30 -> 0.27 ms); the columns of 513 to 1024 products
+// of a scale-20 R-MAT square FP64, 1456 -> 361 us (counting 230 -> 218 us).
 #include <algorithm>
 
 #include "internal.cuh"
@@ -26,8 +28,15 @@
 namespace sg {
 namespace {
 
-// threads per CTA: 8 warps, 4 where a column's slots take 6 KB
-constexpr int st_block(int K) { return K == 16 ? 128 : 256; }
+// threads per CTA: 8 warps, fewer where a column's slots take 7 or 14 KB
+constexpr int st_block(int K) { return K == 32 ? 64 : K == 16 ? 128 : 256; }
+// CTAs per SM that the registers are held to: the most that the slots leave room for
+// (numeric; at K = 8 one less, where a sixth spills: 693 -> 675 us for the 8-lane network
+// of that product and two merges) or that the keys of the counting network allow
+constexpr int st_min_blocks(int K, bool num) {
+    if (num) return K >= 16 ? 8 : K == 8 ? 5 : 6;
+    return K == 32 ? 12 : K == 16 ? 8 : 5;
+}
 
 template <int G, class V>
 __device__ __forceinline__ V shflg(V x, int src) {
@@ -37,20 +46,20 @@ __device__ __forceinline__ V shflg(V x, int src) {
 
 // NUM: rows and values to C (Coff as for launch_block_tier); otherwise counts to nnz_item.
 template <class SR, int G, int K, bool NUM>
-__global__ void __launch_bounds__(st_block(K)) k_sort(Items it, const int2* __restrict__ list, int64_t count,
-                                                   int64_t* __restrict__ nnz_item, const int64_t* __restrict__ Coff,
-                                                   int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv,
-                                                   const int* __restrict__ vals_zero) {
+__global__ void __launch_bounds__(st_block(K), st_min_blocks(K, NUM))
+k_sort(Items it, const int2* __restrict__ list, int64_t count, int64_t* __restrict__ nnz_item,
+       const int64_t* __restrict__ Coff, int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv,
+       const int* __restrict__ vals_zero) {
     using T = typename SR::T;
     using Acc = typename SR::Acc;
     constexpr int N = G * K, SB = ilog2(N), NG = st_block(K) / G, SPAN = st_span<N>();
     constexpr uint32_t NONE = 0xffffffffu;
     constexpr uint32_t NOROW = NONE >> SB;   // no stored row (the host bounds the rows)
     __shared__ Acc s_val[NUM ? NG * SPAN : 1];
-    __shared__ int32_t s_row[NUM ? NG * SPAN : 1];
+    __shared__ uint32_t s_key[NG * SPAN];
     const int lane = threadIdx.x & (G - 1), grp = threadIdx.x / G;
     Acc* sv = s_val + (NUM ? grp * SPAN : 0);
-    int32_t* sr = s_row + (NUM ? grp * SPAN : 0);
+    uint32_t* sk = s_key + grp * SPAN;
     // boolean products whose operands hold no false value: every output value is true
     const bool walk = NUM && (SR::id != SPGEMM_OR_AND_BOOL || vals_zero == nullptr || *vals_zero != 0);
     // the groups of a warp go round together (their shuffles name the whole warp)
@@ -69,10 +78,11 @@ __global__ void __launch_bounds__(st_block(K)) k_sort(Items it, const int2* __re
         }
         const uint32_t m = (uint32_t)pr->A.m;
         const bool b_one = __all_sync(0xffffffffu, pr->B.num == nullptr);   // of every group of the warp
-        uint32_t key[K];
-#pragma unroll
-        for (int r = 0; r < K; ++r) key[r] = NONE;
-        // 1. products: the entries of B(:,j) G at a time (the bin bounds their products by N)
+        // 1. products: the entries of B(:,j) G at a time (the bin bounds their products by N),
+        //    U products per lane in flight; product p to slot p (however many entries they come
+        //    from: keys kept in registers made every G entries pay for all K slots, 499 us
+        //    for the 361 above)
+        constexpr int U = K == 2 ? 1 : K <= 8 ? 2 : 4;
         int base = 0;
         for (int64_t b0 = bs; __any_sync(0xffffffffu, b0 < be && base < N); b0 += G) {
             const int64_t t = b0 + lane;
@@ -88,29 +98,47 @@ __global__ void __launch_bounds__(st_block(K)) k_sort(Items it, const int2* __re
                 if (walk) bv = load_val<SR>(pr->B, t);
             }
             const int inc = scan_g<G>(len, lane);
-            const int tot = __shfl_sync(0xffffffffu, inc, G - 1, G);
-            a0 -= inc - len;   // product p of the chunk is at a0 + p of its entry
+            const int tot = min(__shfl_sync(0xffffffffu, inc, G - 1, G), N - base);
+            a0 -= inc - len;   // product q of the chunk is at a0 + q of its entry
+            for (int q0 = lane; __any_sync(0xffffffffu, q0 < tot); q0 += G * U) {
+                int32_t row[U];
+                T av[U], bvs[U];
 #pragma unroll
-            for (int r = 0; r < K; ++r) {
-                const int p = r * G + lane - base;   // the slot's product within this chunk
-                if (!__any_sync(0xffffffffu, p >= 0 && p < tot)) continue;
-                int src = 0;                         // entries that end at or before product p
+                for (int i = 0; i < U; ++i) {
+                    const int q = q0 + i * G;
+                    int src = 0;                         // entries that end at or before product q
 #pragma unroll
-                for (int st = G / 2; st > 0; st >>= 1)
-                    if (__shfl_sync(0xffffffffu, inc, src + st - 1, G) <= p) src += st;
-                const int64_t as = __shfl_sync(0xffffffffu, a0, src, G);
-                T bvs = T(0);
-                if constexpr (NUM) bvs = shflg<G>(bv, src);
-                if (p >= 0 && p < tot) {
-                    const int32_t row = __ldg(pr->A.ir + as + p);
-                    if ((uint32_t)row < m) {   // else malformed input: skipped
-                        key[r] = ((uint32_t)row << SB) | (uint32_t)(r * G + lane);
-                        if constexpr (NUM)
-                            sv[st_ph(r * G + lane)] = walk ? mul_by<SR>(load_val<SR>(pr->A, as + p), bvs, b_one) : SR::one();
+                    for (int st = G / 2; st > 0; st >>= 1)
+                        if (__shfl_sync(0xffffffffu, inc, src + st - 1, G) <= q) src += st;
+                    const int64_t as = __shfl_sync(0xffffffffu, a0, src, G);
+                    bvs[i] = T(0);
+                    av[i] = T(0);
+                    if constexpr (NUM) bvs[i] = shflg<G>(bv, src);
+                    row[i] = -1;
+                    if (q < tot) {
+                        row[i] = __ldg(pr->A.ir + as + q);
+                        if (walk) av[i] = load_val<SR>(pr->A, as + q);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < U; ++i) {
+                    const int q = q0 + i * G;
+                    if (q < tot) {
+                        const int slot = base + q;
+                        // a row outside A is malformed input: skipped
+                        sk[st_ph(slot)] = (uint32_t)row[i] < m ? ((uint32_t)row[i] << SB) | (uint32_t)slot : NONE;
+                        if constexpr (NUM) sv[st_ph(slot)] = walk ? mul_by<SR>(av[i], bvs[i], b_one) : SR::one();
                     }
                 }
             }
             base += tot;
+        }
+        __syncwarp();
+        uint32_t key[K];
+#pragma unroll
+        for (int r = 0; r < K; ++r) {
+            const int i = r * G + lane;
+            key[r] = i < base ? sk[st_ph(i)] : NONE;
         }
         // 2. order
         sort_keys<G, K>(key, lane);
@@ -130,20 +158,29 @@ __global__ void __launch_bounds__(st_block(K)) k_sort(Items it, const int2* __re
         const int cnt = __shfl_sync(0xffffffffu, inc, G - 1, G);
         if constexpr (!NUM) {
             if (act && lane == 0) nnz_item[u] = cnt;
+            __syncwarp();   // the slots are free for the next column
         } else {
             __syncwarp();
-            Acc v[K];
+            // a run's sum goes to the slot of its last element, which no other lane touches
+            Acc acc = SR::zero();
+            uint32_t head = NONE;   // the last element of the lane's first run, if it ends here
 #pragma unroll
-            for (int r = 0; r < K; ++r) v[r] = key[r] != NONE ? sv[st_ph((int)(key[r] & (N - 1)))] : SR::zero();
-#pragma unroll
-            for (int r = 1; r < K; ++r) {
-                const bool same = key[r] != NONE && (key[r] >> SB) == (key[r - 1] >> SB);
-                if (__any_sync(0xffffffffu, same)) v[r] = same ? SR::add(v[r - 1], v[r]) : v[r];
+            for (int r = 0; r < K; ++r) {
+                Acc* slot = sv + st_ph((int)(key[r] & (N - 1)));
+                const Acc x = key[r] != NONE ? *slot : SR::zero();
+                bool same = false;
+                if (r > 0) same = key[r] != NONE && (key[r] >> SB) == (key[r > 0 ? r - 1 : 0] >> SB);
+                if (r > 0 && __any_sync(0xffffffffu, same)) acc = same ? SR::add(acc, x) : x;
+                else acc = x;
+                if ((end >> r) & 1u) {
+                    *slot = acc;
+                    if ((key[r] >> SB) == first) head = key[r];
+                }
             }
             // a run that continues the lane before's last one takes that lane's sum
             const bool cont = key[0] != NONE && before == first;
             if (__any_sync(0xffffffffu, cont)) {
-                Acc s = v[K - 1];
+                Acc s = acc;
                 int through = cont && last == first && key[K - 1] != NONE;   // one run, from the lane before's
 #pragma unroll
                 for (int d = 1; d < G; d <<= 1) {
@@ -155,22 +192,16 @@ __global__ void __launch_bounds__(st_block(K)) k_sort(Items it, const int2* __re
                     }
                 }
                 const Acc carry = shflg<G>(s, lane > 0 ? lane - 1 : 0);
-#pragma unroll
-                for (int r = 0; r < K; ++r) {
-                    const bool take = cont && ((end >> r) & 1u) && (key[r] >> SB) == first;
-                    if (__any_sync(0xffffffffu, take)) v[r] = take ? SR::add(carry, v[r]) : v[r];
+                if (cont && head != NONE) {
+                    Acc* slot = sv + st_ph((int)(head & (N - 1)));
+                    *slot = SR::add(carry, *slot);
                 }
             }
-            __syncwarp();   // every value is out of its slot
-            // 4. the column in order, then coalesced stores
+            // 4. the last elements of the runs in order, then coalesced stores
             int pos = inc - c;
 #pragma unroll
             for (int r = 0; r < K; ++r)
-                if ((end >> r) & 1u) {
-                    sr[st_ph(pos)] = (int32_t)(key[r] >> SB);
-                    sv[st_ph(pos)] = v[r];
-                    ++pos;
-                }
+                if ((end >> r) & 1u) sk[st_ph(pos++)] = key[r];
             __syncwarp();
             if (act) {
                 const int64_t out0 = __ldg(Coff + u);
@@ -181,8 +212,9 @@ __global__ void __launch_bounds__(st_block(K)) k_sort(Items it, const int2* __re
                 if (cnt <= capn) {
                     const int32_t rb = out_row_base(pr, e.y);
                     for (int i = lane; i < cnt; i += G) {
-                        __stcs(Cir + out0 + i, sr[st_ph(i)] + rb);
-                        Cv[out0 + i] = SR::out(sv[st_ph(i)]);
+                        const uint32_t k = sk[st_ph(i)];
+                        __stcs(Cir + out0 + i, (int32_t)(k >> SB) + rb);
+                        Cv[out0 + i] = SR::out(sv[st_ph((int)(k & (N - 1)))]);
                     }
                 }
             }
@@ -210,6 +242,7 @@ void run_bins(const Lanes& st, const Items& it, const int2* list, const int64_t*
     run<SR, 16, 8, NUM>(st, it, list + off[S + 3], cnt[S + 3], nnz_item, Coff, Cir, Cv, vz);
     run<SR, 32, 8, NUM>(st, it, list + off[S + 4], cnt[S + 4], nnz_item, Coff, Cir, Cv, vz);
     run<SR, 32, 16, NUM>(st, it, list + off[S + 5], cnt[S + 5], nnz_item, Coff, Cir, Cv, vz);
+    run<SR, 32, 32, NUM>(st, it, list + off[S + 6], cnt[S + 6], nnz_item, Coff, Cir, Cv, vz);
 }
 
 }  // namespace
