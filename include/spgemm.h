@@ -99,8 +99,10 @@ typedef struct {
                                  them (SPGEMM_ERR_UNSUPPORTED otherwise).              */
     int summa_merge_every;    /* staged mode: merge after this many stages (0 = after
                                  the last stage, the paper's buffered triples).        */
-    int warp_max_flops;       /* columns with flops <= this use warp-wide hash tables  */
-    int block_max_flops;      /* columns with flops <= this use CTA-wide hash tables;
+    int warp_max_flops;       /* columns with flops <= this (at most 512) are sorted in
+                                 registers or use warp-wide hash tables                 */
+    int block_max_flops;      /* columns with flops <= this are sorted (up to 1024
+                                 products) or use CTA-wide hash tables;
                                  longer columns (the slab tier) are cut into row slabs,
                                  each counted and then accumulated by one CTA (at most
                                  4096).  -1 (default) = automatic: 4096 for operands of
@@ -118,7 +120,7 @@ typedef struct {
                                  bitmap lives in shared memory), rounded to a
                                  multiple of 32 and clamped to [4096, 2^20]; raised
                                  where a column would need more than 64 slabs.
-                                 0 = default (2^19).  A long column of more than
+                                 0 = default (327680).  A long column of more than
                                  64 * (2^20 - 32) rows is SPGEMM_ERR_UNSUPPORTED.   */
     int check_inputs;         /* 1 (default): every product call first checks, on the
                                  device, each borrowed CSC/CSR operand it has not checked
@@ -199,10 +201,10 @@ spgemm_status_t spgemm_mat_destroy(spgemm_mat_t mat);
 #define SPGEMM_NPHASE 8
 typedef enum {
     SPGEMM_PHASE_ANALYZE = 0,        /* flops per column, binning, dense work items     */
-    SPGEMM_PHASE_SYMBOLIC_HASH = 1,  /* symbolic pass, hash-table tiers                 */
+    SPGEMM_PHASE_SYMBOLIC_HASH = 1,  /* symbolic pass, short columns (sort, hash)       */
     SPGEMM_PHASE_SYMBOLIC_DENSE = 2, /* symbolic pass, long columns (ranges / dense)    */
     SPGEMM_PHASE_SCAN = 3,           /* column pointers of C                            */
-    SPGEMM_PHASE_NUMERIC_HASH = 4,   /* numeric pass, hash-table tiers                  */
+    SPGEMM_PHASE_NUMERIC_HASH = 4,   /* numeric pass, short columns (sort, hash)        */
     SPGEMM_PHASE_NUMERIC_DENSE = 5,  /* numeric pass, long columns (ranges / dense)     */
     SPGEMM_PHASE_PREDICT = 6,        /* predictor inference + overflow repair           */
     SPGEMM_PHASE_MERGE = 7           /* SUMMA stage merge                               */
@@ -242,8 +244,8 @@ spgemm_status_t spgemm_numeric(spgemm_plan_t plan, spgemm_mat_t* C);
 spgemm_status_t spgemm_plan_stats(spgemm_plan_t plan, int64_t* flops, int64_t* nnz_C, int64_t* tier_cols4,
                                   int64_t* overflow_cols);
 /* Per-tier totals of the plan: columns, flops, nnz(C) (after the symbolic pass,
- * else -1) and nnz of the B columns, for tiers {empty, warp hash, CTA hash,
- * dense}; any pointer may be NULL. */
+ * else -1) and nnz of the B columns, for tiers {empty, up to warp_max_flops, up to
+ * block_max_flops, long columns}; any pointer may be NULL. */
 spgemm_status_t spgemm_plan_tier_stats(spgemm_plan_t plan, int64_t* cols4, int64_t* flops4, int64_t* nnz4,
                                        int64_t* bnnz4);
 spgemm_status_t spgemm_plan_destroy(spgemm_plan_t plan);

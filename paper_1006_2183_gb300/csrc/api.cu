@@ -505,8 +505,8 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
     for (auto& pr : E->hprods) E->it.max_m = std::max<int64_t>(E->it.max_m, pr.A.m);
     // the sort tier takes the columns that its keys hold (1024 products up to 2^22 rows);
     // where the block tier can take the columns of 257 .. 512 products it is as fast for
-    // them and faster for the merges' long runs (R-MAT 18, 16 x 16 SUMMA, FP64: 26.8 ms
-    // with the line at 256 products, 27.0 at 128, 28.9 at 512)
+    // them and faster for the merges' long runs (R-MAT 18, 16 x 16 SUMMA, FP64: 21.3 ms
+    // with the line at 256 products, 21.4 at 128, 22.7 at 512)
     E->cfg.sort_max = sort_max_products(E->it.max_m);
     if (E->it.max_m <= BLOCK_TIER_MAX_ROWS) E->cfg.sort_max = std::min(E->cfg.sort_max, 256);
     uint64_t* sketch = nullptr;
@@ -822,12 +822,8 @@ spgemm_status_t spgemm_plan_stats(spgemm_plan_t P, int64_t* flops, int64_t* nnz_
     if (flops) *flops = E.flops_total;
     if (nnz_C) *nnz_C = E.nnz_total;
     if (tiers4) {
-        tiers4[0] = E.bin_cnt[0];
-        tiers4[1] = 0;
-        tiers4[2] = 0;
-        for (int b = BIN_SORT0; b < BIN_BLK0; ++b) tiers4[1] += E.bin_cnt[b];
-        for (int b = BIN_BLK0; b < BIN_DENSE; ++b) tiers4[2] += E.bin_cnt[b];
-        tiers4[3] = E.bin_cnt[BIN_DENSE];
+        for (int t = 0; t < 4; ++t) tiers4[t] = 0;
+        for (int b = 0; b < NBIN; ++b) tiers4[tier_of_bin(b)] += E.bin_cnt[b];
     }
     if (overflow) *overflow = E.overflow_items;
     return SPGEMM_OK;

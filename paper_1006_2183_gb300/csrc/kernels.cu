@@ -2060,7 +2060,7 @@ __global__ void k_tier_stats(Items it, const uint8_t* __restrict__ bin, const in
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < it.nitems;
          u += (int64_t)gridDim.x * blockDim.x) {
         int b = bin[u];
-        int t = b == 0 ? 0 : (b < BIN_BLK0 ? 1 : (b < BIN_DENSE ? 2 : 3));
+        int t = tier_of_bin(b);
         int prod = item_prod[u];
         const Prod* pr = it.prods + prod;
         int64_t p = u - __ldg(it.item_base + prod);

@@ -28,6 +28,11 @@ constexpr int BIN_SORT0 = 1;
 constexpr int BIN_WARP0 = BIN_SORT0 + NSORT;
 constexpr int BIN_BLK0 = BIN_WARP0 + NWARP;
 constexpr int BIN_DENSE = NBIN - 1;
+// Tier of a bin in the plan's statistics: 0 empty, 1 up to warp_max_flops, 2 up to
+// block_max_flops, 3 long columns.  The last sort bin holds columns beyond 512 products.
+__host__ __device__ constexpr int tier_of_bin(int b) {
+    return b == 0 ? 0 : b >= BIN_DENSE ? 3 : b >= BIN_BLK0 || b == BIN_WARP0 - 1 ? 2 : 1;
+}
 constexpr int TINY_MAX = 16;
 constexpr int WARP_TBL0 = 64;
 constexpr int BLK_TBL0 = 2048;

@@ -97,3 +97,21 @@ def test_sort_tier_at_the_keys_limits(ctx, m, sr):
             np.testing.assert_allclose(C.vals, R.vals, rtol=0, atol=ATOL)
         else:
             np.testing.assert_array_equal(C.vals, R.vals)
+
+
+@pytest.mark.parametrize("m", [40000, 2 ** 22, 2 ** 25])
+@pytest.mark.parametrize("block_max", [-1, 600, 2048])
+def test_tier_statistics_follow_the_thresholds(ctx, m, block_max):
+    """Which kernel sorts a column does not show in the plan's statistics."""
+    A, B = _operands(m, PT_I64, 0x51)
+    fl = oracle.flops_per_col(A, B)
+    lim = 1024 if block_max < 0 else block_max
+    tier = np.where(fl == 0, 0, np.where(fl <= 512, 1, np.where(fl <= lim, 2, 3)))
+    s = sp()
+    dA, dB = s.Matrix.from_host(ctx, A, PT_I64), s.Matrix.from_host(ctx, B, PT_I64)
+    p = s.spgemm_plan(ctx, dA, dB, PT_I64, s.default_opts(block_max_flops=block_max))
+    s.spgemm_symbolic(p)
+    want = np.bincount(tier, minlength=4).tolist()
+    assert list(p.stats()["tiers"]) == want
+    cols, flops = list(p.tier_stats()["cols"]), list(p.tier_stats()["flops"])
+    assert cols == want and flops == [int(fl[tier == i].sum()) for i in range(4)]
