@@ -414,22 +414,35 @@ __device__ __forceinline__ void bin_offsets(const unsigned long long* cnt, int r
     __syncthreads();
 }
 
+// Where one thread's entry of bin b (<= 0: not listed) goes among the CTA's entries of that
+// bin, which s_n counts.  Whole warps call it.
+__device__ __forceinline__ int bin_rank(int b, int* s_n) {
+    const unsigned peers = __match_any_sync(0xffffffffu, b);
+    const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
+    int at = 0;
+    if (b > 0 && lane == leader) at = atomicAdd(&s_n[b], __popc(peers));
+    return __shfl_sync(0xffffffffu, at, leader) + __popc(peers & ((1u << lane) - 1));
+}
+
+// Where the CTA's entries of every bin start in the lists: one global addition per bin.  All
+// threads call it, after a barrier; ends with one.
+__device__ __forceinline__ void bin_bases(unsigned long long* cursor, const int64_t* s_off, const int* s_n,
+                                          int64_t* s_base) {
+    if (threadIdx.x < NBIN && threadIdx.x > 0 && s_n[threadIdx.x] > 0)
+        s_base[threadIdx.x] = s_off[threadIdx.x] +
+                              (int64_t)atomicAdd(cursor + threadIdx.x, (unsigned long long)s_n[threadIdx.x]);
+    __syncthreads();
+}
+
 // One bin per thread (b <= 0: not listed): its place in the list of bin b, whose entries
 // before this CTA's come from one global addition per bin.  All threads call it.
 __device__ __forceinline__ int64_t list_place(int b, unsigned long long* cursor, const int64_t* s_off, int* s_n,
                                               int64_t* s_base) {
     if (threadIdx.x < NBIN) s_n[threadIdx.x] = 0;
     __syncthreads();
-    const unsigned peers = __match_any_sync(0xffffffffu, b);
-    const int lane = threadIdx.x & 31, leader = __ffs(peers) - 1;
-    int at = 0;
-    if (b > 0 && lane == leader) at = atomicAdd(&s_n[b], __popc(peers));
-    at = __shfl_sync(0xffffffffu, at, leader) + __popc(peers & ((1u << lane) - 1));
+    const int at = bin_rank(b, s_n);
     __syncthreads();
-    if (threadIdx.x < NBIN && threadIdx.x > 0 && s_n[threadIdx.x] > 0)
-        s_base[threadIdx.x] = s_off[threadIdx.x] +
-                              (int64_t)atomicAdd(cursor + threadIdx.x, (unsigned long long)s_n[threadIdx.x]);
-    __syncthreads();
+    bin_bases(cursor, s_off, s_n, s_base);
     return b > 0 ? s_base[b] + at : 0;
 }
 
@@ -2109,7 +2122,10 @@ __device__ __forceinline__ long long block_excl_scan64(long long v, long long* w
 // The end of the counting pass was five launches, two uploads and a memset: three scan
 // launches, the bins from the counts (every thread adding to the same shared counters, 15 us
 // for 4,096 columns), their offsets through the host, and the lists.  It is one launch up to
-// 4,096 columns (11 us) and two up to 8 million: ER 4096^2 flat, a whole call, 137 -> 95 us.
+// 4,096 columns (9.5 us) and two up to 8 million: ER 4096^2 flat, a whole call, 137 -> 95 us.
+// The lists take one round for a thread's four items, whose places in a warp stay close
+// together: four rounds, one item each, took 11.2 us there and put every fourth column of a
+// tile after one another (R*(A*P) on 128^3, a whole call, 646 against 626 us).
 // What the scan of the exact counts does besides: the numeric bin of every item (hash tables
 // need only 2 nnz slots, not 2 min(flops, m); slab-tier and empty items get bin 0, not
 // listed), the bins' counts, and their lists.
@@ -2217,31 +2233,37 @@ __global__ void __launch_bounds__(SCAN_BLOCK) k_scan_apply(const int64_t* __rest
         if (base + i < n) out[base + i + 1] = ex;
     }
     if constexpr (BINS) {
-        int b[SCAN_ITEMS];
-        if (gridDim.x == 1) {
-            if (threadIdx.x < NBIN) s_n[threadIdx.x] = 0;
-            __syncthreads();
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; ++i) {
-                b[i] = base + i < n ? numeric_bin(nb, base + i, v[i]) : 0;
-                if (base + i < n) nb.nbin[base + i] = (uint8_t)b[i];
-                count_bin(b[i], s_n);
-            }
-            __syncthreads();
-            if (threadIdx.x < NBIN) nb.cnt[threadIdx.x] = (unsigned long long)s_n[threadIdx.x];
-            __threadfence();
-            __syncthreads();
-        } else {
-#pragma unroll
-            for (int i = 0; i < SCAN_ITEMS; ++i) b[i] = base + i < n ? nb.nbin[base + i] : 0;
-        }
-        bin_offsets(nb.cnt, 1, s_off);
+        const bool single = gridDim.x == 1;
+        int b[SCAN_ITEMS], at[SCAN_ITEMS];
+        if (threadIdx.x < NBIN) s_n[threadIdx.x] = 0;
+        __syncthreads();
 #pragma unroll
         for (int i = 0; i < SCAN_ITEMS; ++i) {
-            const int64_t at = list_place(b[i], nb.cursor, s_off, s_n, s_base);
+            const int64_t u = base + i;
+            b[i] = u >= n ? 0 : single ? numeric_bin(nb, u, v[i]) : nb.nbin[u];
+            if (single && u < n) nb.nbin[u] = (uint8_t)b[i];
+            at[i] = bin_rank(b[i], s_n);
+        }
+        __syncthreads();
+        if (single) {   // the CTA's counts are the counts
+            if (threadIdx.x < 32) {
+                const int t = threadIdx.x, c = t < NBIN ? s_n[t] : 0;
+                const long long inc = warp_incl_scan64(c);
+                if (t < NBIN) {
+                    nb.cnt[t] = (unsigned long long)c;
+                    s_base[t] = inc - c;
+                }
+            }
+            __syncthreads();
+        } else {
+            bin_offsets(nb.cnt, 1, s_off);
+            bin_bases(nb.cursor, s_off, s_n, s_base);
+        }
+#pragma unroll
+        for (int i = 0; i < SCAN_ITEMS; ++i) {
             if (b[i] > 0) {
                 const int prod = nb.item_prod[base + i];
-                nb.list[at] = make_int2(prod, (int)(base + i - __ldg(nb.it.item_base + prod)));
+                nb.list[s_base[b[i]] + at[i]] = make_int2(prod, (int)(base + i - __ldg(nb.it.item_base + prod)));
             }
         }
     }
