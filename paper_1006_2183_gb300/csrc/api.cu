@@ -115,6 +115,7 @@ spgemm_status_t sync_ctx(spgemm_ctx* ctx) {
     const cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e == cudaSuccess) {
         for (const auto& r : ctx->rb_pending) std::memcpy(r.dst, ctx->rb_host + r.off, r.bytes);
+        ctx->uploads.clear();
     }
     ctx->rb_pending.clear();
     ctx->rb_used = ctx->rb_launched = 0;
@@ -154,6 +155,18 @@ spgemm_status_t read_back(spgemm_ctx* ctx, void* dst, const void* src, size_t by
     ctx->rb_used = off + bytes;
     if (ctx->rb_pending.size() - ctx->rb_launched == RB_MAX) SG_TRY(flush_reads(ctx));
     return SPGEMM_OK;
+}
+
+spgemm_status_t upload(spgemm_ctx* ctx, void* dst, std::vector<char>&& bytes) {
+    if (bytes.empty()) return SPGEMM_OK;
+    ctx->uploads.push_back(std::move(bytes));
+    const std::vector<char>& b = ctx->uploads.back();
+    SG_CUDA(ctx, cudaMemcpyAsync(dst, b.data(), b.size(), cudaMemcpyHostToDevice, ctx->stream));
+    return SPGEMM_OK;
+}
+
+spgemm_status_t upload(spgemm_ctx* ctx, void* dst, const void* src, size_t bytes) {
+    return upload(ctx, dst, std::vector<char>((const char*)src, (const char*)src + bytes));
 }
 
 DMat dmat_of(const spgemm_mat* M) {
@@ -224,8 +237,11 @@ spgemm_status_t spgemm_ctx_create(spgemm_ctx_t* out, void* stream, spgemm_alloc_
 
 spgemm_status_t spgemm_ctx_set_stream(spgemm_ctx_t ctx, void* stream) {
     if (!ctx) return SPGEMM_ERR_INVALID_ARG;
-    // a read left in flight by a failed call still writes the mapped buffer on the old stream
-    if (ctx->rb_host && ctx->stream != (cudaStream_t)stream) cudaStreamSynchronize(ctx->stream);
+    // a read left in flight by a failed call still writes the mapped buffer on the old stream,
+    // and its uploads are kept until a wait for that stream
+    if ((ctx->rb_host || !ctx->uploads.empty()) && ctx->stream != (cudaStream_t)stream &&
+        cudaStreamSynchronize(ctx->stream) == cudaSuccess)
+        ctx->uploads.clear();
     ctx->stream = (cudaStream_t)stream;
     return SPGEMM_OK;
 }
@@ -491,8 +507,7 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         std::vector<char> up(up_bytes, 0);
         if (np > 0) std::memcpy(up.data() + o_prods, E->hprods.data(), sizeof(Prod) * np);
         std::memcpy(up.data() + o_base, E->hitem_base.data(), 8 * (np + 1));
-        // from pageable memory: the call returns once the bytes are out of `up`
-        SG_CUDA(ctx, cudaMemcpyAsync(base, up.data(), up_bytes, cudaMemcpyHostToDevice, st));
+        SG_TRY(upload(ctx, base, std::move(up)));
     }
     E->it.prods = dprods;
     E->it.item_base = dbase;
@@ -522,7 +537,7 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
             hb[i + 1] = hb[i] + E->hprods[i].A.n;
             launch_row_sketch(st, E->hprods[i].A, sketch + hb[i]);
         }
-        SG_CUDA(ctx, cudaMemcpyAsync(skbase, hb.data(), 8 * (np + 1), cudaMemcpyHostToDevice, st));
+        SG_TRY(upload(ctx, skbase, hb.data(), 8 * (np + 1)));
     }
     unsigned long long* const cur = E->ctr + CTR_REP * CTR_STRIDE;
     unsigned long long* const slab_ctr = cur + NBIN;
@@ -743,14 +758,14 @@ static spgemm_status_t product_colptr(Engine* E, std::shared_ptr<DevBuf>* cpbuf,
     auto buf = ctx_buf(E->ctx, 8 * (n + 1) + 16);
     if (!buf) return set_err(E->ctx, SPGEMM_ERR_OOM, "colptr");
     int64_t* cb = (int64_t*)buf->p;
-    int64_t hb[2] = {0, n + 1};
+    const int64_t hb[2] = {0, n + 1};
     auto bb = ctx_buf(E->ctx, 16);
     if (!bb) return set_err(E->ctx, SPGEMM_ERR_OOM, "colptr base");
-    SG_CUDA(E->ctx, cudaMemcpyAsync(bb->p, hb, 16, cudaMemcpyHostToDevice, E->ctx->stream));
+    SG_TRY(upload(E->ctx, bb->p, hb, sizeof(hb)));
     Items one = E->it;
     one.nprod = 1;
     launch_colptrs(E->ctx->stream, one, (const int64_t*)bb->p, n + 1, E->Coff, cb);
-    SG_TRY(sync_ctx(E->ctx));   // keeps hb alive until the copy has run
+    SG_TRY(sync_ctx(E->ctx));   // reports what the launch above raised
     *cpbuf = buf;
     *cp = cb;
     return SPGEMM_OK;

@@ -69,9 +69,8 @@ spgemm_status_t finish_outputs(struct spgemm_plan* P) {
         if (!P->out_cp) return set_err(ctx, SPGEMM_ERR_OOM, "batch column pointers");
         int64_t* cp = (int64_t*)P->out_cp->p;
         int64_t* dcb = cp + std::max<int64_t>(total, 1);
-        SG_CUDA(ctx, cudaMemcpyAsync(dcb, P->colbase.data(), 8 * (np + 1), cudaMemcpyHostToDevice, ctx->stream));
+        SG_TRY(upload(ctx, dcb, P->colbase.data(), 8 * (np + 1)));
         launch_colptrs(ctx->stream, E.it, dcb, total, E.Coff, cp);
-        // P->colbase must outlive the copy: it lives with the plan
         return SPGEMM_OK;
     }
     P->out_cp = ctx_buf(ctx, 8 * std::max<int64_t>(total, 1) + 8 * (2 * np + 2));
@@ -79,7 +78,7 @@ spgemm_status_t finish_outputs(struct spgemm_plan* P) {
     int64_t* cp = (int64_t*)P->out_cp->p;
     int64_t* dcb = cp + std::max<int64_t>(total, 1);
     int64_t* doff = dcb + (np + 1);
-    SG_CUDA(ctx, cudaMemcpyAsync(dcb, P->colbase.data(), 8 * (np + 1), cudaMemcpyHostToDevice, ctx->stream));
+    SG_TRY(upload(ctx, dcb, P->colbase.data(), 8 * (np + 1)));
     launch_colptrs(ctx->stream, E.it, dcb, total, E.Coff, cp);
     launch_gather_offsets(ctx->stream, E.Coff, E.it.item_base, np, doff);
     P->outoff.assign(np + 1, 0);

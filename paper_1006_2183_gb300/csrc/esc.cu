@@ -261,7 +261,7 @@ spgemm_status_t esc_run(Engine* E, std::shared_ptr<DevBuf>* rbuf_out, std::share
         cnnz.push_back(nc_nnz);
         nnz += nc_nnz;
     }
-    SG_CUDA(ctx, cudaMemcpyAsync(E->Coff + U, &nnz, 8, cudaMemcpyHostToDevice, st));
+    SG_TRY(upload(ctx, E->Coff + U, &nnz, sizeof(nnz)));
     std::shared_ptr<DevBuf> rb, vb;
     if (nc == 1) {
         rb = crb[0];
@@ -280,7 +280,7 @@ spgemm_status_t esc_run(Engine* E, std::shared_ptr<DevBuf>* rbuf_out, std::share
         }
     }
     SG_CUDA(ctx, cudaGetLastError());
-    SG_TRY(sync_ctx(ctx));   // the work arrays and the host copy of nnz are released when this call returns
+    SG_TRY(sync_ctx(ctx));   // the work arrays are released when this call returns
     E->nnz_total = nnz;
     E->symbolic_done = true;
     *rbuf_out = rb;

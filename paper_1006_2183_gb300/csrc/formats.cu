@@ -537,8 +537,8 @@ spgemm_status_t check_handles(spgemm_ctx* ctx, const std::vector<spgemm_mat*>& m
     int64_t* db = (int64_t*)(dd + nh);
     int* dbad = (int*)(db + nh + 1);
     cudaStream_t st = ctx->stream;
-    SG_CUDA(ctx, cudaMemcpyAsync(dd, hd.data(), sizeof(VDesc) * nh, cudaMemcpyHostToDevice, st));
-    SG_CUDA(ctx, cudaMemcpyAsync(db, hb.data(), 8 * (nh + 1), cudaMemcpyHostToDevice, st));
+    SG_TRY(upload(ctx, dd, hd.data(), sizeof(VDesc) * nh));
+    SG_TRY(upload(ctx, db, hb.data(), 8 * (nh + 1)));
     SG_CUDA(ctx, cudaMemsetAsync(dbad, 0, 4 * nh, st));
     std::vector<int> hbad(nh, 0);
     if (hb[nh] > 0) {

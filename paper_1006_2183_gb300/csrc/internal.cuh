@@ -47,6 +47,7 @@ struct spgemm_ctx {
     size_t rb_cap = 0, rb_used = 0, rb_launched = 0;
     struct Readback { void* dst; const void* src; size_t off, bytes; };
     std::vector<Readback> rb_pending;   // the first rb_launched of them are on the stream already
+    std::vector<std::vector<char>> uploads;   // bytes of host-to-device copies that may still be under way
 };
 
 // Shared ownership of an allocation (batch outputs share one buffer).
@@ -169,6 +170,10 @@ spgemm_status_t sync_ctx(spgemm_ctx* ctx);
 // before a sync_ctx go to the context stream together, in one launch at that sync_ctx (or
 // before), so src has to keep its bytes until then; dst holds them after it (not before).
 spgemm_status_t read_back(spgemm_ctx* ctx, void* dst, const void* src, size_t bytes);
+// Queues a copy of host bytes to device address dst.  A copy from pageable memory may read it
+// after the call returns, so the context keeps the bytes until its next wait for the stream.
+spgemm_status_t upload(spgemm_ctx* ctx, void* dst, std::vector<char>&& bytes);
+spgemm_status_t upload(spgemm_ctx* ctx, void* dst, const void* src, size_t bytes);
 
 // formats.cu
 // Checks, in one launch and one synchronisation, every handle of `mats` that is a

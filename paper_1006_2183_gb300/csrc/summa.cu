@@ -312,14 +312,14 @@ spgemm_status_t partition(spgemm_ctx* ctx, const DMat& M, size_t w, int g, Block
     hm.insert(hm.end(), hchunk.begin(), hchunk.end());
     hm.insert(hm.end(), hnaux.begin(), hnaux.end());
     hm.push_back(0);
-    SG_CUDA(ctx, cudaMemcpyAsync(dm, hm.data(), 8 * hm.size(), cudaMemcpyHostToDevice, st));
+    SG_TRY(upload(ctx, dm, hm.data(), 8 * hm.size()));
     // about two waves of CTAs: a block's searches one after another were 0.12 ms
     const int aux_y = std::max(1, std::min(32, sm_count() * 32 / nblk));
     k_block_aux<<<dim3(nblk, aux_y), 128, 0, st>>>(nblk, dm, dm + (nblk + 1), dm + 2 * (nblk + 1), dm + 3 * (nblk + 1),
                                       dm + 3 * (nblk + 1) + nblk, (const int32_t*)jcb->p, (int64_t*)cpb->p,
                                       (int32_t*)auxb->p);
     note_launch();
-    SG_TRY(sync_ctx(ctx));   // host vectors above are copied before they go out of scope
+    SG_TRY(sync_ctx(ctx));   // reports what the launches above raised
     out->blk.assign(nblk, DMat());
     for (int b = 0; b < nblk; ++b) {
         const int I = b % g, J = b / g;
