@@ -625,11 +625,10 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         dw.bnd = (int32_t*)(sb + o_bnd);
     }
     if (sr == SPGEMM_OR_AND_BOOL) {
-        // boolean operands without a stored false value: the bitmap tiers take every output as true
-        int* vals_zero = (int*)(slab_ctr + 5);
-        if (ctx->bool_hint >= 0) SG_CUDA(ctx, cudaMemsetAsync(vals_zero, ctx->bool_hint ? 1 : 0, 4, st));
-        else launch_false_values(st, E->it, vals_zero);
-        E->dw.vals_zero = vals_zero;
+        // boolean operands without a stored false value: the tiers but the hash tables take every
+        // output as true
+        E->false_flag = (int*)(slab_ctr + 5);
+        E->dw.vals_zero = E->false_flag;
     }
     SG_CUDA(ctx, cudaGetLastError());
     return SPGEMM_OK;
@@ -733,8 +732,21 @@ spgemm_status_t engine_alloc_out(Engine* E, std::shared_ptr<DevBuf>* rbuf, std::
     return SPGEMM_OK;
 }
 
+void engine_false_values(Engine* E) {
+    if (!E->false_flag) return;
+    spgemm_ctx* ctx = E->ctx;
+    if (ctx->bool_hint >= 0) {
+        cudaMemsetAsync(E->false_flag, ctx->bool_hint ? 1 : 0, 4, ctx->stream);
+    } else {
+        if (E->false_flag_made) cudaMemsetAsync(E->false_flag, 0, 4, ctx->stream);
+        launch_false_values(ctx->stream, E->it, E->false_flag);
+    }
+    E->false_flag_made = true;
+}
+
 spgemm_status_t engine_numeric(Engine* E, int32_t* Cir, void* Cv) {
     if (!E->symbolic_done) SG_TRY(engine_symbolic(E));
+    engine_false_values(E);
     switch (E->sr) {
     case SPGEMM_PLUS_TIMES_F64: dispatch_numeric<PT64>(E, Cir, Cv); break;
     case SPGEMM_MIN_PLUS_F32: dispatch_numeric<MP32>(E, Cir, Cv); break;

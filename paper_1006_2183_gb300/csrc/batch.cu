@@ -132,6 +132,7 @@ void numeric_launches(struct spgemm_plan* P) {
 }
 
 void all_numeric_launches(struct spgemm_plan* P) {
+    engine_false_values(&P->E);
     switch (P->sr) {
     case SPGEMM_PLUS_TIMES_F64: numeric_launches<PT64>(P); break;
     case SPGEMM_MIN_PLUS_F32: numeric_launches<MP32>(P); break;

@@ -109,6 +109,7 @@ spgemm_status_t engine_numeric_bounded(Engine* E, std::shared_ptr<DevBuf>* rbuf,
     auto r = ctx_buf(ctx, 4 * (size_t)std::max<int64_t>(total, 1));
     auto v = ctx_buf(ctx, w * (size_t)std::max<int64_t>(total, 1));
     if (!r || !v) return set_err(ctx, SPGEMM_ERR_OOM, "bounded output of %lld slots", (long long)total);
+    engine_false_values(E);
     switch (E->sr) {
     case SPGEMM_PLUS_TIMES_F64: numeric_launches<PT64>(E, cap_off, (int32_t*)r->p, v->p); break;
     case SPGEMM_MIN_PLUS_F32: numeric_launches<MP32>(E, cap_off, (int32_t*)r->p, v->p); break;

@@ -96,6 +96,8 @@ struct Engine {
     int64_t* bin_off_dev = nullptr;
     int2* list = nullptr;
     sg::DenseWork dw;                    // slab-tier state
+    int* false_flag = nullptr;           // boolean: some operand value is false (device, zero after the set-up)
+    bool false_flag_made = false;
     int64_t* nnz_item = nullptr;
     void* scan_tmp = nullptr;
     float* feat = nullptr;               // predictor inputs (items x 8) when requested
@@ -194,6 +196,10 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
                              std::vector<sg::Prod> prods, bool want_features);
 spgemm_status_t engine_symbolic(Engine* E);
 spgemm_status_t engine_numeric(Engine* E, int32_t* Cir, void* Cv);
+// Boolean products: makes the false-value flag from the values that the operands hold now.  It
+// is queued before every numeric pass, a captured one's too: a plan's operands may have got
+// new values since its set-up.
+void engine_false_values(Engine* E);
 // predictor.cu: numeric pass without the symbolic pass of the hash tiers; returns C's arrays
 spgemm_status_t engine_numeric_predicted(Engine* E, std::shared_ptr<DevBuf>* rbuf, std::shared_ptr<DevBuf>* vbuf);
 // bounded.cu: numeric pass into min(flops, m) slots per hash-tier column (no symbolic pass

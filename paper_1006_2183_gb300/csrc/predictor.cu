@@ -283,6 +283,7 @@ spgemm_status_t engine_numeric_predicted(Engine* E, std::shared_ptr<DevBuf>* rbu
     auto tvb = ctx_buf(ctx, w * (size_t)std::max<int64_t>(total_cap, 1));
     if (!trb || !tvb) return set_err(ctx, SPGEMM_ERR_OOM, "predicted output of %lld entries", (long long)total_cap);
     // numeric into the predicted layout; hash tiers record their exact counts
+    engine_false_values(E);
     {
         PhaseTimer t(ctx, SPGEMM_PHASE_NUMERIC_HASH, E->sr);
         switch (E->sr) {
