@@ -35,10 +35,11 @@ struct MP32 {
     __device__ static Acc one() { return 0.0f; }
     __device__ static Acc mul(T a, T b) { return __fadd_rn(a, b); }
     __device__ static Acc add(Acc a, Acc b) { return b < a ? b : a; }
-    // min on floats through integer atomics: for x >= 0 the IEEE bit patterns
-    // order like signed ints; for x < 0 they order in reverse as unsigned ints.
+    // min on floats through integer atomics: without the sign bit the IEEE bit patterns
+    // order like signed ints, with it in reverse as unsigned ints.  -0 goes with the
+    // negatives: as a signed int it would lie below every one of them.
     __device__ static void atomic_add(Acc* p, Acc x) {
-        if (x >= 0.0f) atomicMin(reinterpret_cast<int*>(p), __float_as_int(x));
+        if (__float_as_int(x) >= 0) atomicMin(reinterpret_cast<int*>(p), __float_as_int(x));
         else atomicMax(reinterpret_cast<unsigned int*>(p), __float_as_uint(x));
     }
     __device__ static T out(Acc a) { return a; }
