@@ -84,33 +84,60 @@ __global__ void k_iota_u32(uint32_t* p, int64_t n) {
 // col[t] = the column of entry t, a tile of EX_TILE entries per CTA: the columns that start in
 // the tile leave their number at their first entry (an empty column's is overwritten by the
 // next one's, which is larger), and a running maximum carries it over the rest.  (Lanes
-// walking one column each took as long as the longest column.)
+// walking one column each took as long as the longest column.)  A tile over more than EX_SPAN
+// columns searches the column of every entry instead: a CTA that walks a long run of empty
+// columns waits for a load per few hundred of them (transpose of 2,000 entries in 2^20 columns
+// 908 -> 89 us, in 2^26 columns 126 -> 0.14 ms).  2^22 columns, walked against searched: 15 / 36
+// us of this kernel at 8,192 columns per tile, 30 / 45 at 32,768.
 constexpr int EX_BLOCK = 256;
 constexpr int EX_ITEMS = 8;
 constexpr int EX_TILE = EX_BLOCK * EX_ITEMS;
+constexpr int64_t EX_SPAN = 32768;
+
+// The last column of [lo, hi] that starts at or before entry t (column lo does), searched by a
+// warp with 32 probes a step: 4 dependent loads for a million columns, where halving has 20.
+__device__ __forceinline__ int64_t last_start(const int64_t* __restrict__ cp, int64_t lo, int64_t hi, int64_t t) {
+    const int lane = threadIdx.x & 31;
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) >> 5;
+        const unsigned after = ~__ballot_sync(0xffffffffu, __ldg(cp + min(lo + step * (lane + 1), hi)) <= t);
+        const int k = after ? __ffs(after) - 1 : 32;   // probes at or before t
+        const int64_t below = k < 32 ? min(lo + step * (k + 1), hi) - 1 : hi;
+        if (k > 0) lo = min(lo + step * k, hi);
+        hi = max(lo, below);
+    }
+    return lo;
+}
+
 __global__ void __launch_bounds__(EX_BLOCK) k_expand_cols(const int64_t* __restrict__ cp, int64_t n, int64_t nnz,
                                                           int32_t* __restrict__ col) {
     __shared__ int s_col[EX_TILE];
     __shared__ int s_w[EX_BLOCK / 32];
-    __shared__ int s_first;
+    __shared__ int s_ends[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t t0 = (int64_t)blockIdx.x * EX_TILE, t1 = min(t0 + EX_TILE, nnz);
-    if (tid == 0) {   // the last column that starts at or before t0
-        int64_t lo = 0, hi = n - 1;
-        while (lo < hi) {
-            const int64_t mid = (lo + hi + 1) >> 1;
-            if (__ldg(cp + mid) <= t0) lo = mid;
-            else hi = mid - 1;
-        }
-        s_first = (int)lo;
+    if (warp < 2) {   // the columns of the tile's first and last entry
+        const int64_t c = last_start(cp, 0, n - 1, warp ? t1 - 1 : t0);
+        if (lane == 0) s_ends[warp] = (int)c;
     }
     for (int i = tid; i < EX_TILE; i += EX_BLOCK) s_col[i] = 0;
     __syncthreads();
-    const int64_t c0 = s_first;
-    for (int64_t j = c0 + 1 + tid; j < n; j += EX_BLOCK) {
+    const int64_t c0 = s_ends[0], c1 = s_ends[1];
+    if (c1 - c0 > EX_SPAN) {
+        for (int64_t t = t0 + tid; t < t1; t += EX_BLOCK) {
+            int64_t lo = c0, hi = c1;
+            while (lo < hi) {
+                const int64_t mid = (lo + hi + 1) >> 1;
+                if (__ldg(cp + mid) <= t) lo = mid;
+                else hi = mid - 1;
+            }
+            col[t] = (int32_t)lo;
+        }
+        return;
+    }
+    for (int64_t j = c0 + 1 + tid; j <= c1; j += EX_BLOCK) {
         const int64_t at = __ldg(cp + j);
-        if (at >= t1) break;
-        if (at > t0) atomicMax(&s_col[at - t0], (int)(j - c0));   // always, in a valid operand
+        if (at > t0 && at < t1) atomicMax(&s_col[at - t0], (int)(j - c0));   // always, in a valid operand
     }
     __syncthreads();
     int v[EX_ITEMS], m = 0;

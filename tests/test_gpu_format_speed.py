@@ -1,0 +1,55 @@
+"""Conversions of matrices whose entries crowd on few rows or columns, or leave most columns
+empty, take about as long as those of evenly filled ones of the same size: no pass leaves such
+a column, row or run to one CTA.  The bounds are a factor of four on the even matrix' time."""
+import pytest
+import torch
+
+from gpu_util import sp
+from helpers import PT_F64
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    return sp().Context()
+
+
+def _time(op):
+    for _ in range(3):
+        op()
+    best = float("inf")
+    for _ in range(7):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        op()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
+def _handle(ctx, m, n, colptr, rows):
+    s = sp()
+    v = torch.ones(rows.numel(), device=ctx.device, dtype=torch.float64)
+    return s.Matrix.csc(ctx, m, n, colptr.to(ctx.device), rows.to(ctx.device, torch.int32), v, PT_F64)
+
+
+def _full(ctx, m, n):
+    return _handle(ctx, m, n, torch.arange(n + 1) * m, torch.arange(m).repeat(n))
+
+
+def _even(ctx, m, n, deg):
+    """`deg` entries per column, spread over the rows."""
+    rows = (torch.arange(n)[:, None] * 7919 + torch.arange(deg) * (m // deg)).remainder(m).sort(1).values
+    return _handle(ctx, m, n, torch.arange(n + 1) * deg, rows.flatten())
+
+
+def test_runs_of_empty_columns(ctx):
+    n = 1 << 22
+    at = torch.arange(1000) * (n // 1000)
+    ptr = torch.zeros(n + 1, dtype=torch.int64)
+    ptr[at + 1] = 1
+    few, even = _handle(ctx, n, n, ptr.cumsum(0), at), _even(ctx, n, n, 1)
+    t = sp().spgemm_mat_transpose
+    assert _time(lambda: t(ctx, few)) < 4 * _time(lambda: t(ctx, even))
