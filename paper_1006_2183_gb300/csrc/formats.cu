@@ -208,6 +208,17 @@ struct SegSort {
     int64_t bound;            // keys are below bound < 2^23
     int32_t* list;            // long columns, *nlist of them
     int* nlist;
+    // columns of more than split_len entries are split by their keys into nwin windows of
+    // 2^wbits keys, in chunks of SEG_CHUNK entries
+    int64_t split_len;
+    int wbits, nwin;
+    int32_t* split;           // the columns, *nsplit of them
+    int2* chunk;              // place in `split` and number of every chunk, *nchunk of them
+    uint32_t* win;            // per column: entries of its SEG_WIN windows
+    uint32_t* off;            // per chunk: where its entries go in every window
+    uint32_t* wkey;           // the entries by windows: key and place in the column (nnz each)
+    uint32_t* widx;
+    int *nsplit, *nchunk;
 };
 constexpr int SEG_SB = 9;                     // slots of a warp's column: at most 512 entries
 constexpr int SEG_MAX = 1 << SEG_SB;
@@ -215,32 +226,41 @@ constexpr int64_t SEG_BOUND = (int64_t(1) << (32 - SEG_SB)) - 1;
 constexpr int SEG_BLOCK = 128;
 constexpr int SEGL_BLOCK = 512;
 constexpr int64_t SEGL_ROWS = 1 << 20;        // keys ranked at a time in a long column
+// A column of more entries than one CTA takes (SEG_SPLIT, fewer where it would read them once per
+// SEGL_ROWS keys) is cut into at most SEG_WIN windows of keys: its chunks count their entries per
+// window, then put them there, and a CTA ranks each window.  One CTA for the whole column took
+// 25.7 ms for a row of 2^22 entries (2.9 now, all of it the row counters), 4.07 ms for the
+// permutation of 8 columns of 2^20 (0.50).  The line: permutation of 8 columns of 32,768 entries
+// 118 us split and 165 whole, of 256 such columns 341 and 331, of 512 columns of 16,384 entries
+// 323 and 289.
+constexpr int64_t SEG_SPLIT = 16384;
+constexpr int SEG_CHUNK = 8192;
+constexpr int SEG_WIN = 256;
+constexpr int SEG_WIN_KEYS = 1 << 15;         // 256 windows of it hold the 2^23 keys
 
-__device__ __forceinline__ uint32_t seg_key(const SegSort& S, int64_t t, int slot) {
+__device__ __forceinline__ int32_t seg_row(const SegSort& S, int64_t t) {
     const int32_t x = __ldg(S.key + t);
-    return ((uint32_t)(S.relabel ? __ldg(S.relabel + x) : x) << SEG_SB) | (uint32_t)slot;
+    return S.relabel ? __ldg(S.relabel + x) : x;
 }
 
-template <int W>
-__device__ __forceinline__ void seg_put(const SegSort& S, int64_t s, int64_t to, uint32_t k) {
-    using T = typename Word<W>::T;
-    S.okey[to] = (int32_t)(k >> SEG_SB);
-    if (S.val) reinterpret_cast<T*>(S.oval)[to] = __ldg(reinterpret_cast<const T*>(S.val) + s + (k & (SEG_MAX - 1)));
+__device__ __forceinline__ uint32_t seg_key(const SegSort& S, int64_t t, int slot) {
+    return ((uint32_t)seg_row(S, t) << SEG_SB) | (uint32_t)slot;
 }
 
 // A column of at most G K entries per group of G lanes (len 0: none); whole warps call it.
-template <int W, int G, int K>
-__device__ __forceinline__ void seg_sort_column(const SegSort& S, int64_t s, int len, int64_t o, uint32_t* stage) {
+// key_at(i) is entry i's key << SEG_SB | i, put(to, k) stores the entry of key k in place `to`.
+template <int G, int K, class Key, class Put>
+__device__ __forceinline__ void seg_sort_column(int len, uint32_t* stage, Key key_at, Put put) {
     const int lane = threadIdx.x & (G - 1);
     uint32_t key[K];
 #pragma unroll
     for (int r = 0; r < K; ++r) {
         const int i = r * G + lane;
-        key[r] = i < len ? seg_key(S, s + i, i) : 0xffffffffu;
+        key[r] = i < len ? key_at(i) : 0xffffffffu;
     }
     sort_keys<G, K>(key, lane);
     if constexpr (K == 1) {
-        if (lane < len) seg_put<W>(S, s, o + lane, key[0]);
+        if (lane < len) put(lane, key[0]);
         return;
     }
 #pragma unroll
@@ -249,9 +269,35 @@ __device__ __forceinline__ void seg_sort_column(const SegSort& S, int64_t s, int
 #pragma unroll
     for (int r = 0; r < K; ++r) {
         const int i = r * G + lane;
-        if (i < len) seg_put<W>(S, s, o + i, stage[st_ph(i)]);
+        if (i < len) put(i, stage[st_ph(i)]);
     }
     __syncwarp();
+}
+
+// The same for a warp and at most SEG_MAX entries.
+template <class Key, class Put>
+__device__ __forceinline__ void seg_sort_warp(int len, uint32_t* stage, Key key_at, Put put) {
+    if (len <= 64) seg_sort_column<32, 2>(len, stage, key_at, put);
+    else if (len <= 128) seg_sort_column<32, 4>(len, stage, key_at, put);
+    else if (len <= 256) seg_sort_column<32, 8>(len, stage, key_at, put);
+    else seg_sort_column<32, 16>(len, stage, key_at, put);
+}
+
+// Entry of key k (its slot in the low bits) of the column at s, stored at `to`.
+template <int W>
+__device__ __forceinline__ void seg_put(const SegSort& S, int64_t s, int64_t to, uint32_t k) {
+    using T = typename Word<W>::T;
+    S.okey[to] = (int32_t)(k >> SEG_SB);
+    if (S.val) reinterpret_cast<T*>(S.oval)[to] = __ldg(reinterpret_cast<const T*>(S.val) + s + (k & (SEG_MAX - 1)));
+}
+
+// A column given up to the split: room for its windows and one record per chunk.
+__device__ __forceinline__ void seg_split(const SegSort& S, int32_t c, int64_t len) {
+    const int v = atomicAdd(S.nsplit, 1), nch = (int)((len + SEG_CHUNK - 1) / SEG_CHUNK);
+    S.split[v] = c;
+    for (int w = 0; w < SEG_WIN; ++w) S.win[(int64_t)v * SEG_WIN + w] = 0u;
+    const int q = atomicAdd(S.nchunk, nch);
+    for (int i = 0; i < nch; ++i) S.chunk[q + i] = make_int2(v, i);
 }
 
 // `per` columns per warp and round (32, or 4 where they are long enough to fill a warp's lanes
@@ -271,7 +317,9 @@ __global__ void __launch_bounds__(SEG_BLOCK) k_seg_sort(SegSort S, int per) {
             len = __ldg(S.in_cp + c + 1) - s;
             if (len > 0) o = __ldg(S.out_cp + (S.out_col ? __ldg(S.out_col + c) : c));
         }
-        if (len > SEG_MAX) {
+        if (len > S.split_len) {
+            seg_split(S, (int32_t)c, len);
+        } else if (len > SEG_MAX) {
             S.list[atomicAdd(S.nlist, 1)] = (int32_t)c;
         } else if (len > 0 && len <= 4) {
             uint32_t k[4];
@@ -302,7 +350,8 @@ __global__ void __launch_bounds__(SEG_BLOCK) k_seg_sort(SegSort S, int per) {
             const int from = src < 0 ? 0 : src;
             const int64_t gs = __shfl_sync(0xffffffffu, s, from), go = __shfl_sync(0xffffffffu, o, from);
             const int gl = __shfl_sync(0xffffffffu, (int)len, from);
-            seg_sort_column<W, 8, 4>(S, gs, src < 0 ? 0 : gl, go, stage + grp * 40);
+            seg_sort_column<8, 4>(src < 0 ? 0 : gl, stage + grp * 40, [&](int i) { return seg_key(S, gs + i, i); },
+                                  [&](int to, uint32_t k) { seg_put<W>(S, gs, go + to, k); });
         }
         unsigned many = __ballot_sync(0xffffffffu, len > 32 && len <= SEG_MAX);
         while (many) {
@@ -310,76 +359,209 @@ __global__ void __launch_bounds__(SEG_BLOCK) k_seg_sort(SegSort S, int per) {
             many &= many - 1;
             const int64_t ws = __shfl_sync(0xffffffffu, s, src), wo = __shfl_sync(0xffffffffu, o, src);
             const int wl = __shfl_sync(0xffffffffu, (int)len, src);
-            if (wl <= 64) seg_sort_column<W, 32, 2>(S, ws, wl, wo, stage);
-            else if (wl <= 128) seg_sort_column<W, 32, 4>(S, ws, wl, wo, stage);
-            else if (wl <= 256) seg_sort_column<W, 32, 8>(S, ws, wl, wo, stage);
-            else seg_sort_column<W, 32, 16>(S, ws, wl, wo, stage);
+            seg_sort_warp(wl, stage, [&](int i) { return seg_key(S, ws + i, i); },
+                          [&](int to, uint32_t k) { seg_put<W>(S, ws, wo + to, k); });
         }
     }
 }
 
-// A CTA per long column: its keys marked in a bitmap in shared memory (SEGL_ROWS keys at a
-// time), and every entry written at its key's rank.
-template <int W>
-__global__ void __launch_bounds__(SEGL_BLOCK) k_seg_long(SegSort S, int rows) {
+// The entries of one column whose keys lie in [base, base + rows), among its `len` ones: marked
+// in a bitmap in shared memory and written at their keys' ranks from `o` on.  key_at(i) is an
+// entry's key, src_at(i) its place in the column.  Returns how many there were; ends with a
+// barrier.
+template <int W, int BLOCK, class Key, class Src>
+__device__ __forceinline__ int seg_rank(const SegSort& S, int64_t s, int64_t len, int base, int rows, int64_t o,
+                                        uint4* bits, int* pre, int* cc, Key key_at, Src src_at) {
     using T = typename Word<W>::T;
-    extern __shared__ __align__(16) unsigned char smem[];
-    const int ng = (rows + 127) >> 7, nch = (ng + 31) >> 5;
-    uint4* bits = reinterpret_cast<uint4*>(smem);
-    int* pre = reinterpret_cast<int*>(bits + ng);   // keys before every 128
-    int* cc = pre + ng;                             // and of every 32 groups
     __shared__ int s_total;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int n = *S.nlist;
-    for (int l = blockIdx.x; l < n; l += gridDim.x) {
-        const int64_t c = S.list[l];
-        const int64_t s = __ldg(S.in_cp + c), len = __ldg(S.in_cp + c + 1) - s;
-        int64_t o = __ldg(S.out_cp + (S.out_col ? __ldg(S.out_col + c) : c));
-        auto key_at = [&](int64_t i) {
-            const int32_t x = __ldg(S.key + s + i);
-            return (int64_t)(S.relabel ? __ldg(S.relabel + x) : x);
-        };
-        for (int64_t base = 0; base < S.bound; base += rows) {
-            for (int g = tid; g < ng; g += SEGL_BLOCK) bits[g] = make_uint4(0u, 0u, 0u, 0u);
-            __syncthreads();
-            for (int64_t i = tid; i < len; i += SEGL_BLOCK) {
-                const int64_t k = key_at(i) - base;
-                if (k >= 0 && k < rows) atomicOr(reinterpret_cast<uint32_t*>(bits) + (k >> 5), 1u << (k & 31));
-            }
-            __syncthreads();
-            for (int q = warp; q < nch; q += SEGL_BLOCK / 32) {
-                const int g = q * 32 + lane;
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (g < ng) v = bits[g];
-                const int k = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w), inc = warp_incl_scan(k);
-                if (g < ng) pre[g] = inc - k;
-                if (lane == 31) cc[q] = inc;
-            }
-            __syncthreads();
-            if (warp == 0) {
-                int run = 0;
-                for (int q0 = 0; q0 < nch; q0 += 32) {
-                    const int v = q0 + lane < nch ? cc[q0 + lane] : 0, inc = warp_incl_scan(v);
-                    if (q0 + lane < nch) cc[q0 + lane] = run + inc - v;
-                    run += __shfl_sync(0xffffffffu, inc, 31);
-                }
-                if (lane == 0) s_total = run;
-            }
-            __syncthreads();
-            for (int64_t i = tid; i < len; i += SEGL_BLOCK) {
-                const int64_t kk = key_at(i), k = kk - base;
-                if (k < 0 || k >= rows) continue;
-                const int g = (int)(k >> 7), y = (int)(k >> 5) & 3;
-                const uint4 v = bits[g];
-                const uint32_t w = y == 0 ? v.x : y == 1 ? v.y : y == 2 ? v.z : v.w;
-                const int rank = cc[g >> 5] + pre[g] + __popc(w & ((1u << (k & 31)) - 1u)) + (y > 0 ? __popc(v.x) : 0) +
-                                 (y > 1 ? __popc(v.y) : 0) + (y > 2 ? __popc(v.z) : 0);
-                S.okey[o + rank] = (int32_t)kk;
-                if (S.val) reinterpret_cast<T*>(S.oval)[o + rank] = __ldg(reinterpret_cast<const T*>(S.val) + s + i);
-            }
-            o += s_total;
-            __syncthreads();
+    const int ng = (rows + 127) >> 7, nch = (ng + 31) >> 5;
+    for (int g = tid; g < ng; g += BLOCK) bits[g] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    for (int64_t i = tid; i < len; i += BLOCK) {
+        const int k = key_at(i) - base;
+        if ((unsigned)k < (unsigned)rows) atomicOr(reinterpret_cast<uint32_t*>(bits) + (k >> 5), 1u << (k & 31));
+    }
+    __syncthreads();
+    // keys before every 128 (pre, inside its chunk of 32 groups) and before every chunk (cc)
+    for (int q = warp; q < nch; q += BLOCK / 32) {
+        const int g = q * 32 + lane;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (g < ng) v = bits[g];
+        const int k = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w), inc = warp_incl_scan(k);
+        if (g < ng) pre[g] = inc - k;
+        if (lane == 31) cc[q] = inc;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        int run = 0;
+        for (int q0 = 0; q0 < nch; q0 += 32) {
+            const int v = q0 + lane < nch ? cc[q0 + lane] : 0, inc = warp_incl_scan(v);
+            if (q0 + lane < nch) cc[q0 + lane] = run + inc - v;
+            run += __shfl_sync(0xffffffffu, inc, 31);
         }
+        if (lane == 0) s_total = run;
+    }
+    __syncthreads();
+    for (int64_t i = tid; i < len; i += BLOCK) {
+        const int k = key_at(i) - base;
+        if ((unsigned)k >= (unsigned)rows) continue;
+        const int g = k >> 7, y = (k >> 5) & 3;
+        const uint4 v = bits[g];
+        const uint32_t w = y == 0 ? v.x : y == 1 ? v.y : y == 2 ? v.z : v.w;
+        const int rank = cc[g >> 5] + pre[g] + __popc(w & ((1u << (k & 31)) - 1u)) + (y > 0 ? __popc(v.x) : 0) +
+                         (y > 1 ? __popc(v.y) : 0) + (y > 2 ? __popc(v.z) : 0);
+        S.okey[o + rank] = k + base;
+        if (S.val) reinterpret_cast<T*>(S.oval)[o + rank] = __ldg(reinterpret_cast<const T*>(S.val) + s + src_at(i));
+    }
+    const int total = s_total;
+    __syncthreads();
+    return total;
+}
+
+// entries [i0, i1) of a chunk, where they start in their column's arrays, and the column's place
+// in the list of split columns
+struct SegChunk {
+    int v;
+    int64_t c, s, i0, i1;
+    __device__ SegChunk(const SegSort& S, int q) {
+        const int2 e = S.chunk[q];
+        v = e.x;
+        c = S.split[v];
+        s = __ldg(S.in_cp + c);
+        const int64_t len = __ldg(S.in_cp + c + 1) - s;
+        i0 = (int64_t)e.y * SEG_CHUNK;
+        i1 = min(len, i0 + SEG_CHUNK);
+    }
+};
+
+// A CTA per long column, SEGL_ROWS keys at a time, and per chunk of a split column: how many of
+// its entries each window of keys gets, and where they go inside it.
+template <int W>
+__global__ void __launch_bounds__(SEGL_BLOCK) k_seg_long(SegSort S, int rows) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint32_t s_win[SEG_WIN];
+    const int ng = (rows + 127) >> 7;
+    uint4* bits = reinterpret_cast<uint4*>(smem);
+    int* pre = reinterpret_cast<int*>(bits + ng);
+    int* cc = pre + ng;
+    const int tid = threadIdx.x;
+    const int n = *S.nlist, total = n + *S.nchunk;
+    for (int l = blockIdx.x; l < total; l += gridDim.x) {
+        if (l < n) {
+            const int64_t c = S.list[l];
+            const int64_t s = __ldg(S.in_cp + c), len = __ldg(S.in_cp + c + 1) - s;
+            int64_t o = __ldg(S.out_cp + (S.out_col ? __ldg(S.out_col + c) : c));
+            for (int64_t base = 0; base < S.bound; base += rows)
+                o += seg_rank<W, SEGL_BLOCK>(S, s, len, (int)base, rows, o, bits, pre, cc,
+                                             [&](int64_t i) { return seg_row(S, s + i); }, [](int64_t i) { return i; });
+            continue;
+        }
+        const int q = l - n;
+        const SegChunk ch(S, q);
+        for (int w = tid; w < SEG_WIN; w += SEGL_BLOCK) s_win[w] = 0u;
+        __syncthreads();
+        for (int64_t i = ch.i0 + tid; i < ch.i1; i += SEGL_BLOCK) atomicAdd(&s_win[seg_row(S, ch.s + i) >> S.wbits], 1u);
+        __syncthreads();
+        for (int w = tid; w < SEG_WIN; w += SEGL_BLOCK) {
+            const uint32_t k = s_win[w];
+            S.off[(int64_t)q * SEG_WIN + w] = k ? atomicAdd(S.win + (int64_t)ch.v * SEG_WIN + w, k) : 0u;
+        }
+        __syncthreads();
+    }
+}
+
+// Where the windows of split column v start inside it: s_at[w], from the windows' counts.  All
+// threads of a CTA of at least SEG_WIN call it; ends with a barrier.
+__device__ __forceinline__ void window_starts(const SegSort& S, int v, uint32_t* s_at, int* s_w) {
+    const int tid = threadIdx.x, lane = tid & 31;
+    int x = 0, inc = 0;
+    if (tid < SEG_WIN) {
+        x = (int)S.win[(int64_t)v * SEG_WIN + tid];
+        inc = warp_incl_scan(x);
+        if (lane == 31) s_w[tid >> 5] = inc;
+    }
+    __syncthreads();
+    if (tid < SEG_WIN) {
+        for (int w = 0; w < (tid >> 5); ++w) inc += s_w[w];
+        s_at[tid] = (uint32_t)(inc - x);
+    }
+    __syncthreads();
+}
+
+// The entries of a chunk put into their windows, in any order inside them.
+__global__ void __launch_bounds__(SEGL_BLOCK) k_seg_scatter(SegSort S) {
+    __shared__ uint32_t s_at[SEG_WIN];
+    __shared__ int s_w[SEG_WIN / 32];
+    const int n = *S.nchunk;
+    for (int q = blockIdx.x; q < n; q += gridDim.x) {
+        const SegChunk ch(S, q);
+        window_starts(S, ch.v, s_at, s_w);
+        for (int w = threadIdx.x; w < SEG_WIN; w += SEGL_BLOCK) s_at[w] += S.off[(int64_t)q * SEG_WIN + w];
+        __syncthreads();
+        for (int64_t i = ch.i0 + threadIdx.x; i < ch.i1; i += SEGL_BLOCK) {
+            const int k = seg_row(S, ch.s + i);
+            const int64_t at = ch.s + atomicAdd(&s_at[k >> S.wbits], 1u);
+            S.wkey[at] = (uint32_t)k;
+            S.widx[at] = (uint32_t)i;
+        }
+        __syncthreads();
+    }
+}
+
+// The windows of the split columns: those of at most SEG_MAX entries sorted by a warp each, eight
+// of a column per CTA and round, then the longer ones ranked by a CTA each.
+template <int W>
+__global__ void __launch_bounds__(SEG_WIN, 4) k_seg_windows(SegSort S) {
+    using T = typename Word<W>::T;
+    constexpr int NG = SEG_WIN_KEYS / 128, NW = SEG_WIN / 32;
+    __shared__ uint4 s_bits[NG];
+    __shared__ int s_pre[NG], s_cc[(NG + 31) / 32], s_w[NW], s_big[SEG_WIN], s_nbig;
+    __shared__ uint32_t s_at[SEG_WIN], s_stage[NW][st_span<SEG_MAX>()];
+    const int tid = threadIdx.x, warp = tid >> 5;
+    const int nsplit = *S.nsplit, per = (S.nwin + NW - 1) / NW;
+    const T* __restrict__ val = reinterpret_cast<const T*>(S.val);
+    int64_t s = 0, o = 0;   // of the column that s_at is for
+    auto column = [&](int v) {
+        window_starts(S, v, s_at, s_w);
+        const int64_t c = S.split[v];
+        s = __ldg(S.in_cp + c);
+        o = __ldg(S.out_cp + (S.out_col ? __ldg(S.out_col + c) : c));
+    };
+    for (int l = blockIdx.x; l < nsplit * per; l += gridDim.x) {
+        const int v = l / per, w = l % per * NW + warp;
+        column(v);
+        const uint32_t len = w < S.nwin ? S.win[(int64_t)v * SEG_WIN + w] : 0u;
+        if (len > 0 && len <= SEG_MAX) {
+            const int base = w << S.wbits;
+            const int64_t at = s + s_at[w], to0 = o + s_at[w];
+            seg_sort_warp((int)len, s_stage[warp], [&](int i) { return (S.wkey[at + i] - base) << SEG_SB | (uint32_t)i; },
+                          [&](int to, uint32_t k) {
+                              S.okey[to0 + to] = (int32_t)(k >> SEG_SB) + base;
+                              if (val)
+                                  reinterpret_cast<T*>(S.oval)[to0 + to] = __ldg(val + s + S.widx[at + (k & (SEG_MAX - 1))]);
+                          });
+        }
+        __syncthreads();   // s_at is free for the next round
+    }
+    // the CTA's share of all windows, looked through by its threads at once
+    const int64_t n = (int64_t)nsplit * S.nwin, step = gridDim.x;
+    for (int64_t l0 = blockIdx.x; l0 < n; l0 += step * SEG_WIN) {
+        if (tid == 0) s_nbig = 0;
+        __syncthreads();
+        const int64_t l = l0 + tid * step;
+        if (l < n && S.win[l / S.nwin * SEG_WIN + l % S.nwin] > SEG_MAX) s_big[atomicAdd(&s_nbig, 1)] = (int)l;
+        __syncthreads();
+        const int nbig = s_nbig;
+        for (int b = 0; b < nbig; ++b) {
+            const int v = s_big[b] / S.nwin, w = s_big[b] % S.nwin;
+            column(v);
+            const int64_t len = S.win[(int64_t)v * SEG_WIN + w], at = s + s_at[w];
+            seg_rank<W, SEG_WIN>(S, s, len, w << S.wbits, 1 << S.wbits, o + s_at[w], s_bits, s_pre, s_cc,
+                                 [&](int64_t i) { return (int)S.wkey[at + i]; },
+                                 [&](int64_t i) { return (int64_t)S.widx[at + i]; });
+        }
+        __syncthreads();
     }
 }
 
@@ -428,9 +610,52 @@ void run_seg_sort(cudaStream_t st, const SegSort& S) {
     smem_at_least((const void*)k_seg_long<W>, smem);
     k_seg_long<W><<<sm_count() * 2, SEGL_BLOCK, smem, st>>>(S, rows);
     note_launch(2);
+    if (S.nnz > S.split_len) {
+        k_seg_scatter<<<(int)std::min<int64_t>(ceil_div64(S.nnz, SEG_CHUNK), sm_count() * 4), SEGL_BLOCK, 0, st>>>(S);
+        k_seg_windows<W><<<sm_count() * 8, SEG_WIN, 0, st>>>(S);
+        note_launch(2);
+    }
 }
 
-// S.list and S.nlist: room for n columns, and a zero
+// The scratch of a sort of n columns and nnz entries with keys below `bound`, laid out by
+// take(bytes) -> offset; bind() sets S's pointers.  The counters are 16 bytes that the caller
+// zeroes; wkey and widx are 4 nnz bytes each, the caller's too where they are given.
+struct SegScratch {
+    int64_t nnz, split_len;
+    size_t o_list, o_split = 0, o_chunk = 0, o_win = 0, o_off = 0, o_wkey = 0, o_widx = 0;
+    template <class Take>
+    SegScratch(int64_t n, int64_t nz, int64_t bound, bool own_entries, Take take) : nnz(nz) {
+        split_len = SEG_SPLIT / std::max<int64_t>(1, ceil_div64(bound, SEGL_ROWS));
+        o_list = take(4 * n);
+        if (nnz <= split_len) return;   // no column to split
+        const int64_t ns = nnz / split_len, nc = nnz / SEG_CHUNK + ns;
+        o_split = take(4 * ns);
+        o_chunk = take(8 * nc);
+        o_win = take(4 * SEG_WIN * ns);
+        o_off = take(4 * SEG_WIN * nc);
+        if (own_entries) {
+            o_wkey = take(4 * nnz);
+            o_widx = take(4 * nnz);
+        }
+    }
+    void bind(char* t, int* counters, uint32_t* wkey, uint32_t* widx, SegSort* S) const {
+        S->list = (int32_t*)(t + o_list);
+        S->nlist = counters;
+        S->nsplit = counters + 1;
+        S->nchunk = counters + 2;
+        S->split_len = split_len;
+        S->wbits = 10;
+        while (S->bound > (int64_t)SEG_WIN << S->wbits) ++S->wbits;
+        S->nwin = (int)ceil_div64(S->bound, int64_t(1) << S->wbits);
+        S->split = (int32_t*)(t + o_split);
+        S->chunk = (int2*)(t + o_chunk);
+        S->win = (uint32_t*)(t + o_win);
+        S->off = (uint32_t*)(t + o_off);
+        S->wkey = wkey ? wkey : (uint32_t*)(t + o_wkey);
+        S->widx = widx ? widx : (uint32_t*)(t + o_widx);
+    }
+};
+
 void launch_seg_sort(cudaStream_t st, const SegSort& S, size_t w) {
     if (S.n <= 0) return;
     switch (w) {
@@ -637,12 +862,13 @@ spgemm_status_t transpose_csc(spgemm_ctx* ctx, int64_t m, int64_t n, int64_t nnz
             off += (bytes + 255) / 256 * 256;
             return o;
         };
-        const size_t o_cnt = take(8 * m + 16), o_list = take(4 * m), o_sc = take(scan_tmp_bytes(m));
+        const size_t o_cnt = take(8 * m + 16), o_sc = take(scan_tmp_bytes(m));
+        const SegScratch scratch(m, nz, n, false, take);
         const size_t o_col = take(4 * nz), o_place = take(4 * nz), o_key = take(4 * nz), o_val = take(num ? w * nz : 0);
         auto tmp = ctx_buf(ctx, off);
         if (!cpb || !irb || !vb || !tmp) return set_err(ctx, SPGEMM_ERR_OOM, "transpose buffers");
         char* t = (char*)tmp->p;
-        unsigned long long* cnt = (unsigned long long*)(t + o_cnt);   // m counts, then the long rows' number
+        unsigned long long* cnt = (unsigned long long*)(t + o_cnt);   // m counts, then the sort's counters
         int32_t* colid = (int32_t*)(t + o_col);
         uint32_t* place = (uint32_t*)(t + o_place);
         int64_t* tcp = (int64_t*)cpb->p;
@@ -658,8 +884,8 @@ spgemm_status_t transpose_csc(spgemm_ctx* ctx, int64_t m, int64_t n, int64_t nnz
         default: k_row_scatter<8><<<grid_for(nz), 256, 0, st>>>(ir, colid, place, num, nz, m, tcp, (int32_t*)(t + o_key), tv); break;
         }
         note_launch();
-        SegSort S{tcp, m, nz, tcp, nullptr, (const int32_t*)(t + o_key), nullptr, tv, (int32_t*)irb->p, vb->p, n,
-                  (int32_t*)(t + o_list), (int*)(cnt + m)};
+        SegSort S{tcp, m, nz, tcp, nullptr, (const int32_t*)(t + o_key), nullptr, tv, (int32_t*)irb->p, vb->p, n};
+        scratch.bind(t, (int*)(cnt + m), place, (uint32_t*)colid, &S);   // both are free by then
         launch_seg_sort(st, S, w);
         SG_CUDA(ctx, cudaGetLastError());
         out->ctx = ctx;
@@ -903,17 +1129,19 @@ static spgemm_status_t permute_csc(spgemm_ctx* ctx, int64_t m, int64_t n, int64_
             off += (bytes + 255) / 256 * 256;
             return o;
         };
-        const size_t o_len = take(8 * n + 16), o_list = take(4 * n), o_sc = take(scan_tmp_bytes(n));
+        const size_t o_len = take(8 * n + 16), o_sc = take(scan_tmp_bytes(n));
+        const SegScratch scratch(n, nnz, m, true, take);
         auto tmp = ctx_buf(ctx, off);
         if (!cpb || !irb || !vb || !tmp) return set_err(ctx, SPGEMM_ERR_OOM, "permute buffers");
         char* t = (char*)tmp->p;
-        int64_t* len = (int64_t*)(t + o_len);   // n lengths, then the long columns' number
+        int64_t* len = (int64_t*)(t + o_len);   // n lengths, then the sort's counters
         int64_t* ocp = (int64_t*)cpb->p;
-        SG_CUDA(ctx, cudaMemsetAsync(len + n, 0, 8, st));
+        SG_CUDA(ctx, cudaMemsetAsync(len + n, 0, 16, st));
         k_perm_lens<<<grid_for(n), 256, 0, st>>>(cp, colp, n, len);
         note_launch();
         launch_exclusive_scan(st, len, n, ocp, t + o_sc);
-        SegSort S{cp, n, nnz, ocp, colp, ir, rowp, num, (int32_t*)irb->p, vb->p, m, (int32_t*)(t + o_list), (int*)(len + n)};
+        SegSort S{cp, n, nnz, ocp, colp, ir, rowp, num, (int32_t*)irb->p, vb->p, m};
+        scratch.bind(t, (int*)(len + n), nullptr, nullptr, &S);
         launch_seg_sort(st, S, w);
         SG_CUDA(ctx, cudaGetLastError());
         out->ctx = ctx;

@@ -53,3 +53,11 @@ def test_runs_of_empty_columns(ctx):
     few, even = _handle(ctx, n, n, ptr.cumsum(0), at), _even(ctx, n, n, 1)
     t = sp().spgemm_mat_transpose
     assert _time(lambda: t(ctx, few)) < 4 * _time(lambda: t(ctx, even))
+
+
+def test_few_long_columns(ctx):
+    m = 1 << 20
+    long, even = _full(ctx, m, 8), _full(ctx, 2896, 2896)
+    p, q = (torch.randperm(k, device=ctx.device).to(torch.int32) for k in (m, 2896))
+    t = sp().spgemm_mat_permute
+    assert _time(lambda: t(ctx, long, p, None)) < 4 * _time(lambda: t(ctx, even, q, None))
