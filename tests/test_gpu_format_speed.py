@@ -61,3 +61,9 @@ def test_few_long_columns(ctx):
     p, q = (torch.randperm(k, device=ctx.device).to(torch.int32) for k in (m, 2896))
     t = sp().spgemm_mat_permute
     assert _time(lambda: t(ctx, long, p, None)) < 4 * _time(lambda: t(ctx, even, q, None))
+
+
+def test_few_long_rows(ctx):
+    long, even = _full(ctx, 8, 1 << 20), _full(ctx, 2896, 2896)
+    t = sp().spgemm_mat_transpose
+    assert _time(lambda: t(ctx, long)) < 2 * _time(lambda: t(ctx, even))
