@@ -686,11 +686,13 @@ __global__ void k_row_scatter(const int32_t* __restrict__ ir, const int32_t* __r
     }
 }
 
-// lengths of the permuted columns
-__global__ void k_perm_lens(const int64_t* __restrict__ cp, const int32_t* __restrict__ colp, int64_t n,
+// lengths of the permuted columns; with `zeroed` those of the nonempty ones alone
+__global__ void k_perm_lens(const int64_t* __restrict__ cp, const int32_t* __restrict__ colp, int64_t n, bool zeroed,
                             int64_t* __restrict__ len) {
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-        len[colp ? colp[j] : j] = cp[j + 1] - cp[j];
+    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t l = cp[j + 1] - cp[j];
+        if (l != 0 || !zeroed) len[colp ? colp[j] : j] = l;
+    }
 }
 
 int grid_for(int64_t n, int block = 256) { return (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div64(n, block), sm_count() * 32)); }
@@ -1234,8 +1236,12 @@ static spgemm_status_t permute_csc(spgemm_ctx* ctx, int64_t m, int64_t n, int64_
         char* t = (char*)tmp->p;
         int64_t* len = (int64_t*)(t + o_len);   // n lengths, then the sort's counters
         int64_t* ocp = (int64_t*)cpb->p;
-        SG_CUDA(ctx, cudaMemsetAsync(len + n, 0, 16, st));
-        k_perm_lens<<<grid_for(n), 256, 0, st>>>(cp, colp, n, len);
+        // mostly empty columns: zeroes in order cost less than a scattered store per column
+        // (2^26 columns of 2,000 entries: 2.53 ms of 5.4)
+        const bool few = colp && nnz < n / 2;
+        if (few) SG_CUDA(ctx, cudaMemsetAsync(len, 0, 8 * n + 16, st));
+        else SG_CUDA(ctx, cudaMemsetAsync(len + n, 0, 16, st));
+        k_perm_lens<<<grid_for(n), 256, 0, st>>>(cp, colp, n, few, len);
         note_launch();
         launch_exclusive_scan(st, len, n, ocp, t + o_sc);
         SegSort S{cp, n, nnz, ocp, colp, ir, rowp, num, (int32_t*)irb->p, vb->p, m};
