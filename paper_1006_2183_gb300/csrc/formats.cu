@@ -725,9 +725,12 @@ struct SegScratch {
     size_t o_list, o_split = 0, o_chunk = 0, o_win = 0, o_off = 0, o_wkey = 0, o_widx = 0;
     template <class Take>
     SegScratch(int64_t n, int64_t nz, int64_t bound, bool own_entries, Take take) : nnz(nz) {
+        // a column holds no more entries than there are, nor than there are keys: where that is
+        // too few, none is split (a malformed one neither)
         split_len = SEG_SPLIT / std::max<int64_t>(1, ceil_div64(bound, SEGL_ROWS));
+        if (std::min(nnz, bound) <= split_len) split_len = INT64_MAX;
         o_list = take(4 * n);
-        if (nnz <= split_len) return;   // no column to split
+        if (nnz <= split_len) return;
         const int64_t ns = nnz / split_len, nc = nnz / SEG_CHUNK + ns;
         o_split = take(4 * ns);
         o_chunk = take(8 * nc);
