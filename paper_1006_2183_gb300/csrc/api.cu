@@ -593,16 +593,16 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         dw.err = (int*)(slab_ctr + 3);
         unsigned long long* store_bound = slab_ctr + 4;
         dw.RB = E->cfg.dense_rows;
-        dw.quads = true;
-        for (const Prod& pr : E->hprods) dw.quads = dw.quads && slab_quads(pr);
         launch_dense_items(st, E->it, dw.dlist, nd, E->flops, E->cfg.part_flops, dw.RB, (int2*)dw.items,
                            slab_ctr + 1, (int8_t*)dw.nparts, (int32_t*)dw.sbase, store_bound,
-                           (int64_t*)dw.bbase, bnd_total);
-        unsigned long long hs[3] = {0, 0, 0};
+                           (int64_t*)dw.bbase, bnd_total, slab_ctr + 7);
+        unsigned long long hs[4] = {0, 0, 0, 0};
         SG_TRY(read_back(ctx, &hs[0], slab_ctr + 1, 8));
         SG_TRY(read_back(ctx, &hs[1], store_bound, 8));
         SG_TRY(read_back(ctx, &hs[2], bnd_total, 8));
+        SG_TRY(read_back(ctx, &hs[3], slab_ctr + 7, 8));
         SG_TRY(sync_ctx(ctx));
+        dw.kinds = (int)hs[3];
         dw.nslabs = (int64_t)hs[0];
         dw.store_cap = (int64_t)hs[1];
         off = 0;

@@ -1173,6 +1173,13 @@ __host__ __device__ __forceinline__ int64_t slab_max_rows(int64_t m, int P) {
     return mx;
 }
 
+// the quad walk applies to a product whose A is a CSC (no DCSC index, no gaps) of fewer than
+// 2^31 entries with 16-byte aligned row and value arrays
+__device__ __forceinline__ bool quads_ok(const Prod* pr) {
+    return pr->A.jc == nullptr && pr->A.ce == nullptr && pr->A.nnz < INT_MAX - 8 && ((uintptr_t)pr->A.ir & 15) == 0 &&
+           ((uintptr_t)pr->A.num & 15) == 0;
+}
+
 // Slabs of the long columns: P per column, items[sbase[d] + q] = (d, q); the
 // storage bound of the slab row sets, sum over columns of min(flops, words),
 // accumulates in *store_bound (a slab stores min(words, rows) 4-byte entries and
@@ -1182,11 +1189,12 @@ __host__ __device__ __forceinline__ int64_t slab_max_rows(int64_t m, int P) {
 __global__ void k_dense_items(Items it, const int2* __restrict__ dlist, int64_t nd, const int64_t* __restrict__ flops,
                               int part_flops, int RB, int2* items, unsigned long long* nitems, int8_t* nparts,
                               int32_t* sbase, unsigned long long* store_bound, int64_t* bbase,
-                              unsigned long long* bnd_total) {
+                              unsigned long long* bnd_total, unsigned long long* kinds) {
     const int64_t d = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     const bool ok = d < nd;
     long long P = 0, bound = 0, bnd = 0;
+    unsigned kind = 0;
     if (ok) {
         const int2 e = dlist[d];
         const Prod* pr = it.prods + e.x;
@@ -1209,13 +1217,16 @@ __global__ void k_dense_items(Items it, const int2* __restrict__ dlist, int64_t 
         // boundary table: P + 1 rows of deg positions (where each slab starts in every A(:,k)),
         // then two rows with where every A(:,k) starts (low and high 32 bits)
         bnd = (P + 3) * deg;
+        kind = quads_ok(pr) ? 1u : 2u;
     }
+    kind = __reduce_or_sync(0xffffffffu, kind);
     const long long ip = warp_incl_scan64(P), ib = warp_incl_scan64(bnd), sb = warp_sum(bound);
     unsigned long long bp = 0, bb = 0;
     if (lane == 31) {
         bp = atomicAdd(nitems, (unsigned long long)ip);
         bb = atomicAdd(bnd_total, (unsigned long long)ib);
         atomicAdd(store_bound, (unsigned long long)sb);
+        if ((*(volatile unsigned long long*)kinds & kind) != kind) atomicOr(kinds, (unsigned long long)kind);
     }
     bp = __shfl_sync(0xffffffffu, bp, 31);
     bb = __shfl_sync(0xffffffffu, bb, 31);
@@ -1230,10 +1241,11 @@ __global__ void k_dense_items(Items it, const int2* __restrict__ dlist, int64_t 
 void launch_dense_items(cudaStream_t st, const Items& it, const int2* dense_list, int64_t ndense, const int64_t* flops,
                         int part_flops, int RB, int2* items, unsigned long long* nitems, int8_t* nparts,
                         int32_t* sbase, unsigned long long* store_bound, int64_t* bbase,
-                        unsigned long long* bnd_total) {
+                        unsigned long long* bnd_total, unsigned long long* kinds) {
     if (ndense == 0) return;
     k_dense_items<<<(int)ceil_div64(ndense, 256), 256, 0, st>>>(it, dense_list, ndense, flops, part_flops, RB, items,
-                                                               nitems, nparts, sbase, store_bound, bbase, bnd_total);
+                                                               nitems, nparts, sbase, store_bound, bbase, bnd_total,
+                                                               kinds);
     note_launch();
 }
 
@@ -1559,13 +1571,6 @@ __device__ __forceinline__ void slab_products(const Prod* pr, int64_t bs, int64_
     }
 }
 
-// the quad walk applies to a product whose A is a CSC (no DCSC index, no gaps) of fewer than
-// 2^31 entries with 16-byte aligned row and value arrays
-__host__ __device__ __forceinline__ bool quads_ok(const Prod* pr) {
-    return pr->A.jc == nullptr && pr->A.ce == nullptr && pr->A.nnz < INT_MAX - 8 && ((uintptr_t)pr->A.ir & 15) == 0 &&
-           ((uintptr_t)pr->A.num & 15) == 0;
-}
-
 // the semiring whose slabs add up in shared memory
 constexpr bool slab_local(int sr) { return sr == SPGEMM_MIN_PLUS_F32; }
 // shared memory of the numeric pass before its accumulators
@@ -1578,9 +1583,10 @@ int slab_acc_entries(int sr, int RB) {
     return (int)((SLAB_SMEM - slab_num_bytes(RB)) / sizeof(MP32::Acc));
 }
 
-// Symbolic slab kernel: mark, count, store the row set.
+// Symbolic slab kernel: mark, count, store the row set.  `mixed`: only the products that QUADS is
+// for; a launch of the other form takes the rest.
 template <bool QUADS>
-__global__ void __launch_bounds__(RT_BLOCK, 4) k_slab_sym(Items it, DenseWork dw) {
+__global__ void __launch_bounds__(RT_BLOCK, 4) k_slab_sym(Items it, DenseWork dw, bool mixed) {
     extern __shared__ __align__(16) unsigned char smem[];
     SegSmem* sc = reinterpret_cast<SegSmem*>(smem);
     uint32_t* bitmap = reinterpret_cast<uint32_t*>(smem + RS_BYTES);
@@ -1601,6 +1607,7 @@ __global__ void __launch_bounds__(RT_BLOCK, 4) k_slab_sym(Items it, DenseWork dw
                        reinterpret_cast<const int4*>(dw.rec + w + gridDim.x) + tid);
         const SlabRec& rc = s_rec[k];
         const Prod* pr = it.prods + rc.prod;
+        if (mixed && quads_ok(pr) != QUADS) continue;
         const int64_t R0 = rc.r0, R1 = rc.r1;
         const int nw = (int)((R1 - R0 + 31) >> 5);
         const int ng = (nw + 3) >> 2;   // groups of 4 words (the bitmap is padded to whole groups)
@@ -1704,7 +1711,7 @@ __global__ void __launch_bounds__(RT_BLOCK, 4) k_slab_sym(Items it, DenseWork dw
 template <class SR, bool QUADS>
 __global__ void __launch_bounds__(RT_BLOCK, slab_local(SR::id) ? 2 : 4) k_slab_num(Items it, DenseWork dw, const int64_t* __restrict__ Coff,
                                                           int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv,
-                                                          int acc_cap) {
+                                                          int acc_cap, bool mixed) {
     using T = typename SR::T;
     using Acc = typename SR::Acc;
     constexpr bool LOCAL = slab_local(SR::id);
@@ -1735,6 +1742,7 @@ __global__ void __launch_bounds__(RT_BLOCK, slab_local(SR::id) ? 2 : 4) k_slab_n
         // only with malformed input, reported by the symbolic pass) is skipped
         if (cnt == 0 || rc.soff < 0) continue;
         const Prod* pr = it.prods + rc.prod;
+        if (mixed && quads_ok(pr) != QUADS) continue;
         const int64_t R0 = rc.r0, R1 = rc.r1;
         const int nw = (int)((R1 - R0 + 31) >> 5);
         const int ng = (nw + 3) >> 2;
@@ -1892,8 +1900,6 @@ __global__ void k_slab_fin(DenseWork dw, const int64_t* __restrict__ Coff) {
         dw.rec[w].ob = __ldg(Coff + dw.rec[w].u) + dw.spref[w];
 }
 
-bool slab_quads(const Prod& pr) { return quads_ok(&pr); }
-
 // CTAs per SM the kernel can keep resident with `smem` bytes, times the SM count
 static int resident_grid(const void* fn, int block, size_t smem) {
     int per_sm = 0;
@@ -1915,21 +1921,28 @@ static void run_slabs(const Lanes& lanes, const Items& it, const DenseWork& dw, 
         k_slab_bounds<<<(int)std::min<int64_t>(nslab_max, sm_count() * (2048 / bnd_block)), bnd_block, 0, st>>>(it, dw);
         note_launch();
         const size_t smem = RS_BYTES + (size_t)(dw.RB / 128 + 1) * 16;
-        auto kern = dw.quads ? k_slab_sym<true> : k_slab_sym<false>;
-        smem_at_least((const void*)kern, smem);
-        const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)kern, RT_BLOCK, smem));
-        kern<<<grid, RT_BLOCK, smem, st>>>(it, dw);
+        for (int kind = 0; kind < 2; ++kind) {
+            if (!((dw.kinds >> kind) & 1)) continue;
+            auto kern = kind == 0 ? k_slab_sym<true> : k_slab_sym<false>;
+            smem_at_least((const void*)kern, smem);
+            const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)kern, RT_BLOCK, smem));
+            kern<<<grid, RT_BLOCK, smem, st>>>(it, dw, dw.kinds == 3);
+            note_launch();
+        }
     } else {
         k_slab_fin<<<(int)std::min<int64_t>(ceil_div64(nslab_max, 256), sm_count() * 8), 256, 0, st>>>(dw, Coff);
         note_launch();
         const int acc_cap = slab_acc_entries(SR::id, dw.RB);
         const size_t smem = slab_num_bytes(dw.RB) + (size_t)acc_cap * sizeof(typename SR::Acc);
-        auto kern = dw.quads ? k_slab_num<SR, true> : k_slab_num<SR, false>;
-        smem_at_least((const void*)kern, smem);
-        const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)kern, RT_BLOCK, smem));
-        kern<<<grid, RT_BLOCK, smem, st>>>(it, dw, Coff, Cir, Cv, acc_cap);
+        for (int kind = 0; kind < 2; ++kind) {
+            if (!((dw.kinds >> kind) & 1)) continue;
+            auto kern = kind == 0 ? k_slab_num<SR, true> : k_slab_num<SR, false>;
+            smem_at_least((const void*)kern, smem);
+            const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)kern, RT_BLOCK, smem));
+            kern<<<grid, RT_BLOCK, smem, st>>>(it, dw, Coff, Cir, Cv, acc_cap, dw.kinds == 3);
+            note_launch();
+        }
     }
-    note_launch();
 }
 
 template <class SR>

@@ -106,7 +106,7 @@ struct DenseWork {
     SlabRec* rec = nullptr;               // per slab: its record
     int* err = nullptr;                   // nonzero: a capacity was exceeded
     int RB = 1 << 19;                     // most rows per slab
-    bool quads = false;                   // every A_i can be read in aligned quads (slab_quads)
+    int kinds = 0;                        // bit 0: some long column's A is read in aligned quads, bit 1: some is not
     // block mode (every A_i has at most BLOCK_TIER_MAX_ROWS rows): long columns
     // are counted with row bitmaps and computed by the block tier; no slabs
     bool dcol = false;
@@ -214,15 +214,14 @@ void launch_count_scan(cudaStream_t st, const Items& it, TierCfg cfg, const uint
                        const int32_t* item_prod, const int64_t* nnz_item, int64_t* out, void* tmp, uint8_t* nbin,
                        unsigned long long* cnt, int2* list);
 // slabs of the long columns (position d in the dense list, slab q); P_d slabs of at
-// most RB rows each; *store_bound accumulates the entries their row sets can need
+// most RB rows each; *store_bound accumulates the entries their row sets can need, *kinds
+// the bits of DenseWork::kinds
 void launch_dense_items(cudaStream_t st, const Items& it, const int2* dense_list, int64_t ndense,
                         const int64_t* flops, int part_flops, int RB, int2* items, unsigned long long* nitems,
                         int8_t* nparts, int32_t* sbase, unsigned long long* store_bound, int64_t* bbase,
-                        unsigned long long* bnd_total);
+                        unsigned long long* bnd_total, unsigned long long* kinds);
 // entries that a slab of at most RB rows can add up in shared memory (0: semirings without)
 int slab_acc_entries(int sr, int RB);
-// whether A of the product can be read in aligned quads by the slab passes
-bool slab_quads(const Prod& pr);
 // *flag = 1 when an operand of some product stores a false value (boolean semiring)
 void launch_false_values(cudaStream_t st, const Items& it, int* flag);
 // *flag = 1 when one of the n bytes at vals is 0 (vals == nullptr: nothing)
