@@ -108,8 +108,9 @@ typedef struct {
                                  4096).  -1 (default) = automatic: 4096 for operands of
                                  at most 32768 rows, 1024 for larger ones.            */
     int dense_part_flops;     /* slab tier: target flops per row slab of a long column
-                                 (default 65536); a column whose B column is long gets
-                                 fewer, larger slabs                                    */
+                                 (default 65536, for min-plus then about 25000 to 45000
+                                 where a slab adds up in shared memory); a column whose
+                                 B column is long gets fewer, larger slabs              */
     float predictor_margin;   /* capacity = (1 + margin) * prediction (+ slack)        */
     int range_table_slots;    /* ignored (kept for the layout of this struct)          */
     int block_kernel;         /* spgemm_summa_blocked stage products: 0 = the column

@@ -430,10 +430,14 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         }
     }
     E->cfg.part_flops = std::max(1024, opts.dense_part_flops);
-    // slabs that add up in shared memory: about twice as many products as it has accumulators
-    // (R-MAT 18 min-plus: 11.0 / 10.6 / 10.5 / 10.6 ms at 1, 1.5, 2 and 4 times as many)
-    if (const int acc = slab_acc_entries(sr, E->cfg.dense_rows))
-        E->cfg.part_flops = std::min(E->cfg.part_flops, std::max(2 * acc, 8192));
+    // slabs that add up in shared memory, unless the caller chose: about twice as many products as
+    // it has accumulators (R-MAT 18 min-plus, 14,424 of them: 9.30 ms, 10.05 at 8,192 products,
+    // 9.38 at 65,536, 9.55 at 131,072).  Slabs of so many rows that fewer than 12,288 are left
+    // keep the default, as most of their columns would not fit anyway (R-MAT 20, 11,012: 56.6
+    // against 55.0 ms; 4,184: 60.5 against 56.1; 600,000 vertices, 12,944: 22.0 against 22.1)
+    const int sums = slab_acc_entries(sr, E->cfg.dense_rows);
+    if (sums >= 12288 && opts.dense_part_flops == DEFAULT_PART_FLOPS)
+        E->cfg.part_flops = std::min(E->cfg.part_flops, 2 * sums);
     cudaStream_t st = ctx->stream;
     {
         const cudaError_t pending = cudaGetLastError();
