@@ -553,7 +553,7 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
     SG_TRY(sync_ctx(ctx));
     E->err_dev = (const int*)(slab_ctr + 3);
     int64_t acc = 0;
-    for (int b = 0; b <= NBIN; ++b)
+    for (int b = 0; b <= CTR_SORT2; ++b)
         for (int r = 1; r < CTR_REP; ++r) hc[b] += hc[r * CTR_STRIDE + b];
     for (int b = 0; b < NBIN; ++b) {
         E->bin_cnt[b] = (int64_t)hc[b];
@@ -561,6 +561,7 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         acc += E->bin_cnt[b];
     }
     E->flops_total = (int64_t)hc[NBIN];
+    E->sort2_cols = (int64_t)hc[CTR_SORT2];
     const int64_t nd = E->bin_cnt[BIN_DENSE];
     E->dw = DenseWork();
     if (nd > 0 && E->it.max_m <= BLOCK_TIER_MAX_ROWS) {
@@ -854,7 +855,9 @@ spgemm_status_t spgemm_plan_stats(spgemm_plan_t P, int64_t* flops, int64_t* nnz_
     if (nnz_C) *nnz_C = E.nnz_total;
     if (tiers4) {
         for (int t = 0; t < 4; ++t) tiers4[t] = 0;
-        for (int b = 0; b < NBIN; ++b) tiers4[tier_of_bin(b)] += E.bin_cnt[b];
+        for (int b = 0; b < NBIN; ++b) tiers4[tier_of_bin(b, 0, 0)] += E.bin_cnt[b];
+        tiers4[1] -= E.sort2_cols;   // sorted, but longer than warp_max_flops
+        tiers4[2] += E.sort2_cols;
     }
     if (overflow) *overflow = E.overflow_items;
     return SPGEMM_OK;
@@ -868,7 +871,7 @@ spgemm_status_t spgemm_plan_tier_stats(spgemm_plan_t P, int64_t* cols4, int64_t*
     if (!buf) return set_err(ctx, SPGEMM_ERR_OOM, "tier stats");
     SG_CUDA(ctx, cudaMemsetAsync(buf->p, 0, 128, ctx->stream));
     launch_tier_stats(ctx->stream, P->E.it, P->E.bin, P->E.item_prod, P->E.flops, P->E.nnz_item,
-                      (unsigned long long*)buf->p);
+                      P->E.cfg.warp_max, (unsigned long long*)buf->p);
     unsigned long long h[16];
     SG_TRY(read_back(ctx, h, buf->p, 128));
     SG_TRY(sync_ctx(ctx));

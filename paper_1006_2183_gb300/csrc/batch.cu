@@ -252,14 +252,17 @@ spgemm_status_t spgemm_autotune(spgemm_ctx_t ctx, int count, const spgemm_mat_t*
                                 spgemm_semiring_t sr, spgemm_opts_t* opts) {
     if (!ctx || !opts) return SPGEMM_ERR_INVALID_ARG;
     int64_t fl = 0;
+    bool warp_matters = true;
     {
-        // total flops class of the batch
+        // total flops class of the batch; whether warp_max_flops moves a column to another
+        // kernel: not where the sort tier takes all it could, nor in the block tier
         std::unique_ptr<struct spgemm_plan> P(new struct spgemm_plan());
         P->ctx = ctx;
         std::vector<Prod> prods;
         SG_TRY(collect_prods(ctx, count, A, B, sr, &prods, &P->convs));
         SG_TRY(engine_setup(&P->E, ctx, sr, *opts, prods, false));
         fl = P->E.flops_total;
+        warp_matters = P->E.cfg.sort_max < 512 && P->E.it.max_m > BLOCK_TIER_MAX_ROWS;
     }
     int lg = 0;
     while ((int64_t(1) << lg) < fl && lg < 62) ++lg;
@@ -278,6 +281,7 @@ spgemm_status_t spgemm_autotune(spgemm_ctx_t ctx, int count, const spgemm_mat_t*
         for (int wm : warp_c)
             for (int bm : block_c)
                 for (int pf : part_c) {
+                    if (!warp_matters && wm != 512) continue;
                     spgemm_opts_t o = *opts;
                     o.warp_max_flops = wm;
                     o.block_max_flops = bm;

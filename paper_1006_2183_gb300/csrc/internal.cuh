@@ -115,6 +115,7 @@ struct Engine {
     bool numeric_bins = false;
     bool slab_rows_short = false;        // a column of the largest m would need > MAX_PARTS slabs
     int64_t flops_total = 0;
+    int64_t sort2_cols = 0;              // columns of the sort bins beyond warp_max_flops
     int64_t nnz_total = -1;
     bool symbolic_done = false;
     bool want_prod_off = false;          // the symbolic pass also returns every product's first output

@@ -114,7 +114,7 @@ __host__ __device__ __forceinline__ int bin_of(int64_t flops, int64_t cap, int w
                                               int sort_max) {
     if (cap <= 0) return 0;
     if (flops <= TINY_MAX) return BIN_SORT0;
-    if (flops <= sort_max && cap <= (flops <= 512 ? warp_max : block_max)) {
+    if (flops <= sort_max && cap <= block_max) {   // block_max is no smaller than warp_max
         int b = BIN_SORT0 + 1;
         for (int64_t t = 2 * TINY_MAX; t < flops; t <<= 1) ++b;
         return b;
@@ -181,13 +181,15 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
                                                  int64_t* __restrict__ maxlen, int64_t* __restrict__ nnz_item) {
     constexpr int GRP = 256 / LPI;   // items of this CTA
     __shared__ unsigned long long s_cnt[NBIN];
-    __shared__ unsigned long long s_fl;
+    __shared__ unsigned long long s_fl, s_sort2;
     __shared__ int s_nlong;
     __shared__ int s_long[GRP];                                              // groups with a long column
     __shared__ unsigned long long s_lf[GRP], s_lmx[GRP], s_lsk[GRP];         // their totals
     if (threadIdx.x < NBIN) s_cnt[threadIdx.x] = 0;
-    if (threadIdx.x == 0) s_fl = 0;
-    if (threadIdx.x == 0) s_nlong = 0;
+    if (threadIdx.x == 0) {
+        s_fl = s_sort2 = 0;
+        s_nlong = 0;
+    }
     __syncthreads();
     const int sub = threadIdx.x & (LPI - 1), grp = threadIdx.x / LPI;
     const int64_t u = (int64_t)blockIdx.x * GRP + grp;
@@ -309,6 +311,8 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
         const unsigned peers = __match_any_sync(0xffffffffu, b);
         const int lane = threadIdx.x & 31;
         if (has && lane == __ffs(peers) - 1) atomicAdd(&s_cnt[b], (unsigned long long)__popc(peers));
+        const unsigned over = __ballot_sync(0xffffffffu, b > BIN_SORT0 && b < BIN_WARP0 && cap > cfg.warp_max);
+        if (lane == 0 && over) atomicAdd(&s_sort2, (unsigned long long)__popc(over));
         unsigned long long fs = has ? (unsigned long long)f : 0ull;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) fs += __shfl_xor_sync(0xffffffffu, fs, o);
@@ -343,6 +347,7 @@ __global__ void __launch_bounds__(256) k_analyze(Items it, TierCfg cfg, int64_t*
     const int rep = (blockIdx.x & (CTR_REP - 1)) * CTR_STRIDE;
     if (threadIdx.x < NBIN && s_cnt[threadIdx.x]) atomicAdd(bin_count + rep + threadIdx.x, s_cnt[threadIdx.x]);
     if (threadIdx.x == 0 && flops_total) atomicAdd(flops_total + rep, s_fl);
+    if (threadIdx.x == 32 && s_sort2) atomicAdd(bin_count + rep + CTR_SORT2, s_sort2);
 }
 
 // item_prod[u] = the product of item u: one CTA per product over its contiguous items.
@@ -2078,7 +2083,7 @@ void launch_fill_i64(cudaStream_t st, int64_t* p, int64_t n, int64_t v) {
 }
 
 __global__ void k_tier_stats(Items it, const uint8_t* __restrict__ bin, const int32_t* __restrict__ item_prod,
-                             const int64_t* __restrict__ flops, const int64_t* __restrict__ nnz_item,
+                             const int64_t* __restrict__ flops, const int64_t* __restrict__ nnz_item, int warp_max,
                              unsigned long long* out) {
     __shared__ unsigned long long s[16];
     if (threadIdx.x < 16) s[threadIdx.x] = 0;
@@ -2086,9 +2091,9 @@ __global__ void k_tier_stats(Items it, const uint8_t* __restrict__ bin, const in
     for (int64_t u = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; u < it.nitems;
          u += (int64_t)gridDim.x * blockDim.x) {
         int b = bin[u];
-        int t = tier_of_bin(b);
         int prod = item_prod[u];
         const Prod* pr = it.prods + prod;
+        int t = tier_of_bin(b, min(flops[u], pr->A.m), warp_max);
         int64_t p = u - __ldg(it.item_base + prod);
         atomicAdd(&s[t], 1ull);
         atomicAdd(&s[4 + t], (unsigned long long)flops[u]);
@@ -2100,10 +2105,10 @@ __global__ void k_tier_stats(Items it, const uint8_t* __restrict__ bin, const in
 }
 
 void launch_tier_stats(cudaStream_t st, const Items& it, const uint8_t* bin, const int32_t* item_prod,
-                       const int64_t* flops, const int64_t* nnz_item, unsigned long long* out) {
+                       const int64_t* flops, const int64_t* nnz_item, int warp_max, unsigned long long* out) {
     if (it.nitems <= 0) return;
     int grid = (int)std::min<int64_t>(ceil_div64(it.nitems, 256), sm_count() * 4);
-    k_tier_stats<<<grid, 256, 0, st>>>(it, bin, item_prod, flops, nnz_item, out);
+    k_tier_stats<<<grid, 256, 0, st>>>(it, bin, item_prod, flops, nnz_item, warp_max, out);
     note_launch();
 }
 

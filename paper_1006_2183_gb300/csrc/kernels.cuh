@@ -29,9 +29,9 @@ constexpr int BIN_WARP0 = BIN_SORT0 + NSORT;
 constexpr int BIN_BLK0 = BIN_WARP0 + NWARP;
 constexpr int BIN_DENSE = NBIN - 1;
 // Tier of a bin in the plan's statistics: 0 empty, 1 up to warp_max_flops, 2 up to
-// block_max_flops, 3 long columns.  The last sort bin holds columns beyond 512 products.
-__host__ __device__ constexpr int tier_of_bin(int b) {
-    return b == 0 ? 0 : b >= BIN_DENSE ? 3 : b >= BIN_BLK0 || b == BIN_WARP0 - 1 ? 2 : 1;
+// block_max_flops, 3 long columns.  A sort bin holds columns of both kinds: `cap` tells.
+__host__ __device__ constexpr int tier_of_bin(int b, int64_t cap, int warp_max) {
+    return b == 0 ? 0 : b >= BIN_DENSE ? 3 : b >= BIN_BLK0 || (b > BIN_SORT0 && b < BIN_WARP0 && cap > warp_max) ? 2 : 1;
 }
 constexpr int TINY_MAX = 16;
 constexpr int WARP_TBL0 = 64;
@@ -52,14 +52,14 @@ constexpr int DEFAULT_PART_FLOPS = 65536;
 // copies of the analysis counters (bin counts, then total flops), two 128-byte lines each
 constexpr int CTR_REP = 16;
 constexpr int CTR_STRIDE = 32;
-static_assert(NBIN + 1 <= CTR_STRIDE, "a copy keeps to its lines");
+constexpr int CTR_SORT2 = NBIN + 1;   // after the total flops: columns of the sort bins that count as tier 2
+static_assert(CTR_SORT2 < CTR_STRIDE, "a copy keeps to its lines");
 
 struct TierCfg {
     int warp_max;     // cap <= warp_max -> warp tables (<= 512)
     int block_max;    // cap <= block_max -> CTA tables (<= 4096)
-    int sort_max = 0; // columns of at most this many products (and cap <= warp_max, or
-                      // <= block_max beyond 512 products) go to the sort tier:
-                      // sort_max_products(rows), less where another tier is faster
+    int sort_max = 0; // columns of at most this many products (and cap <= block_max) go to the
+                      // sort tier: sort_max_products(rows), less where another tier is faster
     int dense_rows;   // RB, most rows of one slab (bitmap bits in shared memory)
     int part_flops;   // target flops per slab of a long column
 };
@@ -270,7 +270,7 @@ void launch_exclusive_scan(cudaStream_t st, const int64_t* in, int64_t n, int64_
 void launch_fill_i64(cudaStream_t st, int64_t* p, int64_t n, int64_t v);
 // per-tier totals {cols, flops, nnz(C), nnz(B)} x 4 tiers into out[16] (device, zeroed by caller)
 void launch_tier_stats(cudaStream_t st, const Items& it, const uint8_t* bin, const int32_t* item_prod,
-                       const int64_t* flops, const int64_t* nnz_item, unsigned long long* out);
+                       const int64_t* flops, const int64_t* nnz_item, int warp_max, unsigned long long* out);
 
 
 // raises a kernel's dynamic shared-memory limit on the current device to at least `bytes`
