@@ -609,6 +609,8 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         SG_TRY(sync_ctx(ctx));
         dw.kinds = (int)hs[3];
         dw.nslabs = (int64_t)hs[0];
+        // a column of P slabs and deg entries has (P + 3) deg of the boundary table's positions
+        dw.many_short = 2 * dw.nslabs >= 3 * nd && (int64_t)hs[2] <= 64 * (dw.nslabs + 3 * nd);
         dw.store_cap = (int64_t)hs[1];
         off = 0;
         const int64_t ns1 = std::max<int64_t>(dw.nslabs, 1);

@@ -1258,10 +1258,12 @@ void launch_dense_items(cudaStream_t st, const Items& it, const int2* dense_list
 // entry t of B(:,j), where slab q starts inside A(:,k) (relative to the column's
 // start); row P holds A(:,k)'s length.  One CTA per slab, every search of the slab
 // in flight at once (the passes that read them no longer wait on search chains at
-// their barriers).  A slab is one chain of loads whatever its entries (29 on average at
-// R-MAT 20): half as many threads per CTA where there are very many slabs put twice as many
-// in flight (R-MAT 20 flat 3.7 -> 2.3 ms), but leave longer columns of B to fewer threads
-// (restriction, 20,000 slabs: 93 -> 173 us).
+// their barriers).  Where most columns are cut, most slabs search, and a search is one chain
+// of loads whatever the slab's entries: with up to 64 of them on average, CTAs of half as many
+// threads put twice as many slabs in flight.  256 against 128 threads: R-MAT 20 (four slabs per
+// column, 35 entries) 3.7 / 2.3 ms, R-MAT 19 (two, 39) 0.82 / 0.71 ms, A S^T of pairs at R-MAT 20
+// (four, 2) 25 / 16 us.  Columns of one slab search nothing, and their time is that of the longest
+// ones: R-MAT 18 (36 entries) 182 / 197 us, R-MAT 16 (31) 50 / 71 us, S (A S^T) (1,600) 91 / 172 us.
 __global__ void __launch_bounds__(256) k_slab_bounds(Items it, DenseWork dw) {
     const int64_t nsym = (int64_t)*dw.nitems;
     for (int64_t w = blockIdx.x; w < nsym; w += gridDim.x) {
@@ -1922,7 +1924,7 @@ static void run_slabs(const Lanes& lanes, const Items& it, const DenseWork& dw, 
     const cudaStream_t st = lanes.next();
     const int64_t nslab_max = dw.nslabs > 0 ? dw.nslabs : dw.ndense * MAX_PARTS;
     if (!numeric) {
-        const int bnd_block = nslab_max >= (1 << 19) ? 128 : 256;
+        const int bnd_block = dw.many_short ? 128 : 256;
         k_slab_bounds<<<(int)std::min<int64_t>(nslab_max, sm_count() * (2048 / bnd_block)), bnd_block, 0, st>>>(it, dw);
         note_launch();
         const size_t smem = RS_BYTES + (size_t)(dw.RB / 128 + 1) * 16;

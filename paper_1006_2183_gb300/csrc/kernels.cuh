@@ -106,6 +106,7 @@ struct DenseWork {
     SlabRec* rec = nullptr;               // per slab: its record
     int* err = nullptr;                   // nonzero: a capacity was exceeded
     int RB = 1 << 19;                     // most rows per slab
+    bool many_short = false;              // slabs of few entries of B, most columns cut into several
     int kinds = 0;                        // bit 0: some long column's A is read in aligned quads, bit 1: some is not
     // block mode (every A_i has at most BLOCK_TIER_MAX_ROWS rows): long columns
     // are counted with row bitmaps and computed by the block tier; no slabs
