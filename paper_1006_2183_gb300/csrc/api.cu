@@ -600,14 +600,14 @@ spgemm_status_t engine_setup(Engine* E, spgemm_ctx* ctx, spgemm_semiring_t sr, c
         dw.RB = E->cfg.dense_rows;
         launch_dense_items(st, E->it, dw.dlist, nd, E->flops, E->cfg.part_flops, dw.RB, (int2*)dw.items,
                            slab_ctr + 1, (int8_t*)dw.nparts, (int32_t*)dw.sbase, store_bound,
-                           (int64_t*)dw.bbase, bnd_total, slab_ctr + 7);
+                           (int64_t*)dw.bbase, bnd_total, np > 1 ? slab_ctr + 7 : nullptr);
         unsigned long long hs[4] = {0, 0, 0, 0};
         SG_TRY(read_back(ctx, &hs[0], slab_ctr + 1, 8));
         SG_TRY(read_back(ctx, &hs[1], store_bound, 8));
         SG_TRY(read_back(ctx, &hs[2], bnd_total, 8));
-        SG_TRY(read_back(ctx, &hs[3], slab_ctr + 7, 8));
+        if (np > 1) SG_TRY(read_back(ctx, &hs[3], slab_ctr + 7, 8));
         SG_TRY(sync_ctx(ctx));
-        dw.kinds = (int)hs[3];
+        dw.kinds = np > 1 ? (int)hs[3] : slab_quads(E->hprods[0]) ? 1 : 2;
         dw.nslabs = (int64_t)hs[0];
         // a column of P slabs and deg entries has (P + 3) deg of the boundary table's positions
         dw.many_short = 2 * dw.nslabs >= 3 * nd && (int64_t)hs[2] <= 64 * (dw.nslabs + 3 * nd);

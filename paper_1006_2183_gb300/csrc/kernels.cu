@@ -1180,7 +1180,7 @@ __host__ __device__ __forceinline__ int64_t slab_max_rows(int64_t m, int P) {
 
 // the quad walk applies to a product whose A is a CSC (no DCSC index, no gaps) of fewer than
 // 2^31 entries with 16-byte aligned row and value arrays
-__device__ __forceinline__ bool quads_ok(const Prod* pr) {
+__host__ __device__ __forceinline__ bool quads_ok(const Prod* pr) {
     return pr->A.jc == nullptr && pr->A.ce == nullptr && pr->A.nnz < INT_MAX - 8 && ((uintptr_t)pr->A.ir & 15) == 0 &&
            ((uintptr_t)pr->A.num & 15) == 0;
 }
@@ -1222,16 +1222,16 @@ __global__ void k_dense_items(Items it, const int2* __restrict__ dlist, int64_t 
         // boundary table: P + 1 rows of deg positions (where each slab starts in every A(:,k)),
         // then two rows with where every A(:,k) starts (low and high 32 bits)
         bnd = (P + 3) * deg;
-        kind = quads_ok(pr) ? 1u : 2u;
+        if (kinds) kind = quads_ok(pr) ? 1u : 2u;
     }
-    kind = __reduce_or_sync(0xffffffffu, kind);
+    if (kinds) kind = __reduce_or_sync(0xffffffffu, kind);
     const long long ip = warp_incl_scan64(P), ib = warp_incl_scan64(bnd), sb = warp_sum(bound);
     unsigned long long bp = 0, bb = 0;
     if (lane == 31) {
         bp = atomicAdd(nitems, (unsigned long long)ip);
         bb = atomicAdd(bnd_total, (unsigned long long)ib);
         atomicAdd(store_bound, (unsigned long long)sb);
-        if ((*(volatile unsigned long long*)kinds & kind) != kind) atomicOr(kinds, (unsigned long long)kind);
+        if (kinds) atomicOr(kinds, (unsigned long long)kind);
     }
     bp = __shfl_sync(0xffffffffu, bp, 31);
     bb = __shfl_sync(0xffffffffu, bb, 31);
@@ -1718,7 +1718,7 @@ __global__ void __launch_bounds__(RT_BLOCK, 4) k_slab_sym(Items it, DenseWork dw
 template <class SR, bool QUADS>
 __global__ void __launch_bounds__(RT_BLOCK, slab_local(SR::id) ? 2 : 4) k_slab_num(Items it, DenseWork dw, const int64_t* __restrict__ Coff,
                                                           int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv,
-                                                          int acc_cap, bool mixed) {
+                                                          int acc_cap) {
     using T = typename SR::T;
     using Acc = typename SR::Acc;
     constexpr bool LOCAL = slab_local(SR::id);
@@ -1746,10 +1746,10 @@ __global__ void __launch_bounds__(RT_BLOCK, slab_local(SR::id) ? 2 : 4) k_slab_n
         const SlabRec& rc = s_rec[kb];
         const int cnt = rc.cnt;
         // the same for every thread of the CTA; a row set that found no room (possible
-        // only with malformed input, reported by the symbolic pass) is skipped
+        // only with malformed input, reported by the symbolic pass) is skipped, and so is
+        // one that a launch of the other form takes (k_slab_fin)
         if (cnt == 0 || rc.soff < 0) continue;
         const Prod* pr = it.prods + rc.prod;
-        if (mixed && quads_ok(pr) != QUADS) continue;
         const int64_t R0 = rc.r0, R1 = rc.r1;
         const int nw = (int)((R1 - R0 + 31) >> 5);
         const int ng = (nw + 3) >> 2;
@@ -1900,12 +1900,19 @@ __global__ void __launch_bounds__(RT_BLOCK, slab_local(SR::id) ? 2 : 4) k_slab_n
     }
 }
 
-// Completes the slab records for the numeric pass: where each slab's rows start in C.
-__global__ void k_slab_fin(DenseWork dw, const int64_t* __restrict__ Coff) {
+// Completes the slab records for the numeric pass: where each slab's rows start in C.  With both
+// kinds of products (only_quads 0 or 1, else -1) the records of the other kind lose their row set
+// for the launch that follows.
+__global__ void k_slab_fin(Items it, DenseWork dw, const int64_t* __restrict__ Coff, int only_quads) {
     const int64_t nsym = (int64_t)*dw.nitems;
-    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nsym; w += (int64_t)gridDim.x * blockDim.x)
+    for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < nsym; w += (int64_t)gridDim.x * blockDim.x) {
         dw.rec[w].ob = __ldg(Coff + dw.rec[w].u) + dw.spref[w];
+        if (only_quads >= 0)
+            dw.rec[w].soff = quads_ok(it.prods + dw.rec[w].prod) == (only_quads != 0) ? dw.soff[w] : -1;
+    }
 }
+
+bool slab_quads(const Prod& pr) { return quads_ok(&pr); }
 
 // CTAs per SM the kernel can keep resident with `smem` bytes, times the SM count
 static int resident_grid(const void* fn, int block, size_t smem) {
@@ -1937,16 +1944,17 @@ static void run_slabs(const Lanes& lanes, const Items& it, const DenseWork& dw, 
             note_launch();
         }
     } else {
-        k_slab_fin<<<(int)std::min<int64_t>(ceil_div64(nslab_max, 256), sm_count() * 8), 256, 0, st>>>(dw, Coff);
-        note_launch();
         const int acc_cap = slab_acc_entries(SR::id, dw.RB);
         const size_t smem = slab_num_bytes(dw.RB) + (size_t)acc_cap * sizeof(typename SR::Acc);
         for (int kind = 0; kind < 2; ++kind) {
             if (!((dw.kinds >> kind) & 1)) continue;
+            k_slab_fin<<<(int)std::min<int64_t>(ceil_div64(nslab_max, 256), sm_count() * 8), 256, 0, st>>>(
+                it, dw, Coff, dw.kinds == 3 ? kind == 0 : -1);
+            note_launch();
             auto kern = kind == 0 ? k_slab_num<SR, true> : k_slab_num<SR, false>;
             smem_at_least((const void*)kern, smem);
             const int grid = (int)std::min<int64_t>(nslab_max, resident_grid((const void*)kern, RT_BLOCK, smem));
-            kern<<<grid, RT_BLOCK, smem, st>>>(it, dw, Coff, Cir, Cv, acc_cap, dw.kinds == 3);
+            kern<<<grid, RT_BLOCK, smem, st>>>(it, dw, Coff, Cir, Cv, acc_cap);
             note_launch();
         }
     }

@@ -216,13 +216,15 @@ void launch_count_scan(cudaStream_t st, const Items& it, TierCfg cfg, const uint
                        unsigned long long* cnt, int2* list);
 // slabs of the long columns (position d in the dense list, slab q); P_d slabs of at
 // most RB rows each; *store_bound accumulates the entries their row sets can need, *kinds
-// the bits of DenseWork::kinds
+// (may be null) the bits of DenseWork::kinds
 void launch_dense_items(cudaStream_t st, const Items& it, const int2* dense_list, int64_t ndense,
                         const int64_t* flops, int part_flops, int RB, int2* items, unsigned long long* nitems,
                         int8_t* nparts, int32_t* sbase, unsigned long long* store_bound, int64_t* bbase,
                         unsigned long long* bnd_total, unsigned long long* kinds);
 // entries that a slab of at most RB rows can add up in shared memory (0: semirings without)
 int slab_acc_entries(int sr, int RB);
+// whether A of the product can be read in aligned quads by the slab passes
+bool slab_quads(const Prod& pr);
 // *flag = 1 when an operand of some product stores a false value (boolean semiring)
 void launch_false_values(cudaStream_t st, const Items& it, int* flag);
 // *flag = 1 when one of the n bytes at vals is 0 (vals == nullptr: nothing)
