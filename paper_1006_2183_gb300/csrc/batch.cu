@@ -17,7 +17,21 @@ namespace {
 
 spgemm_status_t collect_prods(spgemm_ctx* ctx, int count, const spgemm_mat_t* A, const spgemm_mat_t* B,
                               spgemm_semiring_t sr, std::vector<Prod>* prods, std::vector<spgemm_mat_t>* convs,
-                              bool check = false) {
+                              bool check = false, std::vector<ValueRefresh>* refresh = nullptr) {
+    // a replayed plan takes the values of a CSR operand again each time
+    auto operand = [&](spgemm_mat_t M, DMat* d) -> spgemm_status_t {
+        spgemm_mat_t c = nullptr;
+        if (refresh && M->fmt == SPGEMM_FMT_CSR && M->num) {
+            ValueRefresh r;
+            SG_TRY(csr_to_csc_refreshed(ctx, M, &c, &r));
+            refresh->push_back(r);
+            *d = dmat_of(c);
+        } else {
+            SG_TRY(to_csc_operand(ctx, M, &c, d));
+        }
+        if (c) convs->push_back(c);
+        return SPGEMM_OK;
+    };
     if (count < 0 || (count > 0 && (!A || !B))) return set_err(ctx, SPGEMM_ERR_INVALID_ARG, "bad batch arrays");
     if (check) {
         std::vector<spgemm_mat*> ops;
@@ -33,11 +47,8 @@ spgemm_status_t collect_prods(spgemm_ctx* ctx, int count, const spgemm_mat_t* A,
         if (A[i]->sr != sr || B[i]->sr != sr) return set_err(ctx, SPGEMM_ERR_INVALID_ARG, "semiring of pair %d", i);
         if (A[i]->n != B[i]->m) return set_err(ctx, SPGEMM_ERR_DIM_MISMATCH, "pair %d: inner dimensions differ", i);
         Prod pr;
-        spgemm_mat_t ca = nullptr, cb = nullptr;
-        SG_TRY(to_csc_operand(ctx, A[i], &ca, &pr.A));
-        if (ca) convs->push_back(ca);
-        SG_TRY(to_csc_operand(ctx, B[i], &cb, &pr.B));
-        if (cb) convs->push_back(cb);
+        SG_TRY(operand(A[i], &pr.A));
+        SG_TRY(operand(B[i], &pr.B));
         prods->push_back(pr);
     }
     return SPGEMM_OK;
@@ -104,7 +115,8 @@ spgemm_status_t batch_plan_build(spgemm_ctx* ctx, int count, const spgemm_mat_t*
     P->opts = o;
     P->is_batch = true;
     std::vector<Prod> prods;
-    SG_TRY(collect_prods(ctx, count, A, B, sr, &prods, &P->convs, o.check_inputs != 0));
+    SG_TRY(collect_prods(ctx, count, A, B, sr, &prods, &P->convs, o.check_inputs != 0,
+                         run_numeric ? nullptr : &P->refresh));
     Engine& E = P->E;
     const bool learned = o.use_predictor && ctx->pred_ready && run_numeric;
     SG_TRY(engine_setup(&E, ctx, sr, o, prods, learned));
@@ -132,6 +144,7 @@ void numeric_launches(struct spgemm_plan* P) {
 }
 
 void all_numeric_launches(struct spgemm_plan* P) {
+    for (const ValueRefresh& r : P->refresh) refresh_values(P->ctx->stream, r);
     engine_false_values(&P->E);
     switch (P->sr) {
     case SPGEMM_PLUS_TIMES_F64: numeric_launches<PT64>(P); break;

@@ -189,6 +189,14 @@ __global__ void k_gather(const uint32_t* __restrict__ perm, const int32_t* __res
     }
 }
 
+template <int W>
+__global__ void k_take_values(const uint32_t* __restrict__ at, const void* __restrict__ vin, int64_t nnz,
+                              void* __restrict__ vout) {
+    using T = typename Word<W>::T;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += (int64_t)gridDim.x * blockDim.x)
+        reinterpret_cast<T*>(vout)[i] = reinterpret_cast<const T*>(vin)[at[i]];
+}
+
 // ---------------------------------------------------------------- sort within columns
 // Entries of every column put in ascending order of their (distinct) keys, for transpose and
 // permutation, where only the order within a column is unknown: one read and one write of the
@@ -1065,6 +1073,34 @@ spgemm_status_t transpose_csc(spgemm_ctx* ctx, int64_t m, int64_t n, int64_t nnz
     // the temporaries are released with the handle's first owner release; drop them now
     out->owned.pop_back();
     return SPGEMM_OK;
+}
+
+spgemm_status_t csr_to_csc_refreshed(spgemm_ctx* ctx, spgemm_mat_t M, spgemm_mat_t* conv, ValueRefresh* r) {
+    auto idx = ctx_buf(ctx, 4 * std::max<int64_t>(M->nnz, 1));
+    auto val = ctx_buf(ctx, sr_size(M->sr) * std::max<int64_t>(M->nnz, 1));
+    if (!idx || !val) return set_err(ctx, SPGEMM_ERR_OOM, "values of a CSR operand");
+    if (M->nnz > 0) {
+        k_iota_u32<<<grid_for(M->nnz), 256, 0, ctx->stream>>>((uint32_t*)idx->p, M->nnz);
+        note_launch();
+    }
+    std::unique_ptr<spgemm_mat> T(new spgemm_mat());
+    SG_TRY(transpose_csc(ctx, M->n, M->m, M->nnz, M->cp, M->ir, idx->p, 4, T.get()));
+    T->sr = M->sr;
+    *r = ValueRefresh{(const uint32_t*)T->num, M->num, val->p, M->nnz, sr_size(M->sr)};
+    T->num = val->p;
+    T->owned.push_back(val);
+    *conv = T.release();
+    return SPGEMM_OK;
+}
+
+void refresh_values(cudaStream_t st, const ValueRefresh& r) {
+    if (r.nnz <= 0) return;
+    switch (r.w) {
+    case 1: k_take_values<1><<<grid_for(r.nnz), 256, 0, st>>>(r.at, r.from, r.nnz, r.to); break;
+    case 4: k_take_values<4><<<grid_for(r.nnz), 256, 0, st>>>(r.at, r.from, r.nnz, r.to); break;
+    default: k_take_values<8><<<grid_for(r.nnz), 256, 0, st>>>(r.at, r.from, r.nnz, r.to); break;
+    }
+    note_launch();
 }
 
 spgemm_status_t make_dcsc(spgemm_ctx* ctx, const spgemm_mat* M, bool with_aux, spgemm_mat* out) {

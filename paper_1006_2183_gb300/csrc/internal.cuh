@@ -123,6 +123,15 @@ struct Engine {
     int64_t overflow_items = 0;
 };
 
+// CSC of a CSR operand whose values are taken again by refresh_values before every use
+struct ValueRefresh {
+    const uint32_t* at;   // entry i of the conversion is entry at[i] of the operand
+    const void* from;
+    void* to;
+    int64_t nnz;
+    size_t w;
+};
+
 struct spgemm_plan {
     spgemm_ctx* ctx = nullptr;
     spgemm_semiring_t sr;
@@ -133,6 +142,7 @@ struct spgemm_plan {
     // batch plans
     bool is_batch = false;
     std::vector<spgemm_mat_t> convs;                 // owned conversions of batch operands
+    std::vector<ValueRefresh> refresh;               // their values, taken again before a replay
     std::vector<int64_t> pm, pn, colbase, outoff;    // per product: dims, colptr base, first entry
     std::shared_ptr<DevBuf> out_cp, out_r, out_v;
     cudaGraph_t graph = nullptr;
@@ -185,6 +195,8 @@ spgemm_status_t upload(spgemm_ctx* ctx, void* dst, const void* src, size_t bytes
 spgemm_status_t check_handles(spgemm_ctx* ctx, const std::vector<spgemm_mat*>& mats);
 spgemm_status_t transpose_csc(spgemm_ctx* ctx, int64_t m, int64_t n, int64_t nnz, const int64_t* cp,
                               const int32_t* ir, const void* num, size_t w, spgemm_mat_t out_handle);
+spgemm_status_t csr_to_csc_refreshed(spgemm_ctx* ctx, spgemm_mat_t M, spgemm_mat_t* conv, ValueRefresh* r);
+void refresh_values(cudaStream_t st, const ValueRefresh& r);
 spgemm_status_t make_dcsc(spgemm_ctx* ctx, const spgemm_mat* csc, bool aux, spgemm_mat* out);
 // col[t] = the column of entry t of a CSC array
 void launch_expand_cols(cudaStream_t st, const int64_t* cp, int64_t n, int64_t nnz, int32_t* col);
