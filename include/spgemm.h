@@ -99,10 +99,13 @@ typedef struct {
                                  them (SPGEMM_ERR_UNSUPPORTED otherwise).              */
     int summa_merge_every;    /* staged mode: merge after this many stages (0 = after
                                  the last stage, the paper's buffered triples).        */
-    int warp_max_flops;       /* columns with flops <= this (at most 512) are sorted in
-                                 registers or use warp-wide hash tables                 */
+    int warp_max_flops;       /* columns with flops <= this (at most 512) use warp-wide
+                                 hash tables where they are not sorted                  */
     int block_max_flops;      /* columns with flops <= this are sorted (up to 1024
-                                 products) or use CTA-wide hash tables;
+                                 products of operands of at most 2^22 rows, fewer beyond;
+                                 up to 256 of operands of at most 32768 rows, whose
+                                 longer columns take row bitmaps) or use CTA-wide hash
+                                 tables;
                                  longer columns (the slab tier) are cut into row slabs,
                                  each counted and then accumulated by one CTA (at most
                                  4096).  -1 (default) = automatic: 4096 for operands of
