@@ -1715,6 +1715,9 @@ __global__ void __launch_bounds__(RT_BLOCK, 4) k_slab_sym(Items it, DenseWork dw
 // and store their values once: R-MAT 18 7.0 -> 6.0 ms.  Longer ones and the other semirings
 // add into C by L2 reductions: a shared FP64 addition is a compare-and-swap loop (three
 // times slower than the L2 at R-MAT 20), an int64 one two atomics (20 pairs 623 -> 726 us).
+// Min-plus keeps 64 registers and two CTAs per SM, the others 32 (FP64 and int64 spill 28 bytes,
+// boolean 20) and four, or three where a CTA takes more than 55 KB of shared memory (slabs beyond
+// about 273,000 rows).
 template <class SR, bool QUADS>
 __global__ void __launch_bounds__(RT_BLOCK, slab_local(SR::id) ? 2 : 4) k_slab_num(Items it, DenseWork dw, const int64_t* __restrict__ Coff,
                                                           int32_t* __restrict__ Cir, typename SR::T* __restrict__ Cv,

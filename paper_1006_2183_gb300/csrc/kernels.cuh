@@ -39,7 +39,7 @@ constexpr int BLK_TBL0 = 2048;
 // most row slabs of one long column
 constexpr int MAX_PARTS = 64;
 // default most rows of one slab: its row bitmap (and ranks) then leave room for four CTAs of
-// the counting pass per SM and three or four of the numeric pass.  R-MAT 20 flat FP64 with
+// the counting pass per SM and three (up to about 273,000 rows four) of the numeric pass.  R-MAT 20 flat FP64 with
 // one column cut at 2^19 / 2^18 / 2^17 rows: counting 31.3 / 25.3 / 32.3 ms, numeric 55.3 /
 // 51.2 / 56.2 ms; 300,007 rows are better whole than in two slabs (boolean 2.6 against 3.1 ms)
 constexpr int DEFAULT_SLAB_ROWS = 327680;
