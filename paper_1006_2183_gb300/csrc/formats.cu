@@ -242,6 +242,7 @@ constexpr int64_t SEGL_ROWS = 1 << 20;        // keys ranked at a time in a long
 // 118 us split and 165 whole, of 256 such columns 341 and 331, of 512 columns of 16,384 entries
 // 323 and 289.
 constexpr int64_t SEG_SPLIT = 16384;
+constexpr int64_t SEG_WHOLE = 65536;
 constexpr int SEG_CHUNK = 8192;
 constexpr int SEG_WIN = 256;
 constexpr int SEG_WIN_KEYS = 1 << 15;         // 256 windows of it hold the 2^23 keys
@@ -589,10 +590,10 @@ constexpr int RP_HOT = 8;
 constexpr int RP_LOG = 11;                  // slots of the sampled rows: half of them stay free
 constexpr int RP_HLOG = 7;                  // the rows counted in shared memory, four to a hash value
 constexpr int RP_SLOTS = 4 << RP_HLOG;
-constexpr int64_t RP_MIN = 1 << 16;         // no counter of fewer entries queues for long
+constexpr int64_t RP_MIN = 1 << 18;         // no counter of fewer entries queues for long
 
-// zeroes n counters; CTA 0 looks for the rows to count in shared memory: hot[slot], -1 where
-// there is none, and hot[RP_SLOTS] whether there is any
+// Zeroes n counters; CTA 0 looks for the rows to count in shared memory (nnz > 0): hot[slot], -1
+// where there is none, and hot[RP_SLOTS] whether there is any.
 __global__ void __launch_bounds__(RP_SAMPLES) k_row_begin(unsigned long long* __restrict__ cnt, int64_t n,
                                                           const int32_t* __restrict__ ir, int64_t nnz, int64_t m,
                                                           int32_t* __restrict__ hot) {
@@ -607,24 +608,22 @@ __global__ void __launch_bounds__(RP_SAMPLES) k_row_begin(unsigned long long* __
     }
     for (int i = tid; i < RP_SLOTS + 1; i += RP_SAMPLES) s_hot[i] = i < RP_SLOTS ? -1 : 0;
     __syncthreads();
-    if (nnz >= RP_MIN) {
-        uint32_t x = (uint32_t)tid * 0x9E3779B1u;   // scattered: an even step could meet one row every time
-        x ^= x >> 15;
-        x *= 0x85EBCA6Bu;
-        x ^= x >> 13;
-        const int32_t r = ir[(int64_t)(((uint64_t)x * (uint64_t)nnz) >> 32)];
-        if (r >= 0 && r < m) {
-            uint32_t h = hash_row(r) >> (32 - RP_LOG);
-            while (true) {
-                const int held = atomicCAS(s_row + h, -1, r);
-                if (held == -1 || held == r) break;
-                h = (h + 1) & ((1 << RP_LOG) - 1);
-            }
-            if (atomicAdd(s_seen + h, 1) == RP_HOT - 1) {
-                s_hot[RP_SLOTS] = 1;
-                int* q = s_hot + 4 * (hash_row(r) >> (32 - RP_HLOG));
-                for (int i = 0; i < 4 && atomicCAS(q + i, -1, r) != -1; ++i) {}   // a fifth is not counted there
-            }
+    uint32_t x = (uint32_t)tid * 0x9E3779B1u;   // scattered: an even step could meet one row every time
+    x ^= x >> 15;
+    x *= 0x85EBCA6Bu;
+    x ^= x >> 13;
+    const int32_t r = ir[(int64_t)(((uint64_t)x * (uint64_t)nnz) >> 32)];
+    if (r >= 0 && r < m) {
+        uint32_t h = hash_row(r) >> (32 - RP_LOG);
+        while (true) {
+            const int held = atomicCAS(s_row + h, -1, r);
+            if (held == -1 || held == r) break;
+            h = (h + 1) & ((1 << RP_LOG) - 1);
+        }
+        if (atomicAdd(s_seen + h, 1) == RP_HOT - 1) {
+            s_hot[RP_SLOTS] = 1;
+            int* q = s_hot + 4 * (hash_row(r) >> (32 - RP_HLOG));
+            for (int i = 0; i < 4 && atomicCAS(q + i, -1, r) != -1; ++i) {}   // a fifth is not counted there
         }
     }
     __syncthreads();
@@ -635,7 +634,7 @@ __global__ void __launch_bounds__(RP_BLOCK) k_row_place(const int32_t* __restric
                                                         unsigned long long* __restrict__ cnt,
                                                         uint32_t* __restrict__ place, const int32_t* __restrict__ hot) {
     const int tid = threadIdx.x;
-    if (!hot[RP_SLOTS]) {
+    if (!hot || !hot[RP_SLOTS]) {
         for (int64_t t = (int64_t)blockIdx.x * RP_BLOCK + tid; t < nnz; t += (int64_t)gridDim.x * RP_BLOCK) {
             const int32_t r = ir[t];
             if (r >= 0 && r < m) place[t] = (uint32_t)atomicAdd(cnt + r, 1ull);
@@ -720,7 +719,7 @@ void run_seg_sort(cudaStream_t st, const SegSort& S) {
     note_launch(2);
     if (S.nnz > S.split_len) {
         k_seg_scatter<<<(int)std::min<int64_t>(ceil_div64(S.nnz, SEG_CHUNK), sm_count() * 4), SEGL_BLOCK, 0, st>>>(S);
-        k_seg_windows<W><<<sm_count() * 8, SEG_WIN, 0, st>>>(S);
+        k_seg_windows<W><<<sm_count() * 4, SEG_WIN, 0, st>>>(S);
         note_launch(2);
     }
 }
@@ -733,10 +732,12 @@ struct SegScratch {
     size_t o_list, o_split = 0, o_chunk = 0, o_win = 0, o_off = 0, o_wkey = 0, o_widx = 0;
     template <class Take>
     SegScratch(int64_t n, int64_t nz, int64_t bound, bool own_entries, Take take) : nnz(nz) {
-        // a column holds no more entries than there are, nor than there are keys: where that is
-        // too few, none is split (a malformed one neither)
+        // a column holds no more entries than there are, nor than there are keys: up to SEG_WHOLE
+        // of them none is split (a malformed one neither).  The two launches cost 6 us also
+        // where no column needs them, of about 50 for a conversion of that size, and one CTA
+        // takes 0.2 ms for a column of SEG_WHOLE entries.
         split_len = SEG_SPLIT / std::max<int64_t>(1, ceil_div64(bound, SEGL_ROWS));
-        if (std::min(nnz, bound) <= split_len) split_len = INT64_MAX;
+        if (std::min(nnz, bound) <= SEG_WHOLE) split_len = INT64_MAX;
         o_list = take(4 * n);
         if (nnz <= split_len) return;
         const int64_t ns = nnz / split_len, nc = nnz / SEG_CHUNK + ns;
@@ -983,9 +984,15 @@ spgemm_status_t transpose_csc(spgemm_ctx* ctx, int64_t m, int64_t n, int64_t nnz
         int32_t* colid = (int32_t*)(t + o_col);
         uint32_t* place = (uint32_t*)(t + o_place);
         int64_t* tcp = (int64_t*)cpb->p;
-        k_row_begin<<<grid_for(m + 2, RP_SAMPLES), RP_SAMPLES, 0, st>>>(cnt, m + 2, ir, nz, m, (int32_t*)(t + o_hot));
-        k_row_place<<<grid_for(nz), RP_BLOCK, 0, st>>>(ir, nz, m, cnt, place, (int32_t*)(t + o_hot));
-        note_launch(2);
+        int32_t* hot = nz >= RP_MIN ? (int32_t*)(t + o_hot) : nullptr;
+        if (hot) {
+            k_row_begin<<<grid_for(m + 2, RP_SAMPLES), RP_SAMPLES, 0, st>>>(cnt, m + 2, ir, nz, m, hot);
+            note_launch();
+        } else {
+            SG_CUDA(ctx, cudaMemsetAsync(cnt, 0, 8 * m + 16, st));
+        }
+        k_row_place<<<grid_for(nz), RP_BLOCK, 0, st>>>(ir, nz, m, cnt, place, hot);
+        note_launch();
         launch_expand_cols(st, cp, n, nz, colid);
         launch_exclusive_scan(st, (const int64_t*)cnt, m, tcp, t + o_sc);
         void* tv = num ? (void*)(t + o_val) : nullptr;

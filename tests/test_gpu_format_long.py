@@ -1,5 +1,5 @@
 """Transpose and permutation with columns around the lengths from which a column is split over
-several CTAs (16,384 entries for up to 2^20 keys, less for more), alone and several at once,
+several CTAs (16,384 entries for up to 2^20 keys, less for more, none up to 65,536 keys), alone and several at once,
 down to a column that holds every key, with and without values."""
 import numpy as np
 import pytest
@@ -39,6 +39,8 @@ def _check(C, ref, vals=True):
     (3000017, (5461, 5462, 0, 16384, 300000, 513), OR_BOOL),
     (2 ** 23 - 1, (2048, 2049, 8192, 8193, 500000, 1), PT_F64),
     (40000, (16385,), MP_F32),
+    (65536, (65536, 16385), PT_F64),      # no column is split yet
+    (65537, (65537, 16385), PT_F64),
 ])
 def test_long_columns(ctx, m, lengths, sr):
     s = sp()
