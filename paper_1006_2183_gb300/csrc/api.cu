@@ -746,7 +746,9 @@ void engine_false_values(Engine* E) {
         cudaMemsetAsync(E->false_flag, ctx->bool_hint ? 1 : 0, 4, ctx->stream);
     } else {
         if (E->false_flag_made) cudaMemsetAsync(E->false_flag, 0, 4, ctx->stream);
-        launch_false_values(ctx->stream, E->it, E->false_flag);
+        int64_t most = 0;
+        for (const Prod& pr : E->hprods) most = std::max({most, pr.A.nnz, pr.B.nnz});
+        launch_false_values(ctx->stream, E->it, most, E->false_flag);
     }
     E->false_flag_made = true;
 }

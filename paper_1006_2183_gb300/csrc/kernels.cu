@@ -1365,10 +1365,12 @@ void launch_any_false(cudaStream_t st, const void* vals, int64_t n, int* flag) {
     note_launch();
 }
 
-void launch_false_values(cudaStream_t st, const Items& it, int* flag) {
+void launch_false_values(cudaStream_t st, const Items& it, int64_t most, int* flag) {
     if (it.nprod <= 0) return;
     const int gy = (int)std::min<int64_t>(it.nprod, 65535);
-    const int gx = std::max(1, std::min(sm_count() * 4, 4096 / gy));
+    // no more CTAs than four 16-byte loads per thread need: it is queued before every numeric
+    // pass, a replayed one's too
+    const int gx = (int)std::max<int64_t>(1, std::min<int64_t>({(int64_t)sm_count() * 4, 4096 / gy, ceil_div64(most, 256 * 64)}));
     k_false_values<<<dim3(gx, gy), 256, 0, st>>>(it, flag);
     note_launch();
 }

@@ -225,8 +225,9 @@ void launch_dense_items(cudaStream_t st, const Items& it, const int2* dense_list
 int slab_acc_entries(int sr, int RB);
 // whether A of the product can be read in aligned quads by the slab passes
 bool slab_quads(const Prod& pr);
-// *flag = 1 when an operand of some product stores a false value (boolean semiring)
-void launch_false_values(cudaStream_t st, const Items& it, int* flag);
+// *flag = 1 when an operand of some product stores a false value (boolean semiring); `most`: the
+// entries of the largest operand
+void launch_false_values(cudaStream_t st, const Items& it, int64_t most, int* flag);
 // *flag = 1 when one of the n bytes at vals is 0 (vals == nullptr: nothing)
 void launch_any_false(cudaStream_t st, const void* vals, int64_t n, int* flag);
 
