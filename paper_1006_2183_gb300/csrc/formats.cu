@@ -202,7 +202,7 @@ __global__ void k_take_values(const uint32_t* __restrict__ at, const void* __res
 // permutation, where only the order within a column is unknown: one read and one write of the
 // entries instead of the stable radix passes over all of them (three for 18 bits of row and
 // three for 18 of column): P A P^T, A^T and the DCSC form of R-MAT 18 with 4 million entries,
-// all kernels 916 -> 580 us, 60 launches -> 21.
+// all kernels 916 -> 550 us, 60 launches -> 25.
 struct SegSort {
     const int64_t* in_cp;     // column c: entries [in_cp[c], in_cp[c+1]) of key and val
     int64_t n, nnz;
