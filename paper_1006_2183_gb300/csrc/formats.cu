@@ -193,8 +193,11 @@ template <int W>
 __global__ void k_take_values(const uint32_t* __restrict__ at, const void* __restrict__ vin, int64_t nnz,
                               void* __restrict__ vout) {
     using T = typename Word<W>::T;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += (int64_t)gridDim.x * blockDim.x)
-        reinterpret_cast<T*>(vout)[i] = reinterpret_cast<const T*>(vin)[at[i]];
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t t = at[i];
+        if (t < nnz)   // a malformed operand's conversion leaves entries out
+            reinterpret_cast<T*>(vout)[i] = reinterpret_cast<const T*>(vin)[t];
+    }
 }
 
 // ---------------------------------------------------------------- sort within columns
